@@ -34,7 +34,9 @@ __device__ __forceinline__ uint32_t xor_columns(const uint32_t *col, uint32_t v)
 // DSI kernels as polynomials in the converted word fz = (T)Z with coefficients that
 // depend only on beta, i.e. on clz(Z) (the Theorem of Sec. 5.3; x = fz 2^-32):
 //   order 1: K = 1 - 3 t1                         (1 at Z = 0)
-//   order 2: K = (3/2 - 5/2 t1) - beta 2^-32 fz
+//   order 2: K = (3/2 - 5/2 t1) - beta 2^-32 fz; FP64 rows hold (3/2 - 5/2 t1 + beta, -beta),
+//            both exact, and take X = 1 + fz 2^-32 (mantissa bits, no conversion): the same
+//            real number -beta X + (A + beta) rounded once, one FP64 instruction
 //   order 3: K = (-1 + 43/18 (1 - t2)) - 5 (1 - t1) 2^-32 fz + beta 2^-64 fz^2
 //   order 4: K = (-1 + 701/294 (1 - t3)) - 43/9 (1 - t2) 2^-32 fz + 5 (1 - t1) 2^-64 fz^2
 //                - 2/3 beta 2^-96 fz^3 - beta/24 S'(Z)
@@ -107,6 +109,7 @@ __host__ __device__ constexpr DsiTable<T> make_dsi_table() {
     } else if (ALPHA == 2) {
       A = 1.5 - 2.5 * t1;
       B = -b * pow2neg(32);
+      if (sizeof(T) == 8) A += b, B = -b;
     } else if (ALPHA == 3) {
       A = -1.0 + (43.0 / 18.0) * (1.0 - t2);
       B = -5.0 * (1.0 - t1) * pow2neg(32);
@@ -206,9 +209,7 @@ __device__ void build_dsi_tab(T *tab) {
 }
 
 __device__ __forceinline__ float word_to(float, uint32_t Z) { return __uint2float_rn(Z); }
-__device__ __forceinline__ double word_to(double, uint32_t Z) {
-  return __hiloint2double(0x43300000, (int)Z) - 4503599627370496.0;  // exact
-}
+__device__ __forceinline__ double word_to(double, uint32_t Z) { return u32_to_double(Z, 0); }  // exact
 
 // K_alpha(Z) for a DSI kernel from the shared coefficient rows (vector row loads).
 template <typename T, int ALPHA>
@@ -217,18 +218,14 @@ __device__ __forceinline__ T dsi_tab_eval(const T *tab, uint32_t Z) {
   const T *row = tab + __clz(Z) * S;
   if constexpr (ALPHA == 1) {
     return row[0];
+  } else if constexpr (ALPHA == 2 && sizeof(T) == 8) {
+    const double2 v = *reinterpret_cast<const double2 *>(row);
+    return fma(v.y, __hiloint2double((int)(0x3FF00000u | (Z >> 12)), (int)(Z << 20)), v.x);
   } else {
     const T fz = word_to(T(), Z);
     if constexpr (ALPHA == 2) {
-      T a, b;
-      if constexpr (sizeof(T) == 4) {
-        const float2 v = *reinterpret_cast<const float2 *>(row);
-        a = v.x, b = v.y;
-      } else {
-        const double2 v = *reinterpret_cast<const double2 *>(row);
-        a = v.x, b = v.y;
-      }
-      return fmadd(b, fz, a);
+      const float2 v = *reinterpret_cast<const float2 *>(row);
+      return fmadd(v.y, fz, v.x);
     } else {
       T c0, c1, c2, c3;
       if constexpr (sizeof(T) == 4) {
@@ -507,23 +504,25 @@ __device__ __forceinline__ float rcp_approx(float a) {
   return r;
 }
 // a / b in FP64 without the FP64 divide (GB300 has about two FP64 lanes per SM and cycle):
-// the reciprocal of b by two Newton-Raphson steps r <- r + r (1 - b r), each squaring the
-// relative error, from the FP32 reciprocal estimate of b (b's leading 24 bits, rel. error
-// below 2^-22); the second step's error is below one unit in the last place, then one
-// product: within 2 ulp of the rounded quotient (checked against the divide by
-// qk_ratio_selftest).  Five FP64 operations; b outside [2^-100, 2^100] in magnitude, zero,
-// subnormal, inf or NaN, takes the divide.
-__device__ __forceinline__ double ratio(double a, double b) {
+// from the FP32 reciprocal estimate r of b (its leading 24 bits, relative error e below
+// 2^-22), q0 = a r, then q0 (1 + e + e^2) with e = 1 - b r rounded once: what is left is e^3,
+// below 2^-66, so the result is within 2 ulp of the rounded quotient (checked against the
+// divide by qk_ratio_selftest).  Four FP64 instructions.  False for b outside
+// 2^-100 .. 2^100 in magnitude (zero, subnormal, inf and NaN included).
+__device__ __forceinline__ bool ratio_fast(double a, double b, double &q) {
   const uint32_t hi = (uint32_t)__double2hiint(b), lo = (uint32_t)__double2loint(b);
   const uint32_t ex = (hi >> 20) & 0x7FFu;
-  if (ex - 923u > 200u) return a / b;
+  if (ex - 923u > 200u) return false;
   const uint32_t fb = (hi & 0x80000000u) | ((ex - 896u) << 23) | ((hi & 0xFFFFFu) << 3) | (lo >> 29);
-  double r = f2d_exact(rcp_approx(__uint_as_float(fb)));
-  double e = fma(-b, r, 1.0);
-  r = fma(r, e, r);
-  e = fma(-b, r, 1.0);
-  r = fma(r, e, r);
-  return a * r;
+  const double r = f2d_exact(rcp_approx(__uint_as_float(fb)));
+  const double e = fma(-b, r, 1.0);
+  const double q0 = a * r;
+  q = fma(q0, fma(e, e, e), q0);
+  return true;
+}
+__device__ __forceinline__ double ratio(double a, double b) {
+  double q;
+  return ratio_fast(a, b, q) ? q : a / b;
 }
 
 // Warp sums of four per-lane values, the pair (a0, a1) of one dimension and (b0, b1) of
@@ -531,8 +530,8 @@ __device__ __forceinline__ double ratio(double a, double b) {
 // sends the other's, at the xor-8 step it keeps one value of that pair, and the last three
 // steps finish one sum per group of 8 lanes.  Lane 0 ends with the total of a0, lane 8 of
 // a1, lane 16 of b0 and lane 24 of b1 (every lane of a group of 8 holds its group's total).
-// Each sum is formed in the same order of additions as a full xor butterfly, so the FP64
-// totals equal those of one butterfly per value; FP32 totals are float-float pairs (s, e).
+// Each sum is formed in the same order of additions as a full xor butterfly; the totals are
+// float-float pairs (s, e).
 // 5 shuffle steps for 4 values instead of 20.
 __device__ __forceinline__ void warp_sum4_ff(float a0, float a1, float b0, float b1, float &s, float &e) {
   const int lane = threadIdx.x & 31;
@@ -553,109 +552,68 @@ __device__ __forceinline__ void warp_sum4_ff(float a0, float a1, float b0, float
     ff_merge(s, e, s2, e2);
   }
 }
-__device__ __forceinline__ double warp_sum4(double a0, double a1, double b0, double b1) {
-  const int lane = threadIdx.x & 31;
-  const bool h16 = lane & 16, h8 = lane & 8;
-  const double s0 = (h16 ? b0 : a0) + __shfl_xor_sync(0xffffffffu, h16 ? a0 : b0, 16);
-  const double s1 = (h16 ? b1 : a1) + __shfl_xor_sync(0xffffffffu, h16 ? a1 : b1, 16);
-  double s = (h8 ? s1 : s0) + __shfl_xor_sync(0xffffffffu, h8 ? s0 : s1, 8);
-#pragma unroll
-  for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  return s;
-}
-
-// Gradient sweep: for each dimension j, warp-reduced sums over this warp's points of
-// u_i dk1_i/dc_j and dk1_i/dc_j (float-float pairs in FP32 sweeps, doubles in FP64
-// sweeps), written to red[warp][2d] and totalled by red_total, with
-// dk1_i/dc_j = k1_i K_ij / (1 + c_j K_ij).  wk[l] = u_l k1_l, both zero for points with
-// !ok[l]; uget(l) returns u_l and is called only for the rare exact zero of
+// FP32 gradient sweep: for each dimension j, warp-reduced sums over this warp's points of
+// u_i dk1_i/dc_j and dk1_i/dc_j (float-float pairs), written to red[warp][2d] and totalled by
+// red_total, with dk1_i/dc_j = k1_i K_ij / (1 + c_j K_ij).  wk[l] = u_l k1_l, both zero for
+// points with !ok[l]; uget(l) returns u_l and is called only for the rare exact zero of
 // 1 + c_j K_ij, handled after the loop by the explicit product over the other dimensions.
-// ALL_OK (unpacked sweeps): every point is valid, so no per-point validity select.
-// Dimensions are reduced in pairs (warp_sum4*): an even dimension's two lane sums wait in
+// Dimensions are reduced in pairs (warp_sum4_ff): an even dimension's two lane sums wait in
 // registers for the next dimension's; an odd d leaves the last dimension to a butterfly.
-template <typename T, int FAM, int ALPHA, int L, bool ALL_OK = false, typename UF>
-__device__ __forceinline__ void gradient_sweep(const ColJob &job, const DiffTables &tb, const T *wT,
-                                               const uint32_t (&bi)[L], const T (&k1)[L], const T (&wk)[L],
+// (FP64 sweeps: qk_grad.cuh.)
+template <int FAM, int ALPHA, int L, typename UF>
+__device__ __forceinline__ void gradient_sweep(const ColJob &job, const DiffTables &tb, const float *wT,
+                                               const uint32_t (&bi)[L], const float (&k1)[L], const float (&wk)[L],
                                                const bool (&ok)[L], UF uget, double *red) {
+  static_assert(L % 4 == 0, "quads of points");
   const uint32_t d = job.d;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  constexpr bool PACKED = sizeof(T) == 4 && L % 4 == 0;
-  // packed form: points (2h, 2h+1) share one f32x2 fma / mul, with the two halves summed
-  // separately; a zero 1 + c_j K gives an infinite reciprocal, so the sums come out
-  // non-finite and the exact fallback below runs instead of a per-point zero test.
-  // Points with !ok[l] carry wk[l] = k1[l] = 0 and add nothing (or a NaN, which again
-  // sends the thread to the fallback, where they are skipped).
-  unsigned long long WK[PACKED ? L / 2 : 1], K1[PACKED ? L / 2 : 1];
-  if constexpr (PACKED) {
+  // points (2h, 2h+1) share one f32x2 fma / mul, with the two halves summed separately; a zero
+  // 1 + c_j K gives an infinite reciprocal, so the sums come out non-finite and the exact
+  // fallback below runs instead of a per-point zero test.  Points with !ok[l] carry
+  // wk[l] = k1[l] = 0 and add nothing (or a NaN, which again sends the thread to the
+  // fallback, where they are skipped).
+  unsigned long long WK[L / 2], K1[L / 2];
 #pragma unroll
-    for (int h = 0; h < L / 2; ++h) {
-      WK[h] = pack_f2(wk[2 * h], wk[2 * h + 1]);
-      K1[h] = pack_f2(k1[2 * h], k1[2 * h + 1]);
-    }
+  for (int h = 0; h < L / 2; ++h) {
+    WK[h] = pack_f2(wk[2 * h], wk[2 * h + 1]);
+    K1[h] = pack_f2(k1[2 * h], k1[2 * h + 1]);
   }
-  T cu = T(0), c1 = T(0);  // lane sums of the even dimension of the current pair
+  float cu = 0.f, c1 = 0.f;  // lane sums of the even dimension of the current pair
   for (uint32_t j = 0; j < d; ++j) {
-    const T wj = wT[j];
-    T su = T(0), s1 = T(0);
+    const float wj = wT[j];
     uint32_t base = 0;
     if constexpr (FAM == 0) base = tb.zlane[j * 32 + lane] ^ tb.zwarp[warp * d + j];
-    bool anyzero = false;
-    if constexpr (PACKED) {
-      const unsigned long long W = pack_f2(wj, wj), ONE = pack_f2(1.f, 1.f);
-      unsigned long long SU = pack_f2(0.f, 0.f), S1 = SU;
+    const unsigned long long W = pack_f2(wj, wj), ONE = pack_f2(1.f, 1.f);
+    unsigned long long SU = pack_f2(0.f, 0.f), S1 = SU;
 #pragma unroll
-      for (int l = 0; l < L; l += 4) {
-        uint32_t z[4];
-        diff_words4<FAM, L>(tb, base, bi, l, j, z);
+    for (int l = 0; l < L; l += 4) {
+      uint32_t z[4];
+      diff_words4<FAM, L>(tb, base, bi, l, j, z);
 #pragma unroll
-        for (int i = 0; i < 4; i += 2) {
-          const int h = (l + i) >> 1;
-          const T ka = kfac<T, FAM, ALPHA>(tb, z[i]), kb = kfac<T, FAM, ALPHA>(tb, z[i + 1]);
-          const unsigned long long KK = pack_f2(ka, kb);
-          float fa, fb;
-          unpack_f2(fma_f2(W, KK, ONE), fa, fb);
-          const unsigned long long Q = mul_f2(KK, pack_f2(rcp_approx(fa), rcp_approx(fb)));
-          SU = fma_f2(WK[h], Q, SU);
-          S1 = fma_f2(K1[h], Q, S1);
-        }
-      }
-      float a, b;
-      unpack_f2(SU, a, b);
-      su = a + b;
-      unpack_f2(S1, a, b);
-      s1 = a + b;
-      anyzero = !(isfinite(su) && isfinite(s1));
-    } else {
-      auto step = [&](int l, uint32_t z) {
-        const T K = kfac<T, FAM, ALPHA>(tb, z);
-        const T f = fmadd(wj, K, T(1));
-        anyzero |= f == T(0);
-        T q = ratio(K, f);
-        if constexpr (!ALL_OK) q = ok[l] ? q : T(0);
-        su = fmadd(wk[l], q, su);
-        s1 = fmadd(k1[l], q, s1);
-      };
-      if constexpr (L % 4 == 0) {
-#pragma unroll
-        for (int l = 0; l < L; l += 4) {
-          uint32_t z[4];
-          diff_words4<FAM, L>(tb, base, bi, l, j, z);
-#pragma unroll
-          for (int i = 0; i < 4; ++i) step(l + i, z[i]);
-        }
-      } else {
-#pragma unroll
-        for (int l = 0; l < L; ++l) step(l, diff_word<FAM, L>(tb, d, base, bi[l], l, j));
+      for (int i = 0; i < 4; i += 2) {
+        const int h = (l + i) >> 1;
+        const float ka = kfac<float, FAM, ALPHA>(tb, z[i]), kb = kfac<float, FAM, ALPHA>(tb, z[i + 1]);
+        const unsigned long long KK = pack_f2(ka, kb);
+        float fa, fb;
+        unpack_f2(fma_f2(W, KK, ONE), fa, fb);
+        const unsigned long long Q = mul_f2(KK, pack_f2(rcp_approx(fa), rcp_approx(fb)));
+        SU = fma_f2(WK[h], Q, SU);
+        S1 = fma_f2(K1[h], Q, S1);
       }
     }
-    if (anyzero) {  // exact zeros of 1 + c_j K: use prod_{j' != j} (1 + c_j' K_j') directly
-      su = T(0), s1 = T(0);
+    float a, b;
+    unpack_f2(SU, a, b);
+    float su = a + b;
+    unpack_f2(S1, a, b);
+    float s1 = a + b;
+    if (!(isfinite(su) && isfinite(s1))) {  // exact zeros of 1 + c_j K: prod_{j' != j} (1 + c_j' K_j') directly
+      su = 0.f, s1 = 0.f;
 #pragma unroll
       for (int l = 0; l < L; ++l) {
         if (!ok[l]) continue;
-        const T K = kfac<T, FAM, ALPHA>(tb, diff_word<FAM, L>(tb, d, base, bi[l], l, j));
-        const T f = fmadd(wj, K, T(1));
-        const T dk = f == T(0) ? dk_explicit<T, FAM, ALPHA, L>(job, tb, wT, bi[l], l, j) : k1[l] * ratio(K, f);
+        const float K = kfac<float, FAM, ALPHA>(tb, diff_word<FAM, L>(tb, d, base, bi[l], l, j));
+        const float f = fmadd(wj, K, 1.f);
+        const float dk = f == 0.f ? dk_explicit<float, FAM, ALPHA, L>(job, tb, wT, bi[l], l, j) : k1[l] * ratio(K, f);
         su = fmadd(uget(l), dk, su);
         s1 += dk;
       }
@@ -664,61 +622,34 @@ __device__ __forceinline__ void gradient_sweep(const ColJob &job, const DiffTabl
       cu = su, c1 = s1;
       continue;
     }
-    if constexpr (sizeof(T) == 4) {
-      // float-float warp sums, kept as (hi, lo) pairs: no FP64 arithmetic per dimension
-      float2 *r2 = reinterpret_cast<float2 *>(red) + (size_t)warp * 2 * d;
-      if (j & 1) {
-        float s, e;
-        warp_sum4_ff(cu, c1, su, s1, s, e);
-        if (!(lane & 7)) r2[((lane & 8) ? d : 0) + j - ((lane & 16) ? 0 : 1)] = make_float2(s, e);
-      } else {
-        float ue = 0.f, oe = 0.f;
-        warp_sum_ff(su, ue);
-        warp_sum_ff(s1, oe);
-        if (lane == 0) {
-          r2[j] = make_float2(su, ue);
-          r2[d + j] = make_float2(s1, oe);
-        }
-      }
+    // float-float warp sums, kept as (hi, lo) pairs: no FP64 arithmetic per dimension
+    float2 *r2 = reinterpret_cast<float2 *>(red) + (size_t)warp * 2 * d;
+    if (j & 1) {
+      float s, e;
+      warp_sum4_ff(cu, c1, su, s1, s, e);
+      if (!(lane & 7)) r2[((lane & 8) ? d : 0) + j - ((lane & 16) ? 0 : 1)] = make_float2(s, e);
     } else {
-      double *rw = red + (size_t)warp * 2 * d;
-      if (j & 1) {
-        const double s = warp_sum4(cu, c1, su, s1);
-        if (!(lane & 7)) rw[((lane & 8) ? d : 0) + j - ((lane & 16) ? 0 : 1)] = s;
-      } else {
-        double du = su, d1 = s1;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          du += __shfl_xor_sync(0xffffffffu, du, o);
-          d1 += __shfl_xor_sync(0xffffffffu, d1, o);
-        }
-        if (lane == 0) {
-          rw[j] = du;
-          rw[d + j] = d1;
-        }
+      float ue = 0.f, oe = 0.f;
+      warp_sum_ff(su, ue);
+      warp_sum_ff(s1, oe);
+      if (lane == 0) {
+        r2[j] = make_float2(su, ue);
+        r2[d + j] = make_float2(s1, oe);
       }
     }
   }
 }
 
-// Entry q of the per-warp gradient partials red[warp][nq] summed over the warps: FP32
-// sweeps leave float-float pairs (summed in float-float, converted once), FP64 sweeps
-// doubles.
-template <typename T>
+// Entry q of the per-warp gradient partials red[warp][nq] (float-float pairs) summed over the
+// warps in float-float, converted once.
 __device__ __forceinline__ double red_total(const double *red, int warps, uint32_t nq, uint32_t q) {
-  if constexpr (sizeof(T) == 4) {
-    const float2 *r2 = reinterpret_cast<const float2 *>(red);
-    float s = 0.f, e = 0.f;
-    for (int w = 0; w < warps; ++w) {
-      const float2 p = r2[(size_t)w * nq + q];
-      ff_merge(s, e, p.x, p.y);
-    }
-    return (double)s + (double)e;
-  } else {
-    double s = 0.0;
-    for (int w = 0; w < warps; ++w) s += red[(size_t)w * nq + q];
-    return s;
+  const float2 *r2 = reinterpret_cast<const float2 *>(red);
+  float s = 0.f, e = 0.f;
+  for (int w = 0; w < warps; ++w) {
+    const float2 p = r2[(size_t)w * nq + q];
+    ff_merge(s, e, p.x, p.y);
   }
+  return (double)s + (double)e;
 }
 
 }  // namespace qk

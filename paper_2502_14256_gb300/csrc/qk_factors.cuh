@@ -29,6 +29,24 @@ __device__ __forceinline__ double small_int_to(double, uint32_t v) {
   return __hiloint2double(0x43300000, (int)v) - 4503599627370496.0;  // v < 2^32
 }
 
+// v 2^-t as a double (RN) by integer operations: GB300 issues some 60 integer instructions in
+// the time of one FP64 add or conversion (t: binary places, |t| small).
+__device__ __forceinline__ double u64_to_double(uint64_t v, int t) {
+  const int c = __clzll((long long)v);
+  const uint64_t x = v << (c & 63);                      // leading one at bit 63
+  const uint32_t rem = (uint32_t)x & 0x7FFu;
+  uint64_t mant = x >> 11;                               // 53 bits, the leading one at bit 52
+  mant += (rem > 0x400u) | ((rem == 0x400u) & ((uint32_t)mant & 1u));
+  const uint64_t bits = ((uint64_t)(uint32_t)(1085 - c - t) << 52) + mant;
+  return __longlong_as_double(v ? (long long)bits : 0ll);
+}
+__device__ __forceinline__ double u32_to_double(uint32_t v, int t) {  // exact
+  const int c = __clz(v);
+  const uint32_t x = v << (c & 31);
+  const uint32_t hi = ((uint32_t)(1053 - c - t) << 20) + (x >> 11);
+  return __hiloint2double(v ? (int)hi : 0, (int)(x << 21));
+}
+
 // S' = sum_{a >= 0, bit (31-a) of Z set} 8^-a, to the precision of T.
 __device__ __forceinline__ float octal_tail(float, uint32_t Z) {
   return __uint2float_rn(spread3_10(Z >> 22)) * 0x1p-27f;  // a = 0..9
@@ -70,12 +88,15 @@ __device__ __forceinline__ T dsi_factor(uint32_t Z) {
 
 template <typename T, int ALPHA>
 __device__ __forceinline__ T si_factor(uint32_t W) {
-  const T x = word_to_unit(T(), W);
-  // x (1 - x): in FP64, 1 - x is exact (x has 32 significant bits), so x * (1 - x) and the
-  // fused x - x * x both round the same real number once; the fused form is one operation
+  // x (1 - x) = W (2^32 - W) 2^-64: in FP64 the exact 64-bit product rounded once, without
+  // FP64 instructions (the bits of fma(-x, x, x))
   T q;
-  if constexpr (sizeof(T) == 8) q = fma(-x, x, x);
-  else q = x * (T(1) - x);
+  if constexpr (sizeof(T) == 8) {
+    q = u64_to_double((uint64_t)W * (uint32_t)(0u - W), 64);
+  } else {
+    const T x = word_to_unit(T(), W);
+    q = x * (T(1) - x);
+  }
   if constexpr (ALPHA == 1) {
     return T(3.2898681336964528729) - T(19.739208802178717238) * q;  // pi^2/3, 2 pi^2
   } else {

@@ -266,13 +266,17 @@ bool fused_supported(const qk_task &t, int dtype) {
 
 static size_t fused_elem(int dtype) { return dtype == QK_F64 ? 8 : 4; }
 
+static uint64_t fused_gblocks(uint32_t m, int dtype) {
+  return dtype == QK_F64 ? grad64_blocks(m) : (1ull << m) >> FCfg<float>::LOGT;
+}
+
 size_t fused_ws_bytes(const qk_task &t, int dtype, int refine) {
   const int LOGT = dtype == QK_F64 ? FCfg<double>::LOGT : FCfg<float>::LOGT;
   const uint64_t R = t.ps.R, n = 1ull << t.m, tiles = n >> LOGT, nv = R * t.nrhs;
   const size_t e = fused_elem(dtype);
   size_t s = 2 * align256(e * R * n) + 2 * align256(e * nv * n);
   s += 2 * align256(8 * R * tiles) + align256(8 * nv * tiles) + align256(16 * nv * tiles);
-  s += align256(8 * nv * tiles * 2 * (uint64_t)t.ps.d);
+  s += align256(8 * nv * fused_gblocks(t.m, dtype) * 2 * (uint64_t)t.ps.d);
   if ((refine > 0 && dtype == QK_F32) || dtype == QK_F32W) s += align256(e * nv * n);  // lo parts of y'
   if (dtype == QK_F32W) s += align256(e * R * n);                                      // lo parts of p'
   return s;
@@ -289,6 +293,7 @@ static FTask make_ftask(const qk_task &t, const ColJob &job, int dtype, int refi
   ft.job = job;
   ft.nrhs = t.nrhs;
   ft.tiles = (uint32_t)tiles;
+  ft.gblocks = (uint32_t)fused_gblocks(t.m, dtype);
   ft.cB = 2 * LOGT - (int)t.m;
   ft.eta = t.eta;
   ft.y = t.y;
@@ -306,7 +311,7 @@ static FTask make_ftask(const qk_task &t, const ColJob &job, int dtype, int refi
   ft.sy = (double *)p, p += align256(8 * nv * tiles);
   ft.qg = (double *)p, p += align256(16 * nv * tiles);
   ft.gr = (double *)p;
-  p += align256(8 * nv * tiles * 2 * (uint64_t)t.ps.d);
+  p += align256(8 * nv * fused_gblocks(t.m, dtype) * 2 * (uint64_t)t.ps.d);
   ft.yL = nullptr;
   ft.pTL = nullptr;
   if ((dtype == QK_F32 && refine > 0) || dtype == QK_F32W) {
@@ -406,7 +411,7 @@ int persist_setup(const std::vector<qk_task> &tasks, int dtype, int refine, uint
       pu.ft = make_ftask(one, job, dtype, refine, base + (size_t)(units.size() % nslot) * slot, nullptr);
       pu.tiles = (uint32_t)(n >> LOGT);
       pu.nrhs = t.nrhs;
-      pu.ncv = (t.c || t.grad) ? pu.tiles * t.nrhs : 0;
+      pu.ncv = (t.c || t.grad) ? (dtype == QK_F64 ? pu.tiles : pu.tiles * t.nrhs) : 0;
       units.push_back(pu);
     }
   }

@@ -19,7 +19,8 @@
 //      quadratic form and of g; high bits of the inverse WHT of c^ and g.
 //   C  (contiguous tiles)  low bits of the inverse -> c = K^-1 y (stored) and
 //      u = H g; gradient sweep sum_i u_i dk1_i/dc_j, sum_i dk1_i/dc_j, with the
-//      factors recomputed and k_1 from the stored p.
+//      factors recomputed and k_1 from the stored p.  FP64: C stores u (in place of g) and
+//      the sweep is qk_grad.cuh's, once for all right-hand sides of a randomization.
 // A final kernel reduces the partial sums into the MLL outputs and gradient.
 //
 // Inside a tile every thread holds the L elements e = threadIdx.x + 256 l: the
@@ -35,6 +36,7 @@
 #include "qk_column.cuh"
 #include "qk_common.cuh"
 #include "qk_factors.cuh"
+#include "qk_grad.cuh"
 #include "qk_internal.h"
 
 namespace qk {
@@ -50,6 +52,7 @@ template <typename T> constexpr int two_pass_max_m() { return 2 * FCfg<T>::LOGT 
 struct FTask {
   ColJob job;
   uint32_t nrhs, tiles;  // tiles = n >> LOGT
+  uint32_t gblocks;      // gradient partial sums per vector: tiles (FP32) or grad64_blocks(m)
   int cB;                // phase-B contiguous column bits (= 2 LOGT - m)
   double eta;
   const void *y;
@@ -804,23 +807,16 @@ __global__ void __launch_bounds__(kFNT, 2) k_fused_B(FTask ft) {
 }
 
 // ------------------------------------------------------------------ phase C
-template <typename T, int FAM, int ALPHA>
-__device__ __forceinline__ void fused_C_item(const FTask &ft, uint32_t v, uint32_t tile, unsigned char *smem) {
-  constexpr int LOGT = FCfg<T>::LOGT, L = FCfg<T>::L;
-  const ColJob &job = ft.job;
-  const uint32_t d = job.d;
-  double *wd;
-  DiffTables tb;
-  carve_tables<L>(smem, d, &wd, tb);
-  T *wT = reinterpret_cast<T *>(wd);
-  T *sm = reinterpret_cast<T *>(smem + align256(col_smem_bytes<L>(d)));
-  double *red = reinterpret_cast<double *>(smem + align256(col_smem_bytes<L>(d)) + xtile_bytes<T>());
-  const uint32_t r = v / ft.nrhs;
-  const uint64_t n = 1ull << job.m, base = (uint64_t)tile << LOGT;
+// Inverse low bits of one vector's tile: c stored, u returned in layout L0 (grad wanted).
+template <typename T>
+__device__ __forceinline__ void fused_C_transforms(const FTask &ft, uint32_t v, uint64_t base, T *sm,
+                                                   T (&uu)[FCfg<T>::L]) {
+  constexpr int L = FCfg<T>::L;
+  const uint64_t n = 1ull << ft.job.m;
   const int t = threadIdx.x;
   const T *YT = reinterpret_cast<const T *>(ft.yT) + (uint64_t)v * n + base;
   const T *GT = reinterpret_cast<const T *>(ft.gT) + (uint64_t)v * n + base;
-  T cc[L], uu[L];
+  T cc[L];
 #pragma unroll
   for (int l = 0; l < L; ++l) cc[l] = __ldcg(&YT[e_of<T>(2, t, l)]);
   xwht_full<T>(cc, sm, 1);  // L2 -> L0: the thread's own points
@@ -833,35 +829,97 @@ __device__ __forceinline__ void fused_C_item(const FTask &ft, uint32_t v, uint32
 #pragma unroll
   for (int l = 0; l < L; ++l) uu[l] = __ldcg(&GT[e_of<T>(2, t, l)]);
   xwht_full<T>(uu, sm, 1);
+}
+
+// FP32: one vector's tile, transforms and gradient sweep.
+template <int FAM, int ALPHA>
+__device__ __forceinline__ void fused_C_item(const FTask &ft, uint32_t v, uint32_t tile, unsigned char *smem) {
+  constexpr int LOGT = FCfg<float>::LOGT, L = FCfg<float>::L;
+  const ColJob &job = ft.job;
+  const uint32_t d = job.d;
+  double *wd;
+  DiffTables tb;
+  carve_tables<L>(smem, d, &wd, tb);
+  float *wT = reinterpret_cast<float *>(wd);
+  float *sm = reinterpret_cast<float *>(smem + align256(col_smem_bytes<L>(d)));
+  double *red = reinterpret_cast<double *>(smem + align256(col_smem_bytes<L>(d)) + xtile_bytes<float>());
+  const uint32_t r = v / ft.nrhs;
+  const uint64_t n = 1ull << job.m, base = (uint64_t)tile << LOGT;
+  const int t = threadIdx.x;
+  float uu[L];
+  fused_C_transforms<float>(ft, v, base, sm, uu);
+  if (!ft.grad) return;
 #pragma unroll
   for (int l = 0; l < L; ++l) sm[t + (l << kLOGNT)] = uu[l];  // own entries, for the rare fallback
-  for (uint32_t q = t; q < d; q += kFNT) wT[q] = (T)job.w[q];
-  build_all<T, FAM, ALPHA, L>(job, job.Ct + (size_t)r * d * 32, job.g, base, tb);
-  const T *P = reinterpret_cast<const T *>(ft.p) + (uint64_t)r * n + base;
-  const T zeta = (T)job.zeta;
-  T k1[L];
+  for (uint32_t q = t; q < d; q += kFNT) wT[q] = (float)job.w[q];
+  build_all<float, FAM, ALPHA, L>(job, job.Ct + (size_t)r * d * 32, job.g, base, tb);
+  const float *P = reinterpret_cast<const float *>(ft.p) + (uint64_t)r * n + base;
+  const float zeta = (float)job.zeta;
+  float k1[L];
   uint32_t bi[L];
   bool ok[L];
 #pragma unroll
   for (int l = 0; l < L; ++l) {
-    k1[l] = zeta * (T(1) + __ldcg(&P[t + (l << kLOGNT)]));
+    k1[l] = zeta * (1.f + __ldcg(&P[t + (l << kLOGNT)]));
     bi[l] = __brev((uint32_t)(base + t + (l << kLOGNT)));
     ok[l] = true;
     uu[l] *= k1[l];  // from here on uu holds u k1
   }
   __syncthreads();
-  // u itself stays in the transform tile (sm) after tile_wht; each thread reads its own
-  gradient_sweep<T, FAM, ALPHA, L, true>(job, tb, wT, bi, k1, uu, ok,
-                                   [&](int l) { return sm[t + (l << kLOGNT)]; }, red);
+  // u itself stays in the transform tile (sm) after the transform; each thread reads its own
+  gradient_sweep<FAM, ALPHA, L>(job, tb, wT, bi, k1, uu, ok, [&](int l) { return sm[t + (l << kLOGNT)]; }, red);
   __syncthreads();
   double *dst = ft.gr + ((uint64_t)v * ft.tiles + tile) * 2 * d;
-  for (uint32_t q = t; q < 2 * d; q += kFNT) dst[q] = red_total<T>(red, kFNT / 32, 2 * d, q);
+  for (uint32_t q = t; q < 2 * d; q += kFNT) dst[q] = red_total(red, kFNT / 32, 2 * d, q);
 }
 
-template <typename T, int FAM, int ALPHA>
+// FP64: one vector's tile of transforms; u takes the place of g's tile.
+__device__ __forceinline__ void fused_C64_transforms(const FTask &ft, uint32_t v, uint32_t tile, unsigned char *smem) {
+  constexpr int LOGT = FCfg<double>::LOGT, L = FCfg<double>::L;
+  const uint64_t base = (uint64_t)tile << LOGT;
+  double uu[L];
+  fused_C_transforms<double>(ft, v, base, reinterpret_cast<double *>(smem), uu);
+  if (!ft.grad) return;
+  double *GT = reinterpret_cast<double *>(ft.gT) + ((uint64_t)v << ft.job.m) + base;  // this CTA's tile only
+#pragma unroll
+  for (int l = 0; l < L; ++l) GT[threadIdx.x + (l << kLOGNT)] = uu[l];
+}
+
+// FP64 in the persistent schedule: one tile of a randomization, every right-hand side, then
+// the gradient blocks of the tile (the partial sums of k_grad64, bit for bit: the order of the
+// additions does not depend on the number of vectors per pass).
+template <int ALPHA>
+__device__ __forceinline__ void fused_C64_item(const FTask &ft, uint32_t tile, unsigned char *smem) {
+  for (uint32_t v = 0; v < ft.nrhs; ++v) fused_C64_transforms(ft, v, tile, smem);
+  if (!ft.grad) return;
+  __syncthreads();  // this CTA's stores of u, read back below through L2
+  const ColJob &job = ft.job;
+  const uint64_t n = 1ull << job.m;
+  const uint32_t cnt = grad64_points(job.m), per = (1u << FCfg<double>::LOGT) / cnt, d2 = 2 * job.d;
+  const double *U = reinterpret_cast<const double *>(ft.gT), *P = reinterpret_cast<const double *>(ft.p);
+  for (uint32_t b = tile * per; b < (tile + 1) * per; ++b) {
+    const uint32_t base = b * cnt;
+    auto run = [&](auto nv, uint32_t q0, uint32_t nva) {
+      auto u = [&](uint32_t v, uint32_t i) { return __ldcg(&U[(uint64_t)(q0 + v) * n + base + i]); };
+      grad64_item<0, ALPHA, decltype(nv)::value>(job, job.Ct, base, cnt, nva, u, P + base,
+                                                 ft.gr + ((uint64_t)q0 * ft.gblocks + b) * d2, (size_t)ft.gblocks * d2, smem);
+    };
+    if (ft.nrhs == 1) run(std::integral_constant<int, 1>(), 0, 1);
+    else
+      for (uint32_t q0 = 0; q0 < ft.nrhs; q0 += 8)
+        run(std::integral_constant<int, 8>(), q0, ft.nrhs - q0 < 8 ? ft.nrhs - q0 : 8);
+  }
+}
+
+template <int FAM, int ALPHA>
 __global__ void __launch_bounds__(kFNT, 2) k_fused_C(FTask ft) {
   extern __shared__ __align__(16) unsigned char smem[];
-  fused_C_item<T, FAM, ALPHA>(ft, blockIdx.y, blockIdx.x, smem);
+  fused_C_item<FAM, ALPHA>(ft, blockIdx.y, blockIdx.x, smem);
+}
+
+static __global__ void __launch_bounds__(kFNT, 2) k_fused_C64(FTask ft) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  fused_C64_transforms(ft, blockIdx.y, blockIdx.x, smem);
 }
 
 // ------------------------------------------------------------------ final
@@ -903,7 +961,7 @@ __device__ __forceinline__ void fused_final_item(const FTask &ft, uint32_t v) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (uint32_t j = warp; j < 2 * d; j += blockDim.x >> 5) {
     double s = 0.0;
-    for (uint32_t b = lane; b < tiles; b += 32) s += __ldcg(&ft.gr[((uint64_t)v * tiles + b) * 2 * d + j]);
+    for (uint32_t b = lane; b < ft.gblocks; b += 32) s += __ldcg(&ft.gr[((uint64_t)v * ft.gblocks + b) * 2 * d + j]);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (lane == 0) {
@@ -936,7 +994,7 @@ static __global__ void __launch_bounds__(256) k_fused_final(FTask ft) { fused_fi
 // the launch finishes.
 struct PUnit {
   FTask ft;                   // one randomization: r = 0, scratch in slot u mod nslot
-  uint32_t tiles, nrhs, ncv;  // ncv: C items (tiles x nrhs, 0 when neither c nor grad is wanted)
+  uint32_t tiles, nrhs, ncv;  // ncv: C items (tiles x nrhs; FP64: tiles; 0 when neither c nor grad is wanted)
 };
 struct PSched {
   const PUnit *units;
@@ -1032,7 +1090,8 @@ __global__ void __launch_bounds__(kFNT, 2) k_fused_persist(PSched ps) {
     } else if (kind == PK_B) {
       fused_B_item<T, COMP, WIDE>(pu.ft, 0, idx, smem, ps.status);
     } else if (kind == PK_C) {
-      fused_C_item<T, FAM, ALPHA>(pu.ft, idx / pu.tiles, idx % pu.tiles, smem);
+      if constexpr (sizeof(T) == 8) fused_C64_item<ALPHA>(pu.ft, idx, smem);
+      else fused_C_item<FAM, ALPHA>(pu.ft, idx / pu.tiles, idx % pu.tiles, smem);
     } else {
       fused_final_item(pu.ft, idx);
     }
@@ -1050,10 +1109,8 @@ int launch_fused_t(const FTask &ft, cudaStream_t st, LaunchTimer *tm) {
   // phase A keeps a second tile for the lo parts when compensating
   const size_t smA = colb + xtile_bytes<T>() + 32 * sizeof(double);
   const size_t smB = 3 * xtile_bytes<T>() + 32 * sizeof(double);
-  const size_t smC = colb + xtile_bytes<T>() + (size_t)(kFNT / 32) * 2 * d * sizeof(double);
   smem_optin<k_fused_A<T, FAM, ALPHA, COMP, WIDE>>(smA);
   smem_optin<k_fused_B<T, COMP, WIDE>>(smB);
-  smem_optin<k_fused_C<T, FAM, ALPHA>>(smC);
   if (tm) tm->begin("k_fused_A", st);
   k_fused_A<T, FAM, ALPHA, COMP, WIDE><<<dim3(ft.tiles, R), kFNT, smA, st>>>(ft);
   if (tm) tm->end(st);
@@ -1065,9 +1122,23 @@ int launch_fused_t(const FTask &ft, cudaStream_t st, LaunchTimer *tm) {
   if ((rc = check_launch("fused B"))) return rc;
   if (ft.c || ft.grad) {
     if (tm) tm->begin("k_fused_C", st);
-    k_fused_C<T, FAM, ALPHA><<<dim3(ft.tiles, R * ft.nrhs), kFNT, smC, st>>>(ft);
+    if constexpr (sizeof(T) == 8) {
+      k_fused_C64<<<dim3(ft.tiles, R * ft.nrhs), kFNT, xtile_bytes<double>(), st>>>(ft);
+    } else {
+      const size_t smC = colb + xtile_bytes<T>() + (size_t)(kFNT / 32) * 2 * d * sizeof(double);
+      smem_optin<k_fused_C<FAM, ALPHA>>(smC);
+      k_fused_C<FAM, ALPHA><<<dim3(ft.tiles, R * ft.nrhs), kFNT, smC, st>>>(ft);
+    }
     if (tm) tm->end(st);
     if ((rc = check_launch("fused C"))) return rc;
+  }
+  if constexpr (sizeof(T) == 8) {
+    if (ft.grad) {
+      if (tm) tm->begin("k_grad64", st);
+      rc = launch_grad_partials_f64(ft.job, ft.nrhs, (const double *)ft.gT, ft.gr, st, false, (const double *)ft.p);
+      if (tm) tm->end(st);
+      if (rc) return rc;
+    }
   }
   if (tm) tm->begin("k_fused_final", st);
   k_fused_final<<<R * ft.nrhs, 256, 0, st>>>(ft);
@@ -1092,7 +1163,8 @@ int persist_launch_t(const PSched &ps, uint32_t dmax, cudaStream_t st) {
   const size_t colb = align256(col_smem_bytes<L>(dmax));
   const size_t smA = colb + xtile_bytes<T>() + 32 * sizeof(double);
   const size_t smB = 3 * xtile_bytes<T>() + 32 * sizeof(double);
-  const size_t smC = colb + xtile_bytes<T>() + (size_t)(kFNT / 32) * 2 * dmax * sizeof(double);
+  const size_t smC = sizeof(T) == 8 ? grad64_smem(dmax, QK_MAX_M, 8)  // above its transforms' xtile_bytes (in smA)
+                                    : colb + xtile_bytes<T>() + (size_t)(kFNT / 32) * 2 * dmax * sizeof(double);
   size_t sm = smA > smB ? smA : smB;
   if (smC > sm) sm = smC;
   smem_optin<k_fused_persist<T, FAM, ALPHA, COMP, WIDE>>(sm);

@@ -12,6 +12,7 @@
 #include "qk_column.cuh"
 #include "qk_common.cuh"
 #include "qk_factors.cuh"
+#include "qk_grad.cuh"
 #include "qk_internal.h"
 
 namespace qk {
@@ -218,12 +219,12 @@ static int dispatch_col_ho(const qk_hopointset *ps, const qk_kernel *k, uint32_t
 // sum_i u_i dk1_i/dc_j and sum_i dk1_i/dc_j with dk1_i/dc_j = k1_i K_ij / (1 + c_j K_ij)
 // (the explicit product over the other dimensions where 1 + c_j K_ij = 0), the factors
 // recomputed from the 64-digit words; written as partial[v][blockIdx.x][2d] (the layout
-// of the 32-digit gradient partials, 2048 points per block).
-template <typename T, int ALPHA>
+// of the 32-digit gradient partials, 2048 points per block).  FP32; FP64 sweeps: qk_grad.cuh.
+template <int ALPHA>
 __global__ void __launch_bounds__(kHoNT) k_grad_partials_ho(uint32_t d, int order, uint32_t m, uint32_t nrhs,
                                                             const uint64_t *__restrict__ Chat,
                                                             const double *__restrict__ w, double zeta,
-                                                            const T *__restrict__ u, double *__restrict__ partial) {
+                                                            const float *__restrict__ u, double *__restrict__ partial) {
   extern __shared__ __align__(16) unsigned char gsm2[];
   double *wd = reinterpret_cast<double *>(gsm2);
   double *red = wd + d;                                     // [warp][2d]
@@ -249,42 +250,42 @@ __global__ void __launch_bounds__(kHoNT) k_grad_partials_ho(uint32_t d, int orde
     zl[q] = xor_columns64(Cr + j * 32, order_map(order, (uint32_t)(tile_base | ((uint64_t)l << 8))));
   }
   __syncthreads();
-  T p[kHoColL], uu[kHoColL], k1[kHoColL];
+  float p[kHoColL], uu[kHoColL], k1[kHoColL];
   bool ok[kHoColL];
 #pragma unroll
   for (int l = 0; l < kHoColL; ++l) {
     const uint64_t i = tile_base + t + ((uint64_t)l << 8);
     ok[l] = i < n;
-    uu[l] = ok[l] ? u[(size_t)v * n + i] : T(0);
-    p[l] = T(0);
+    uu[l] = ok[l] ? u[(size_t)v * n + i] : 0.f;
+    p[l] = 0.f;
   }
   for (uint32_t j = 0; j < d; ++j) {
-    const T wj = (T)wd[j];
+    const float wj = (float)wd[j];
     const uint64_t b = zlane[j * 32 + lane] ^ zwarp[warp * d + j];
 #pragma unroll
-    for (int l = 0; l < kHoColL; ++l) p[l] = pm1_step(p[l], wj * dsi_factor64<T, ALPHA>(b ^ zl[j * kHoColL + l]));
+    for (int l = 0; l < kHoColL; ++l) p[l] = pm1_step(p[l], wj * dsi_factor64<float, ALPHA>(b ^ zl[j * kHoColL + l]));
   }
 #pragma unroll
-  for (int l = 0; l < kHoColL; ++l) k1[l] = ok[l] ? (T)zeta * (T(1) + p[l]) : T(0);
+  for (int l = 0; l < kHoColL; ++l) k1[l] = ok[l] ? (float)zeta * (1.f + p[l]) : 0.f;
   for (uint32_t j = 0; j < d; ++j) {
-    const T wj = (T)wd[j];
+    const float wj = (float)wd[j];
     const uint64_t b = zlane[j * 32 + lane] ^ zwarp[warp * d + j];
     double su = 0.0, s1 = 0.0;
 #pragma unroll
     for (int l = 0; l < kHoColL; ++l) {
       if (!ok[l]) continue;
       const uint64_t bl = b ^ zl[j * kHoColL + l];
-      const T K = dsi_factor64<T, ALPHA>(bl);
-      const T f = fmadd(wj, K, T(1));
-      T dk;
-      if (f != T(0)) {
+      const float K = dsi_factor64<float, ALPHA>(bl);
+      const float f = fmadd(wj, K, 1.f);
+      float dk;
+      if (f != 0.f) {
         dk = k1[l] * (K / f);
       } else {  // 1 + c_j K = 0: the product of the other factors, explicitly
-        dk = (T)zeta * K;
+        dk = (float)zeta * K;
         for (uint32_t jj = 0; jj < d; ++jj) {
           if (jj == j) continue;
           const uint64_t bj = zlane[jj * 32 + lane] ^ zwarp[warp * d + jj] ^ zl[jj * kHoColL + l];
-          dk *= T(1) + (T)wd[jj] * dsi_factor64<T, ALPHA>(bj);
+          dk *= 1.f + (float)wd[jj] * dsi_factor64<float, ALPHA>(bj);
         }
       }
       su += (double)uu[l] * (double)dk;
@@ -309,36 +310,42 @@ __global__ void __launch_bounds__(kHoNT) k_grad_partials_ho(uint32_t d, int orde
   }
 }
 
-template <typename T, int ALPHA>
-static int launch_grad_ho_t(const ColJob &job, uint32_t nrhs, const T *u, double *partial, cudaStream_t st) {
+template <int ALPHA>
+static int launch_grad_ho_t(const ColJob &job, uint32_t nrhs, const float *u, double *partial, cudaStream_t st) {
   const uint32_t d = job.d;
   const uint64_t n = 1ull << job.m;
   const size_t smem = sizeof(double) * ((size_t)d + (kHoNT / 32) * 2 * d) +
                       sizeof(uint64_t) * ((size_t)32 * d + (kHoNT / 32) * d + kHoColL * d);
-  smem_optin<k_grad_partials_ho<T, ALPHA>>(smem);
+  smem_optin<k_grad_partials_ho<ALPHA>>(smem);
   const uint64_t nvec = (uint64_t)job.nr * nrhs;
   if (nvec > 65535) return fail(QK_EINVAL, "higher-order gradient: more than 65535 vectors per call");
   dim3 grid(ceil_div_u(n, kHoNT * kHoColL), (unsigned)nvec);
-  k_grad_partials_ho<T, ALPHA><<<grid, kHoNT, smem, st>>>(d, job.order, job.m, nrhs, job.Chat, job.w, job.zeta, u,
+  k_grad_partials_ho<ALPHA><<<grid, kHoNT, smem, st>>>(d, job.order, job.m, nrhs, job.Chat, job.w, job.zeta, u,
                                                           partial);
   return check_launch("higher-order gradient partials");
 }
 
-template <typename T>
-static int dispatch_grad_ho(const ColJob &job, uint32_t nrhs, const T *u, double *partial, cudaStream_t st) {
+static int dispatch_grad_ho(const ColJob &job, uint32_t nrhs, const float *u, double *partial, cudaStream_t st) {
   switch (job.alpha) {
-    case 1: return launch_grad_ho_t<T, 1>(job, nrhs, u, partial, st);
-    case 2: return launch_grad_ho_t<T, 2>(job, nrhs, u, partial, st);
-    case 3: return launch_grad_ho_t<T, 3>(job, nrhs, u, partial, st);
-    case 4: return launch_grad_ho_t<T, 4>(job, nrhs, u, partial, st);
+    case 1: return launch_grad_ho_t<1>(job, nrhs, u, partial, st);
+    case 2: return launch_grad_ho_t<2>(job, nrhs, u, partial, st);
+    case 3: return launch_grad_ho_t<3>(job, nrhs, u, partial, st);
+    case 4: return launch_grad_ho_t<4>(job, nrhs, u, partial, st);
     default: return fail(QK_EINVAL, "DSI order must be 1..4");
   }
 }
 
 int launch_grad_partials_ho(const ColJob &job, uint32_t nrhs, int32_t dtype, const void *u, double *partial,
                             cudaStream_t st) {
-  return dtype == QK_F64 ? dispatch_grad_ho<double>(job, nrhs, (const double *)u, partial, st)
-                         : dispatch_grad_ho<float>(job, nrhs, (const float *)u, partial, st);
+  if (dtype != QK_F64) return dispatch_grad_ho(job, nrhs, (const float *)u, partial, st);
+  const double *ud = (const double *)u;
+  switch (job.alpha) {
+    case 1: return launch_grad64<2, 1>(job, job.Chat, job.nr, nrhs, ud, 0, nullptr, partial, st);
+    case 2: return launch_grad64<2, 2>(job, job.Chat, job.nr, nrhs, ud, 0, nullptr, partial, st);
+    case 3: return launch_grad64<2, 3>(job, job.Chat, job.nr, nrhs, ud, 0, nullptr, partial, st);
+    case 4: return launch_grad64<2, 4>(job, job.Chat, job.nr, nrhs, ud, 0, nullptr, partial, st);
+    default: return fail(QK_EINVAL, "DSI order must be 1..4");
+  }
 }
 
 static int check_hopointset(const qk_hopointset *ps, uint32_t r0, uint32_t nr) {

@@ -51,10 +51,12 @@ int launch_kernel_col(const ColJob &job, int32_t dtype, int32_t form, void *out,
 // instead: vector v is the real (v even) or imaginary (v odd) part of complex vector v / 2.
 // pcol (nullable): the job's first column in p form, FP64 (nr, n), read instead of a
 // second column sweep.  partial: (nr * nrhs, blocks, 2d) doubles with
-// blocks = grad_blocks(m): [0, d) sum_i u_i dk1_i/dc_j, [d, 2d) sum_i dk1_i/dc_j.
+// blocks = grad_blocks(m, dtype is QK_F64): [0, d) sum_i u_i dk1_i/dc_j, [d, 2d) sum_i dk1_i/dc_j.
 int launch_grad_partials(const ColJob &job, uint32_t nrhs, int32_t dtype, const void *u,
                          double *partial, cudaStream_t st, bool pairs = false, const double *pcol = nullptr);
-uint32_t grad_blocks(uint32_t m);
+uint32_t grad_blocks(uint32_t m, bool fp64);
+int launch_grad_partials_f64(const ColJob &job, uint32_t nrhs, const double *u, double *partial, cudaStream_t st,
+                             bool pairs, const double *pcol);
 
 int launch_gen_points(const qk_pointset *ps, uint32_t r0, uint32_t nr, uint64_t i0, uint64_t n,
                       uint32_t *X, cudaStream_t st);

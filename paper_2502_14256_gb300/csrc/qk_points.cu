@@ -16,6 +16,7 @@
 #include "qk_factors.cuh"
 #include "qk_internal.h"
 #include "qk_column.cuh"
+#include "qk_grad.cuh"
 
 namespace qk {
 
@@ -339,27 +340,28 @@ int launch_kernel_col(const ColJob &job, int32_t dtype, int32_t form, void *out,
 
 // ------------------------------------------------------- gradient partials
 // dk_1[i]/dc_j = zeta K_ij prod_{j' != j} f_ij' with f_ij = 1 + c_j K_ij, computed as
-// zeta (1 + p_i) K_ij / f_ij (explicit product where f_ij == 0).
-template <typename T, int FAM, int ALPHA>
-__global__ void __launch_bounds__(kNT) k_grad_partials(ColJob job, uint32_t nrhs, const T *__restrict__ u,
+// zeta (1 + p_i) K_ij / f_ij (explicit product where f_ij == 0).  FP32 sweeps; FP64 ones are in
+// qk_grad.cuh.
+template <int FAM, int ALPHA>
+__global__ void __launch_bounds__(kNT) k_grad_partials(ColJob job, uint32_t nrhs, const float *__restrict__ u,
                                                        double *__restrict__ partial, int pairs,
                                                        const double *__restrict__ pcol) {
   extern __shared__ __align__(16) unsigned char smem[];
   double *wd;
   DiffTables tb;
   carve_tables<kL>(smem, job.d, &wd, tb);
-  T *wT = reinterpret_cast<T *>(wd);
+  float *wT = reinterpret_cast<float *>(wd);
   const uint32_t d = job.d;
   double *red = reinterpret_cast<double *>(smem + col_smem_bytes<kL>(d));  // [warp][2d]
   const uint32_t v = blockIdx.y;  // vector = r * nrhs + rhs
   const uint32_t rl = v / nrhs;
   const uint64_t n = 1ull << job.m;
   const uint64_t tile_base = (uint64_t)blockIdx.x * kTile;
-  for (uint32_t q = threadIdx.x; q < d; q += kNT) wT[q] = (T)job.w[q];
-  build_all<T, FAM, ALPHA, kL>(job, job.Ct ? job.Ct + (size_t)rl * d * 32 : nullptr, job.g, tile_base, tb);
+  for (uint32_t q = threadIdx.x; q < d; q += kNT) wT[q] = (float)job.w[q];
+  build_all<float, FAM, ALPHA, kL>(job, job.Ct ? job.Ct + (size_t)rl * d * 32 : nullptr, job.g, tile_base, tb);
   __syncthreads();
   uint32_t bi[kL];
-  T uu[kL], k1[kL];
+  float uu[kL], k1[kL];
   bool ok[kL];
 #pragma unroll
   for (int l = 0; l < kL; ++l) {
@@ -367,32 +369,32 @@ __global__ void __launch_bounds__(kNT) k_grad_partials(ColJob job, uint32_t nrhs
     bi[l] = __brev((uint32_t)i);
     ok[l] = i < n;
     const size_t ui = pairs ? ((((size_t)(v >> 1) * n) + i) << 1) + (v & 1) : (size_t)v * n + i;
-    uu[l] = ok[l] ? u[ui] : T(0);
+    uu[l] = ok[l] ? u[ui] : 0.f;
   }
-  T p[kL];
+  float p[kL];
   if (pcol) {  // the first column as computed before (p form, FP64): no second column sweep
 #pragma unroll
     for (int l = 0; l < kL; ++l) {
       const uint64_t i = tile_base + threadIdx.x + ((uint64_t)l << 8);
-      p[l] = ok[l] ? (T)pcol[(size_t)rl * n + i] : T(0);
+      p[l] = ok[l] ? (float)pcol[(size_t)rl * n + i] : 0.f;
     }
   } else {
-    column_sweep<T, FAM, ALPHA, kL>(job, tb, wT, bi, p);
+    column_sweep<float, FAM, ALPHA, kL>(job, tb, wT, bi, p);
   }
-  const T zeta = (T)job.zeta;
-  T wk[kL];
+  const float zeta = (float)job.zeta;
+  float wk[kL];
 #pragma unroll
   for (int l = 0; l < kL; ++l) {
-    k1[l] = ok[l] ? zeta * (T(1) + p[l]) : T(0);
+    k1[l] = ok[l] ? zeta * (1.f + p[l]) : 0.f;
     wk[l] = uu[l] * k1[l];
   }
-  gradient_sweep<T, FAM, ALPHA, kL>(job, tb, wT, bi, k1, wk, ok, [&](int l) { return uu[l]; }, red);
+  gradient_sweep<FAM, ALPHA, kL>(job, tb, wT, bi, k1, wk, ok, [&](int l) { return uu[l]; }, red);
   __syncthreads();
   double *dst = partial + ((size_t)v * gridDim.x + blockIdx.x) * 2 * d;
-  for (uint32_t q = threadIdx.x; q < 2 * d; q += kNT) dst[q] = red_total<T>(red, kNT / 32, 2 * d, q);
+  for (uint32_t q = threadIdx.x; q < 2 * d; q += kNT) dst[q] = red_total(red, kNT / 32, 2 * d, q);
 }
 
-uint32_t grad_blocks(uint32_t m) { return ceil_div_u(1ull << m, kTile); }
+uint32_t grad_blocks(uint32_t m, bool fp64) { return fp64 ? grad64_blocks(m) : ceil_div_u(1ull << m, kTile); }
 
 __global__ void k_ratio_selftest(const double *__restrict__ a, const double *__restrict__ b, double *__restrict__ q,
                                  uint64_t n) {
@@ -400,30 +402,29 @@ __global__ void k_ratio_selftest(const double *__restrict__ a, const double *__r
     q[i] = ratio(a[i], b[i]);
 }
 
-template <typename T, int FAM, int ALPHA>
-static void launch_grad_t(const ColJob &job, uint32_t nrhs, const T *u, double *partial, int pairs,
+template <int FAM, int ALPHA>
+static void launch_grad_t(const ColJob &job, uint32_t nrhs, const float *u, double *partial, int pairs,
                           const double *pcol, cudaStream_t st) {
-  dim3 grid(grad_blocks(job.m), job.nr * nrhs);
+  dim3 grid(grad_blocks(job.m, false), job.nr * nrhs);
   const size_t smem = col_smem_bytes<kL>(job.d) + (size_t)(kNT / 32) * 2 * job.d * sizeof(double);
-  smem_optin<k_grad_partials<T, FAM, ALPHA>>(smem);
-  k_grad_partials<T, FAM, ALPHA><<<grid, kNT, smem, st>>>(job, nrhs, u, partial, pairs, pcol);
+  smem_optin<k_grad_partials<FAM, ALPHA>>(smem);
+  k_grad_partials<FAM, ALPHA><<<grid, kNT, smem, st>>>(job, nrhs, u, partial, pairs, pcol);
 }
 
-template <typename T>
-static int dispatch_grad(const ColJob &job, uint32_t nrhs, const T *u, double *partial, int pairs,
+static int dispatch_grad(const ColJob &job, uint32_t nrhs, const float *u, double *partial, int pairs,
                          const double *pcol, cudaStream_t st) {
   if (job.family == QK_DSI) {
     switch (job.alpha) {
-      case 1: launch_grad_t<T, 0, 1>(job, nrhs, u, partial, pairs, pcol, st); break;
-      case 2: launch_grad_t<T, 0, 2>(job, nrhs, u, partial, pairs, pcol, st); break;
-      case 3: launch_grad_t<T, 0, 3>(job, nrhs, u, partial, pairs, pcol, st); break;
-      case 4: launch_grad_t<T, 0, 4>(job, nrhs, u, partial, pairs, pcol, st); break;
+      case 1: launch_grad_t<0, 1>(job, nrhs, u, partial, pairs, pcol, st); break;
+      case 2: launch_grad_t<0, 2>(job, nrhs, u, partial, pairs, pcol, st); break;
+      case 3: launch_grad_t<0, 3>(job, nrhs, u, partial, pairs, pcol, st); break;
+      case 4: launch_grad_t<0, 4>(job, nrhs, u, partial, pairs, pcol, st); break;
       default: return fail(QK_EINVAL, "DSI order must be 1..4");
     }
   } else {
     switch (job.alpha) {
-      case 1: launch_grad_t<T, 1, 1>(job, nrhs, u, partial, pairs, pcol, st); break;
-      case 2: launch_grad_t<T, 1, 2>(job, nrhs, u, partial, pairs, pcol, st); break;
+      case 1: launch_grad_t<1, 1>(job, nrhs, u, partial, pairs, pcol, st); break;
+      case 2: launch_grad_t<1, 2>(job, nrhs, u, partial, pairs, pcol, st); break;
       default: return fail(QK_EINVAL, "SI smoothness must be 1 or 2");
     }
   }
@@ -437,8 +438,8 @@ int launch_grad_partials(const ColJob &job, uint32_t nrhs, int32_t dtype, const 
     if (pairs || pcol) return fail(QK_EINVAL, "gradient partials: pair layout and stored column are for lattices");
     return launch_grad_partials_ho(job, nrhs, dtype, u, partial, st);
   }
-  return dtype == QK_F64 ? dispatch_grad<double>(job, nrhs, (const double *)u, partial, pairs ? 1 : 0, pcol, st)
-                         : dispatch_grad<float>(job, nrhs, (const float *)u, partial, pairs ? 1 : 0, pcol, st);
+  return dtype == QK_F64 ? launch_grad_partials_f64(job, nrhs, (const double *)u, partial, st, pairs, pcol)
+                         : dispatch_grad(job, nrhs, (const float *)u, partial, pairs ? 1 : 0, pcol, st);
 }
 
 }  // namespace qk

@@ -529,7 +529,7 @@ size_t ws_mll(int family, uint32_t m, uint32_t nr, uint32_t nrhs, int dtype, uin
   s = add_sat(s, align256(nv * spec_blocks(m) * 2 * sizeof(double)));
   s = add_sat(s, align256((uint64_t)nr * spec_blocks(m) * sizeof(double)));
   s = add_sat(s, align256(nv * spec_blocks(m) * sizeof(double)));
-  s = add_sat(s, align256(nv * grad_blocks(m) * 2 * (uint64_t)d * sizeof(double)));
+  s = add_sat(s, align256(nv * grad_blocks(m, dtype == QK_F64) * 2 * (uint64_t)d * sizeof(double)));
   return s;
 }
 
@@ -904,7 +904,7 @@ static int mll_t(const ColJob &job, uint32_t nrhs, const double *lam, const T *y
   fa.d = job.d;
   fa.bspec = bs;
   fa.blog = bs;
-  fa.bgrad = grad_blocks(m);
+  fa.bgrad = grad_blocks(m, sizeof(T) == 8);
   fa.m = (int)m;
   fa.zeta = job.zeta;
   fa.lam = lam;
@@ -935,7 +935,7 @@ static size_t ws_mll_si_t(uint32_t m, uint32_t nr, uint32_t nrhs, uint32_t d, bo
   s = add_sat(s, align256(nv * spec_blocks(m) * 2 * sizeof(double)));
   s = add_sat(s, align256((uint64_t)nr * spec_blocks(m) * sizeof(double)));
   s = add_sat(s, align256(nv * spec_blocks(m) * sizeof(double)));
-  s = add_sat(s, align256(nv * grad_blocks(m) * 2 * (uint64_t)d * sizeof(double)));
+  s = add_sat(s, align256(nv * grad_blocks(m, sizeof(EO) == sizeof(double2)) * 2 * (uint64_t)d * sizeof(double)));
   return s;
 }
 
@@ -1005,7 +1005,7 @@ static int mll_si_t(const ColJob &job, uint32_t nrhs, const double *lam, const T
   fa.d = job.d;
   fa.bspec = bs;
   fa.blog = bs;
-  fa.bgrad = grad_blocks(m);
+  fa.bgrad = grad_blocks(m, sizeof(T) == 8);
   fa.m = (int)m;
   fa.zeta = job.zeta;
   fa.lam = lam;
