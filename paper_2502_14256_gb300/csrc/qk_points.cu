@@ -217,79 +217,111 @@ int launch_gen_points(const qk_pointset *ps, uint32_t r0, uint32_t nr, uint64_t 
   return check_launch("qk_gen_points");
 }
 
-template <typename T, int FAM, int ALPHA>
-__global__ void __launch_bounds__(kNT) k_kernel_col(ColJob job, int form, T *__restrict__ out) {
+// First columns.  A CTA covers kNT L points of one randomization (positions job.i0 + [0, n);
+// job.i0 is a multiple of kTile, so position bits split into disjoint tile, l, warp and lane
+// fields for the XOR tables) and writes `copies` equal rows: a lattice's differences do not
+// depend on the shift, so its column is formed once for all randomizations (n = 2^18, d = 32,
+// 16 shifts, FP64: 1278 us one by one, 95 us once).
+template <typename T, int FAM, int ALPHA, int L>
+__global__ void __launch_bounds__(kNT) k_kernel_col(ColJob job, int form, uint32_t copies, T *__restrict__ out) {
   extern __shared__ __align__(16) unsigned char smem[];
   double *wd;
   DiffTables tb;
-  carve_tables<kL>(smem, job.d, &wd, tb);
+  carve_tables<L>(smem, job.d, &wd, tb);
   T *wT = reinterpret_cast<T *>(wd);
   const uint32_t rl = blockIdx.y;
   const uint64_t n = 1ull << job.m;
-  // positions job.i0 + [0, n); job.i0 is a multiple of kTile, so position bits split into
-  // disjoint tile, l, warp and lane fields for the XOR tables
-  const uint64_t tile_base = job.i0 + (uint64_t)blockIdx.x * kTile;
+  const uint64_t tile_base = job.i0 + (uint64_t)blockIdx.x * (kNT * L);
   for (uint32_t q = threadIdx.x; q < job.d; q += kNT) wT[q] = (T)job.w[q];
-  build_all<T, FAM, ALPHA, kL>(job, job.Ct ? job.Ct + (size_t)rl * job.d * 32 : nullptr, job.g, tile_base, tb);
+  build_all<T, FAM, ALPHA, L>(job, job.Ct ? job.Ct + (size_t)rl * job.d * 32 : nullptr, job.g, tile_base, tb);
   __syncthreads();
-  uint32_t bi[kL];
+  uint32_t bi[L];
 #pragma unroll
-  for (int l = 0; l < kL; ++l) bi[l] = __brev((uint32_t)(tile_base + threadIdx.x + (l << 8)));
-  T p[kL];
-  column_sweep<T, FAM, ALPHA, kL>(job, tb, wT, bi, p);
+  for (int l = 0; l < L; ++l) bi[l] = __brev((uint32_t)(tile_base + threadIdx.x + (l << 8)));
+  T p[L];
+  column_sweep<T, FAM, ALPHA, L>(job, tb, wT, bi, p);
   const T zeta = (T)job.zeta;
 #pragma unroll
-  for (int l = 0; l < kL; ++l) {
-    const uint64_t i = tile_base - job.i0 + threadIdx.x + ((uint64_t)l << 8);
-    if (i < n) out[(size_t)rl * n + i] = form == QK_COL_P ? p[l] : zeta * (T(1) + p[l]);
-  }
-}
-
-template <typename T, int FAM, int ALPHA>
-static void launch_col_t(const ColJob &job, int form, T *out, cudaStream_t st) {
-  const uint64_t n = 1ull << job.m;
-  dim3 grid(ceil_div_u(n, kTile), job.nr);
-  const size_t smem = col_smem_bytes<kL>(job.d);
-  smem_optin<k_kernel_col<T, FAM, ALPHA>>(smem);
-  k_kernel_col<T, FAM, ALPHA><<<grid, kNT, smem, st>>>(job, form, out);
+  for (int l = 0; l < L; ++l)
+    if (form != QK_COL_P) p[l] = zeta * (T(1) + p[l]);
+  for (uint32_t c = 0; c < copies; ++c)
+#pragma unroll
+    for (int l = 0; l < L; ++l) {
+      const uint64_t i = tile_base - job.i0 + threadIdx.x + ((uint64_t)l << 8);
+      if (i < n) out[((size_t)rl + c) * n + i] = p[l];
+    }
 }
 
 // The first column in float-float arithmetic on the FP32 pipes (about 2^-46 relative per
 // factor), written as FP64: for spectra that reach far below eps32 ||k_1||, where an FP32
 // column would perturb the small eigenvalues beyond the 1/lambda-weighted outputs' tolerance.
-template <int FAM, int ALPHA>
-__global__ void __launch_bounds__(kNT) k_kernel_col_ff(ColJob job, int form, double *__restrict__ out) {
+template <int FAM, int ALPHA, int L>
+__global__ void __launch_bounds__(kNT) k_kernel_col_ff(ColJob job, int form, uint32_t copies, double *__restrict__ out) {
   extern __shared__ __align__(16) unsigned char smem[];
   double *wd;
   DiffTables tb;
-  carve_tables<kL>(smem, job.d, &wd, tb);
+  carve_tables<L>(smem, job.d, &wd, tb);
   float2 *wff = reinterpret_cast<float2 *>(wd);
   const uint32_t rl = blockIdx.y;
   const uint64_t n = 1ull << job.m;
-  const uint64_t tile_base = job.i0 + (uint64_t)blockIdx.x * kTile;
+  const uint64_t tile_base = job.i0 + (uint64_t)blockIdx.x * (kNT * L);
   for (uint32_t q = threadIdx.x; q < job.d; q += kNT) wff[q] = ff_split(job.w[q]);
-  build_all_ff<FAM, ALPHA, kL>(job, job.Ct ? job.Ct + (size_t)rl * job.d * 32 : nullptr, job.g, tile_base, tb);
+  build_all_ff<FAM, ALPHA, L>(job, job.Ct ? job.Ct + (size_t)rl * job.d * 32 : nullptr, job.g, tile_base, tb);
   __syncthreads();
-  uint32_t bi[kL];
+  uint32_t bi[L];
 #pragma unroll
-  for (int l = 0; l < kL; ++l) bi[l] = __brev((uint32_t)(tile_base + threadIdx.x + (l << 8)));
-  float ph[kL], pl[kL];
-  column_sweep_ff<FAM, ALPHA, kL>(job, tb, wff, bi, ph, pl);
+  for (int l = 0; l < L; ++l) bi[l] = __brev((uint32_t)(tile_base + threadIdx.x + (l << 8)));
+  float ph[L], pl[L];
+  column_sweep_ff<FAM, ALPHA, L>(job, tb, wff, bi, ph, pl);
 #pragma unroll
-  for (int l = 0; l < kL; ++l) {
+  for (int l = 0; l < L; ++l) {
     const uint64_t i = tile_base - job.i0 + threadIdx.x + ((uint64_t)l << 8);
-    const double p = f2d_exact(ph[l]) + f2d_exact(pl[l]);
-    if (i < n) out[(size_t)rl * n + i] = form == QK_COL_P ? p : job.zeta + job.zeta * p;
+    double p = f2d_exact(ph[l]) + f2d_exact(pl[l]);
+    if (form != QK_COL_P) p = job.zeta + job.zeta * p;
+    if (i < n)
+      for (uint32_t c = 0; c < copies; ++c) out[((size_t)rl + c) * n + i] = p;
   }
 }
 
+// Rows to compute and copies of each: lattices one row for all randomizations.
+static void col_rows(const ColJob &job, uint32_t &rows, uint32_t &copies) {
+  const bool shared = job.kind == QK_LATTICE;
+  rows = shared ? 1 : job.nr;
+  copies = shared ? job.nr : 1;
+}
+// Points per thread: 8, or LS where tiles of 8 would leave fewer than four CTAs per SM (a
+// column of 2^18 points is 128 tiles of 2048 on 152 SMs).
+static bool col_small(const ColJob &job, uint32_t rows) {
+  return (uint64_t)ceil_div_u(1ull << job.m, kTile) * rows < 4ull * sm_count();
+}
+
+template <typename T, int FAM, int ALPHA, int L>
+static void launch_col_l(const ColJob &job, int form, uint32_t rows, uint32_t copies, T *out, cudaStream_t st) {
+  const size_t smem = col_smem_bytes<L>(job.d);
+  smem_optin<k_kernel_col<T, FAM, ALPHA, L>>(smem);
+  k_kernel_col<T, FAM, ALPHA, L><<<dim3(ceil_div_u(1ull << job.m, kNT * L), rows), kNT, smem, st>>>(job, form, copies, out);
+}
+template <typename T, int FAM, int ALPHA>
+static void launch_col_t(const ColJob &job, int form, T *out, cudaStream_t st) {
+  constexpr int LS = sizeof(T) == 8 ? 2 : 4;
+  uint32_t rows, copies;
+  col_rows(job, rows, copies);
+  if (col_small(job, rows)) launch_col_l<T, FAM, ALPHA, LS>(job, form, rows, copies, out, st);
+  else launch_col_l<T, FAM, ALPHA, kL>(job, form, rows, copies, out, st);
+}
+
+template <int FAM, int ALPHA, int L>
+static void launch_col_ff_l(const ColJob &job, int form, uint32_t rows, uint32_t copies, double *out, cudaStream_t st) {
+  const size_t smem = col_smem_bytes<L>(job.d);
+  smem_optin<k_kernel_col_ff<FAM, ALPHA, L>>(smem);
+  k_kernel_col_ff<FAM, ALPHA, L><<<dim3(ceil_div_u(1ull << job.m, kNT * L), rows), kNT, smem, st>>>(job, form, copies, out);
+}
 template <int FAM, int ALPHA>
 static void launch_col_ff(const ColJob &job, int form, double *out, cudaStream_t st) {
-  const uint64_t n = 1ull << job.m;
-  dim3 grid(ceil_div_u(n, kTile), job.nr);
-  const size_t smem = col_smem_bytes<kL>(job.d);
-  smem_optin<k_kernel_col_ff<FAM, ALPHA>>(smem);
-  k_kernel_col_ff<FAM, ALPHA><<<grid, kNT, smem, st>>>(job, form, out);
+  uint32_t rows, copies;
+  col_rows(job, rows, copies);
+  if (col_small(job, rows)) launch_col_ff_l<FAM, ALPHA, 4>(job, form, rows, copies, out, st);
+  else launch_col_ff_l<FAM, ALPHA, kL>(job, form, rows, copies, out, st);
 }
 
 static int dispatch_col_ff(const ColJob &job, int form, double *out, cudaStream_t st) {
@@ -372,11 +404,12 @@ __global__ void __launch_bounds__(kNT) k_grad_partials(ColJob job, uint32_t nrhs
     uu[l] = ok[l] ? u[ui] : 0.f;
   }
   float p[kL];
-  if (pcol) {  // the first column as computed before (p form, FP64): no second column sweep
+  if (pcol) {  // the first column as computed before (p form, FP64; lattices: one row for all shifts)
+    const uint32_t pr = FAM == 1 ? 0u : rl;
 #pragma unroll
     for (int l = 0; l < kL; ++l) {
       const uint64_t i = tile_base + threadIdx.x + ((uint64_t)l << 8);
-      p[l] = ok[l] ? (float)pcol[(size_t)rl * n + i] : 0.f;
+      p[l] = ok[l] ? (float)pcol[(size_t)pr * n + i] : 0.f;
     }
   } else {
     column_sweep<float, FAM, ALPHA, kL>(job, tb, wT, bi, p);
