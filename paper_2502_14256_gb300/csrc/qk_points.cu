@@ -49,171 +49,193 @@ int launch_lms(uint32_t d, uint32_t R, const uint32_t *C, const uint32_t *S, uin
 }
 
 // ---------------------------------------------------------- point generation
-// By tiles: a CTA builds NP consecutive points (aligned to NP) of every dimension of one
-// randomization in shared memory, row-major as in the output, then writes the part inside
-// [i0, i0 + n) as one contiguous, coalesced run of words.  Inside the tile a thread makes a
-// run of kGenRL = 8 consecutive points of one dimension:
-//   nets: the index maps h(i) = i and i ^ (i >> 1) are linear over GF(2) and the tile, run
-//   and step bits of i are disjoint, so the run's first point is the XOR of a per-tile word,
-//   a per-run word (both tables built once per CTA) and the shift; each next point is one
-//   XOR with a column known at compile time: Gray order changes digit ctz(k + 1) (Sec. 4.3,
-//   Gray code), natural order all digits below it (the XOR of columns 0 .. ctz(k + 1));
-//   lattices: X_i = brev(i) g + D, one multiply-add per point.
-constexpr int kGenNT = 256, kGenRL = 8, kGenWords = 8192;
+// Store-bound: 4 n d R bytes.  A tile is NP = 2^lognp consecutive points (aligned to NP) of every
+// dimension of one randomization: NP d consecutive output words, written by NTA = NP d / 32
+// threads as 8 groups of 4 words each, thread t's group `it` at word 4 t + 4 NTA it: whole warps
+// store 512 consecutive bytes.  4 NTA words are 2^(lognp - 3) points, so a thread's four words
+// keep their dimensions, and the points' index bits split into disjoint fields: position inside
+// the group, it (3 bits), tile.  The index maps h(i) = i and i ^ (i >> 1) are linear over GF(2),
+// so with one word per field
+//   nets:     X = F(thread) ^ A(it) ^ T(tile), T stepping by the XOR of the columns of the tile
+//             bits that flip (one table word per step);
+//   lattices: brev(i) g is additive over the fields: X = F + A(it) + T, T = brev(tile) g + D,
+// i.e. one XOR or add per word and a 16-byte store per four, no shared-memory staging and no
+// barrier between tiles (32 x 1000003 x 13 words: see the launch below).
+// Groups are aligned to 16 bytes in memory: where a randomization's tiles start phi words past
+// such a boundary, the groups shift down by phi; thread 0's first phi words then belong to the
+// end of the group region before (for its first group: to the tile's end), and it stores word by
+// word.  So do the tiles cut by the range's ends.
+constexpr int kGenNT = 256;
 
-// log2 of the tile's point count: the largest power of two with NP d <= kGenWords (NP >= RL).
+// log2 of the tile's points: NTA = 2^(lognp - 5) d threads, the largest that fit a CTA.
 static uint32_t gen_lognp(uint32_t d) {
-  uint32_t l = 0;
-  while ((2u << l) * d <= (uint32_t)kGenWords) ++l;
-  return l < 3 ? 3 : l;
+  uint32_t k = 5;
+  while ((2u << (k - 5)) * d <= (uint32_t)kGenNT) ++k;
+  return k;
 }
 
 template <bool NET>
-__global__ void __launch_bounds__(kGenNT) k_points_tiled(uint32_t d, int order, const uint32_t *__restrict__ Ct,
-                                                         const uint32_t *__restrict__ g, const uint32_t *__restrict__ D,
-                                                         uint32_t r0, uint32_t nr, uint64_t i0, uint64_t n,
-                                                         uint32_t lognp, uint32_t tiles, int direct,
-                                                         uint32_t *__restrict__ X) {
-  extern __shared__ __align__(16) uint32_t gsm[];
-  const uint32_t NP = 1u << lognp, runs = (NP / kGenRL) * d;
-  // direct: rows of d >= 16 words are written from registers (a warp's store covers whole
-  // 64-byte row pieces); otherwise the tile is staged in shared memory first
-  uint32_t *tile = gsm;             // NP x d (staged form only)
-  uint32_t *sC = tile + (direct ? 0 : NP * d);  // nets: d x 32 columns; lattices: g
-  uint32_t *zrun = sC + 32 * d;     // nets: (NP / RL) x d run words
-  uint32_t *ztile = zrun + runs;    // d tile words (shift included)
-  const int t = threadIdx.x;
-  // work items (randomization, tile) in order; each CTA takes one contiguous chunk, so the
-  // per-randomization set-up (columns, run words) is redone only where the chunk crosses
-  // into the next randomization
+__device__ __forceinline__ uint32_t gen_add(uint32_t a, uint32_t b) {
+  if constexpr (NET) return a ^ b;
+  else return a + b;
+}
+
+template <bool NET>
+__global__ void __launch_bounds__(kGenNT) k_points(uint32_t d, int order, const uint32_t *__restrict__ Ct,
+                                                   const uint32_t *__restrict__ g, const uint32_t *__restrict__ D,
+                                                   uint32_t r0, uint32_t nr, uint64_t i0, uint64_t n, uint32_t lognp,
+                                                   uint32_t tiles, uint32_t *__restrict__ X) {
+  // nets: sC[j][k] = word of position 1 << k (Gray order: columns k and k - 1), rows of 33 words;
+  // sP[j][c] = XOR of the words of tile bits 0 .. c
+  extern __shared__ uint32_t gsm[];
+  uint32_t *sC = gsm, *sP = gsm + 33 * d;
+  const uint32_t t = threadIdx.x, NP = 1u << lognp, NTA = d << (lognp - 5), words = NP * d;
+  const bool active = t < NTA;
   const uint64_t total = (uint64_t)nr * tiles, chunk = (total + gridDim.x - 1) / gridDim.x;
   const uint64_t it0 = (uint64_t)blockIdx.x * chunk, it1 = it0 + chunk < total ? it0 + chunk : total;
-  uint32_t cur = 0xFFFFFFFFu;
-  for (uint64_t it = it0; it < it1; ++it) {
-    const uint32_t rl = (uint32_t)(it / tiles), tt = (uint32_t)(it - (uint64_t)rl * tiles), r = r0 + rl;
-    if (rl != cur) {  // the previous item's run phase ended at a barrier: sC / zrun are free
-      cur = rl;
+  if (it0 >= it1) return;
+  uint32_t rl = (uint32_t)(it0 / tiles), tt = (uint32_t)(it0 - (uint64_t)rl * tiles);
+  bool fresh = true;                        // a new randomization: tables and the thread's words
+  uint32_t phi = 0;                         // its alignment shift
+  uint32_t F[4], A[3][4], T[4], J[4], E[4];  // E: word index in the group's region; J: nets j, lattices g_j
+  uint32_t *out = X;                        // word 0 of the tile
+  for (uint64_t left = it1 - it0; left; --left) {
+    const uint32_t r = r0 + rl;
+    const uint64_t tile = (i0 >> lognp) + tt, base = tile << lognp;  // < 2^32
+    if (fresh) {
       if constexpr (NET) {
-        for (uint32_t q = t; q < 32 * d; q += kGenNT) sC[q] = Ct[(size_t)r * d * 32 + q];
         __syncthreads();
-        for (uint32_t w = t; w < runs; w += kGenNT) {
-          const uint32_t q = w / d, j = w - q * d;
-          zrun[w] = xor_columns(sC + j * 32, order_map(order, q * kGenRL));
+        const uint32_t *C = Ct + (size_t)r * d * 32;
+        for (uint32_t q = t; q < 32 * d; q += blockDim.x) {
+          const uint32_t j = q >> 5, k = q & 31;
+          const uint32_t c = C[q];
+          sC[j * 33 + k] = order == QK_GRAY && k ? c ^ C[q - 1] : c;
+        }
+        __syncthreads();
+        for (uint32_t j = t; j < d; j += blockDim.x) {
+          uint32_t acc = 0;
+          for (uint32_t c = lognp; c < 32; ++c) sP[j * 33 + c - lognp] = acc ^= sC[j * 33 + c];
+        }
+        __syncthreads();
+      }
+      // word index of position i, dimension j: (rl n + i - i0) d + j, modulo 2^64 (the tile may
+      // start before i0)
+      const uint64_t first = ((uint64_t)rl * n - i0 + base) * d;
+      out = X + (int64_t)first;
+      phi = ((uint32_t)first + (uint32_t)((uintptr_t)X >> 2)) & 3u;
+      if (active) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const uint32_t e = 4 * t + k >= phi ? 4 * t + k - phi : words / 8 - phi + k;
+          const uint32_t p = e / d, j = e - p * d;
+          E[k] = e;
+          uint32_t f = 0, z = 0;
+          if constexpr (NET) {
+            const uint32_t *c = sC + j * 33;
+            for (uint32_t b = 0; b < lognp; ++b) f ^= (p >> b) & 1u ? c[b] : 0u;
+            for (uint32_t b = lognp; b < 32; ++b) z ^= (uint32_t)(base >> b) & 1u ? c[b] : 0u;
+            for (int b = 0; b < 3; ++b) A[b][k] = c[lognp - 3 + b];
+            z ^= D ? D[(size_t)r * d + j] : 0u;
+            J[k] = j;
+          } else {
+            const uint32_t gj = J[k] = g[j];
+            f = __brev(p) * gj;
+            for (int b = 0; b < 3; ++b) A[b][k] = __brev(1u << (lognp - 3 + b)) * gj;
+            z = __brev((uint32_t)base) * gj + (D ? D[(size_t)r * d + j] : 0u);
+          }
+          F[k] = f, T[k] = z;
+        }
+      }
+    } else if (active) {  // the next tile: bits 0 .. ctz(tile) of the tile index flip
+      const uint32_t c = __ffs((int)(uint32_t)tile) - 1;
+      const uint32_t db = __brev((uint32_t)base) - __brev((uint32_t)(base - NP));
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        if constexpr (NET) T[k] ^= sP[J[k] * 33 + c];
+        else T[k] += db * J[k];
+      }
+    }
+    if (active) {
+      const uint64_t lo = base > i0 ? base : i0, hi = base + NP < i0 + n ? base + NP : i0 + n;
+      const uint32_t elo = (uint32_t)(lo - base) * d, ehi = (uint32_t)(hi - base) * d;
+      const bool split = t == 0 && phi != 0;
+      uint32_t V[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) V[k] = gen_add<NET>(F[k], T[k]);
+      if (elo == 0 && ehi == words) {
+        // thread 0's words below phi belong to the region before: their values lag one group
+        uint32_t *dst = out + (int32_t)(4 * t - phi);
+        uint32_t prev[4] = {0, 0, 0, 0};
+#pragma unroll
+        for (int it = 0; it < 8; ++it) {
+          uint32_t v[4], o[4];
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            v[k] = V[k];
+#pragma unroll
+            for (int b = 0; b < 3; ++b)
+              if (it & (1 << b)) v[k] = gen_add<NET>(v[k], A[b][k]);
+            o[k] = split && (uint32_t)k < phi ? prev[k] : v[k];
+            prev[k] = v[k];
+          }
+          if (it == 0 && split) {
+#pragma unroll
+            for (int k = 1; k < 4; ++k)
+              if ((uint32_t)k >= phi) dst[k] = o[k];
+          } else {
+            *reinterpret_cast<uint4 *>(dst + 4 * NTA * it) = make_uint4(o[0], o[1], o[2], o[3]);
+          }
+        }
+        if (split) {
+#pragma unroll
+          for (int k = 0; k < 3; ++k)
+            if ((uint32_t)k < phi) out[words - phi + k] = prev[k];
         }
       } else {
-        for (uint32_t j = t; j < d; j += kGenNT) sC[j] = g[j];
-      }
-    }
-    const uint64_t base = ((i0 >> lognp) + tt) << lognp;  // < 2^32 (i0 + n <= 2^32)
-    if constexpr (NET) {
-      // the tile word of dimension j: one warp XOR-reduces the columns selected by the
-      // digits of h(base), lane k holding column k
-      const uint32_t hb = order_map(order, (uint32_t)base), lane = t & 31;
-      for (uint32_t j = t >> 5; j < d; j += kGenNT / 32) {
-        const uint32_t v = __reduce_xor_sync(0xffffffffu, ((hb >> lane) & 1u) ? sC[j * 32 + lane] : 0u);
-        if (lane == 0) ztile[j] = v ^ (D ? D[(size_t)r * d + j] : 0u);
-      }
-    } else {
-      for (uint32_t j = t; j < d; j += kGenNT) ztile[j] = D ? D[(size_t)r * d + j] : 0u;
-    }
-    // also separates the previous item's copy-out (reads of the tile) from this item's writes
-    __syncthreads();
-    // run (q, j): points q RL .. q RL + 7 of the tile in dimension j
-    const uint64_t lo = base > i0 ? base : i0, hi = (base + NP) < (i0 + n) ? (base + NP) : (i0 + n);
-    auto run = [&](uint32_t q, uint32_t j, uint32_t w) {
-      if (direct) {  // straight to the output rows, positions inside [i0, i0 + n) only
-        const uint64_t p0 = base + (uint64_t)q * kGenRL;
-        uint32_t *dst = X + ((uint64_t)rl * n) * d + j;
-        uint32_t xs[kGenRL];
-        if constexpr (NET) {
-          const uint32_t *cj = sC + j * 32;
-          const uint32_t c0 = cj[0], c1 = cj[1], c2 = cj[2];
-          const uint32_t s0 = c0, s1 = order == QK_GRAY ? c1 : (c0 ^ c1), s2 = order == QK_GRAY ? c2 : (c0 ^ c1 ^ c2);
-          xs[0] = ztile[j] ^ zrun[w];
-          xs[1] = xs[0] ^ s0, xs[2] = xs[1] ^ s1, xs[3] = xs[2] ^ s0, xs[4] = xs[3] ^ s2;
-          xs[5] = xs[4] ^ s0, xs[6] = xs[5] ^ s1, xs[7] = xs[6] ^ s0;
-        } else {
-          const uint32_t gj = sC[j], dj = ztile[j];
+        for (uint32_t it = 0; it < 8; ++it) {
 #pragma unroll
-          for (int k = 0; k < kGenRL; ++k) xs[k] = __brev((uint32_t)p0 + k) * gj + dj;
+          for (int k = 0; k < 4; ++k) {
+            const uint32_t q = split && (uint32_t)k < phi ? (it + 7) & 7 : it, e = E[k] + 4 * NTA * q;
+            uint32_t v = V[k];
+#pragma unroll
+            for (int b = 0; b < 3; ++b)
+              if (q & (1u << b)) v = gen_add<NET>(v, A[b][k]);
+            if (e >= elo && e < ehi) out[e] = v;
+          }
         }
-#pragma unroll
-        for (int k = 0; k < kGenRL; ++k)
-          if (p0 + k >= lo && p0 + k < hi) dst[(p0 + k - i0) * d] = xs[k];
-        return;
-      }
-      uint32_t *dst = tile + q * kGenRL * d + j;
-      if constexpr (NET) {
-        const uint32_t *cj = sC + j * 32;
-        const uint32_t c0 = cj[0], c1 = cj[1], c2 = cj[2];
-        // step k -> k + 1 flips digit ctz(k + 1) of the Gray index, digits 0 .. ctz(k + 1) of i
-        const uint32_t s0 = c0, s1 = order == QK_GRAY ? c1 : (c0 ^ c1), s2 = order == QK_GRAY ? c2 : (c0 ^ c1 ^ c2);
-        uint32_t x = ztile[j] ^ zrun[w];
-        dst[0] = x;
-        x ^= s0, dst[1 * d] = x;
-        x ^= s1, dst[2 * d] = x;
-        x ^= s0, dst[3 * d] = x;
-        x ^= s2, dst[4 * d] = x;
-        x ^= s0, dst[5 * d] = x;
-        x ^= s1, dst[6 * d] = x;
-        x ^= s0, dst[7 * d] = x;
-      } else {
-        const uint32_t gj = sC[j], dj = ztile[j];
-        const uint32_t i = (uint32_t)base + q * kGenRL;
-#pragma unroll
-        for (int k = 0; k < kGenRL; ++k) dst[k * d] = __brev(i + k) * gj + dj;
-      }
-    };
-    if (kGenNT % d == 0) {  // a thread keeps its dimension and steps through the runs
-      const uint32_t j = (uint32_t)t % d;
-      for (uint32_t q = (uint32_t)t / d; q < NP / kGenRL; q += kGenNT / d) run(q, j, q * d + j);
-    } else {
-      for (uint32_t w = t; w < runs; w += kGenNT) {
-        const uint32_t q = w / d;
-        run(q, w - q * d, w);
       }
     }
-    __syncthreads();
-    if (direct) continue;  // the barrier above also separates this item's run phase from the next
-    const uint64_t words = (hi - lo) * d, soff = (lo - base) * d;
-    const uint32_t *src = tile + soff;
-    uint32_t *out = X + ((uint64_t)rl * n + (lo - i0)) * d;
-    if ((((uintptr_t)out | (uintptr_t)src) & 15u) == 0 && (words & 3u) == 0) {  // 16-byte rows
-      const uint4 *s4 = reinterpret_cast<const uint4 *>(src);
-      uint4 *o4 = reinterpret_cast<uint4 *>(out);
-      for (uint64_t e = t; e < (words >> 2); e += kGenNT) o4[e] = s4[e];
-    } else {
-      for (uint64_t e = t; e < words; e += kGenNT) out[e] = src[e];
-    }
+    out += words;
+    fresh = ++tt == tiles;
+    if (fresh) tt = 0, ++rl;
   }
 }
 
 int launch_gen_points(const qk_pointset *ps, uint32_t r0, uint32_t nr, uint64_t i0, uint64_t n,
                       uint32_t *X, cudaStream_t st) {
   if (n == 0 || nr == 0) return QK_OK;
-  const uint32_t d = ps->d, lognp = gen_lognp(d), NP = 1u << lognp;
-  const uint64_t tiles = ((i0 + n - 1) >> lognp) - (i0 >> lognp) + 1;  // <= 2^29
-  const int direct = d >= 16;
-  const size_t smem = sizeof(uint32_t) * ((direct ? 0 : (size_t)NP * d) + 32 * d + (NP / kGenRL) * d + d);
+  const uint32_t d = ps->d, lognp = gen_lognp(d), threads = ((d << (lognp - 5)) + 31) & ~31u;
+  const uint64_t tiles = ((i0 + n - 1) >> lognp) - (i0 >> lognp) + 1;  // <= 2^27
+  const bool net = ps->kind == QK_NET_B2;
+  const size_t smem = net ? sizeof(uint32_t) * 66 * d : 0;
   int occ = 0;
-  if (ps->kind == QK_NET_B2) {
-    smem_optin<k_points_tiled<true>>(smem);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_points_tiled<true>, kGenNT, smem);
+  if (net) {
+    smem_optin<k_points<true>>(smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_points<true>, (int)threads, smem);
   } else {
-    smem_optin<k_points_tiled<false>>(smem);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_points_tiled<false>, kGenNT, smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_points<false>, (int)threads, smem);
   }
   if (occ < 1) occ = 1;
   // one wave of resident CTAs, each taking an equal contiguous chunk of the (r, tile) items
   const uint64_t total = (uint64_t)nr * tiles;
   uint64_t grid = (uint64_t)sm_count() * occ;
   if (grid > total) grid = total;
-  if (ps->kind == QK_NET_B2)
-    k_points_tiled<true><<<(unsigned)grid, kGenNT, smem, st>>>(d, ps->order, ps->Ct, nullptr, ps->D, r0, nr, i0, n,
-                                                               lognp, (uint32_t)tiles, direct, X);
+  if (net)
+    k_points<true><<<(unsigned)grid, threads, smem, st>>>(d, ps->order, ps->Ct, nullptr, ps->D, r0, nr, i0, n, lognp,
+                                                          (uint32_t)tiles, X);
   else
-    k_points_tiled<false><<<(unsigned)grid, kGenNT, smem, st>>>(d, ps->order, nullptr, ps->g, ps->D, r0, nr, i0, n,
-                                                                lognp, (uint32_t)tiles, direct, X);
+    k_points<false><<<(unsigned)grid, threads, smem, st>>>(d, ps->order, nullptr, ps->g, ps->D, r0, nr, i0, n, lognp,
+                                                           (uint32_t)tiles, X);
   return check_launch("qk_gen_points");
 }
 
