@@ -13,6 +13,7 @@
 #include "qk_common.cuh"
 #include "qk_factors.cuh"
 #include "qk_internal.h"
+#include "qk_quotient.cuh"
 
 namespace qk {
 
@@ -497,34 +498,6 @@ __device__ T dk_explicit(const ColJob &job, const DiffTables &tb, const T *wT, u
 }
 
 __device__ __forceinline__ float ratio(float a, float b) { return __fdividef(a, b); }  // 2 ulp
-// Approximate reciprocal (PTX rcp.approx.ftz.f32, max 1 ulp; subnormals flush to 0): 1/0 = inf.
-__device__ __forceinline__ float rcp_approx(float a) {
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
-  return r;
-}
-// a / b in FP64 without the FP64 divide (GB300 has about two FP64 lanes per SM and cycle):
-// from the FP32 reciprocal estimate r of b (its leading 24 bits, relative error e below
-// 2^-22), q0 = a r, then q0 (1 + e + e^2) with e = 1 - b r rounded once: what is left is e^3,
-// below 2^-66, so the result is within 2 ulp of the rounded quotient (checked against the
-// divide by qk_ratio_selftest).  Four FP64 instructions.  False for b outside
-// 2^-100 .. 2^100 in magnitude (zero, subnormal, inf and NaN included).
-__device__ __forceinline__ bool ratio_fast(double a, double b, double &q) {
-  const uint32_t hi = (uint32_t)__double2hiint(b), lo = (uint32_t)__double2loint(b);
-  const uint32_t ex = (hi >> 20) & 0x7FFu;
-  if (ex - 923u > 200u) return false;
-  const uint32_t fb = (hi & 0x80000000u) | ((ex - 896u) << 23) | ((hi & 0xFFFFFu) << 3) | (lo >> 29);
-  const double r = f2d_exact(rcp_approx(__uint_as_float(fb)));
-  const double e = fma(-b, r, 1.0);
-  const double q0 = a * r;
-  q = fma(q0, fma(e, e, e), q0);
-  return true;
-}
-__device__ __forceinline__ double ratio(double a, double b) {
-  double q;
-  return ratio_fast(a, b, q) ? q : a / b;
-}
-
 // Warp sums of four per-lane values, the pair (a0, a1) of one dimension and (b0, b1) of
 // the next, by a reduce-scatter: at the xor-16 step a lane keeps one dimension's pair and
 // sends the other's, at the xor-8 step it keeps one value of that pair, and the last three

@@ -16,7 +16,7 @@ QK_FUSED_PRECISIONS(QK_FUSED_EXTERN)
 // x <- H x * scale for vectors of n = 2^m with LOGT < m <= 2 LOGT - LOGL, in place, in two
 // tile passes: low LOGT bits on contiguous tiles, the high bits on column tiles.
 template <typename T>
-__global__ void __launch_bounds__(kFNT, 5) k_wht_low(T *__restrict__ x) {
+__global__ void __launch_bounds__(kFNT, sizeof(T) == 8 ? 3 : 5) k_wht_low(T *__restrict__ x) {
   constexpr int LOGT = FCfg<T>::LOGT, L = FCfg<T>::L;
   extern __shared__ __align__(16) unsigned char smem[];
   T *sm = reinterpret_cast<T *>(smem);
@@ -31,7 +31,7 @@ __global__ void __launch_bounds__(kFNT, 5) k_wht_low(T *__restrict__ x) {
 }
 
 template <typename T, int M>
-__global__ void __launch_bounds__(kFNT) k_wht_high(T *__restrict__ x, T scale) {
+__global__ void __launch_bounds__(kFNT, sizeof(T) == 8 ? 3 : 1) k_wht_high(T *__restrict__ x, T scale) {
   constexpr int LOGT = FCfg<T>::LOGT, L = FCfg<T>::L;
   extern __shared__ __align__(16) unsigned char smem[];
   T *sm = reinterpret_cast<T *>(smem);
@@ -56,7 +56,7 @@ __global__ void __launch_bounds__(kFNT) k_wht_high(T *__restrict__ x, T scale) {
 // vector's column tiles `lag` vectors later.  Past the wait limit a column tile is skipped
 // and QK_STATUS_TIMEOUT is raised.
 template <typename T, int M>
-__global__ void __launch_bounds__(kFNT, 5) k_wht_persist(T *__restrict__ x, T scale, WhtSched sc,
+__global__ void __launch_bounds__(kFNT, sizeof(T) == 8 ? 3 : 5) k_wht_persist(T *__restrict__ x, T scale, WhtSched sc,
                                                          uint32_t *__restrict__ ctr, uint32_t *status,
                                                          uint32_t spin_limit, uint32_t first_item) {
   constexpr int LOGT = FCfg<T>::LOGT, L = FCfg<T>::L, m = M, c = 2 * LOGT - M;
@@ -117,6 +117,28 @@ __global__ void __launch_bounds__(kFNT, 5) k_wht_persist(T *__restrict__ x, T sc
   }
 }
 
+// One pass of the generic multi-pass FP64 transform (sizes beyond two passes): a tile of 2^c
+// contiguous elements times 2^(12 - c) rows, 2^s apart, s = 0 with c = 0 for the first pass.
+__global__ void __launch_bounds__(kFNT, 3) k_wht64_pass(double *__restrict__ x, int m, int s, int c, double scale) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int t = threadIdx.x, other = m - 12, lo = s - c;  // tiles per vector 2^other
+  const uint64_t v = blockIdx.x >> other, tau = blockIdx.x & ((1u << other) - 1);
+  const uint64_t base = (v << m) + ((tau >> lo) << (s + 12 - c)) + ((tau & ((1ull << lo) - 1)) << c);
+  auto at = [&](int e) -> uint64_t { return base + ((uint64_t)(e >> c) << s) + (uint64_t)(e & ((1 << c) - 1)); };
+  double r[16];
+#pragma unroll
+  for (int l = 0; l < 16; ++l) r[l] = x[at(e_of<double>(0, t, l))];
+  xwht64(r, reinterpret_cast<double *>(smem), c, 0);
+#pragma unroll
+  for (int l = 0; l < 16; ++l) x[at(e_of<double>(2, t, l))] = r[l] * scale;
+}
+
+int wht64_pass(double *x, int m, int s, int c, uint64_t blocks, double scale, cudaStream_t st) {
+  smem_optin<k_wht64_pass>(xtile_bytes<double>());
+  k_wht64_pass<<<(unsigned)blocks, kFNT, xtile_bytes<double>(), st>>>(x, m, s, c, scale);
+  return check_launch("transform pass (FP64 integers)");
+}
+
 size_t persist_wht_ws_bytes(uint64_t nvec) { return align256(sizeof(uint32_t) * (1 + nvec)); }
 
 // Every m of the two-pass range gets its own instantiation: with the tile split known at
@@ -129,6 +151,9 @@ template <typename T> struct WhtKernels {
 };
 template <typename T, int M>
 static WhtKernels<T> wht_kernels_m() {
+  smem_optin<k_wht_low<T>>(xtile_bytes<T>());
+  smem_optin<k_wht_high<T, M>>(xtile_bytes<T>());
+  smem_optin<k_wht_persist<T, M>>(xtile_bytes<T>());
   return WhtKernels<T>{k_wht_low<T>, k_wht_high<T, M>, k_wht_persist<T, M>};
 }
 template <typename T, int... I>

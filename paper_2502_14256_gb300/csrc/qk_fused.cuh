@@ -38,6 +38,7 @@
 #include "qk_factors.cuh"
 #include "qk_grad.cuh"
 #include "qk_internal.h"
+#include "qk_wht96.cuh"
 
 namespace qk {
 
@@ -65,72 +66,6 @@ struct FTask {
   uint32_t *status;
 };
 
-template <typename T>
-__device__ __forceinline__ int fpad(int e) { return e + (e >> FCfg<T>::PAD); }
-
-template <typename T>
-__host__ __device__ constexpr size_t tile_smem_bytes() {
-  return (size_t)((1 << FCfg<T>::LOGT) + ((1 << FCfg<T>::LOGT) >> FCfg<T>::PAD)) * sizeof(T);
-}
-
-// Radix-2^R WHT round on tile bits [b, b+R) held in shared memory.
-template <typename T, int R>
-__device__ __forceinline__ void smem_round(T *sm, int b) {
-  constexpr int G = (1 << FCfg<T>::LOGT) >> R;
-  for (int g = threadIdx.x; g < G; g += kFNT) {
-    const int e0 = (g & ((1 << b) - 1)) | ((g >> b) << (b + R));
-    T v[1 << R];
-#pragma unroll
-    for (int q = 0; q < (1 << R); ++q) v[q] = sm[fpad<T>(e0 | (q << b))];
-#pragma unroll
-    for (int h = 0; h < R; ++h)
-#pragma unroll
-      for (int q = 0; q < (1 << R); ++q)
-        if (!(q & (1 << h))) {
-          const T a = v[q], bb = v[q | (1 << h)];
-          v[q] = a + bb;
-          v[q | (1 << h)] = a - bb;
-        }
-#pragma unroll
-    for (int q = 0; q < (1 << R); ++q) sm[fpad<T>(e0 | (q << b))] = v[q];
-  }
-}
-
-// WHT butterflies over tile bits [c, LOGT) of the tile held as v[l] at e = tid + 256 l;
-// the result is returned in v with the same mapping.  sm: the padded tile scratch.
-template <typename T>
-__device__ __forceinline__ void tile_wht(T (&v)[FCfg<T>::L], T *sm, int c) {
-  constexpr int L = FCfg<T>::L, LOGL = FCfg<T>::LOGL;
-#pragma unroll
-  for (int h = 0; h < LOGL; ++h) {
-    if (kLOGNT + h >= c) {
-#pragma unroll
-      for (int q = 0; q < L; ++q)
-        if (!(q & (1 << h))) {
-          const T a = v[q], b = v[q | (1 << h)];
-          v[q] = a + b;
-          v[q | (1 << h)] = a - b;
-        }
-    }
-  }
-  if (c < kLOGNT) {
-#pragma unroll
-    for (int l = 0; l < L; ++l) sm[fpad<T>(threadIdx.x + (l << kLOGNT))] = v[l];
-    __syncthreads();
-    for (int b = c; b < kLOGNT; b += 4) {
-      const int r = (kLOGNT - b) < 4 ? (kLOGNT - b) : 4;
-      if (r == 4) smem_round<T, 4>(sm, b);
-      else if (r == 3) smem_round<T, 3>(sm, b);
-      else if (r == 2) smem_round<T, 2>(sm, b);
-      else smem_round<T, 1>(sm, b);
-      __syncthreads();
-    }
-#pragma unroll
-    for (int l = 0; l < L; ++l) v[l] = sm[fpad<T>(threadIdx.x + (l << kLOGNT))];
-    __syncthreads();
-  }
-}
-
 // s + e tracks a sum exactly up to the rounding of e: the error of each addition to s
 // (TwoSum) is accumulated in e.  (Kahan's single correction term is not enough here: its
 // s - c keeps an error of ~u sum|v| per partial, and Sum y of a centred integrand is a
@@ -154,66 +89,6 @@ __device__ __forceinline__ void cbfly(T &ah, T &al, T &bh, T &bl) {
   ah = s, al = sl, bh = d, bl = dl;
 }
 
-template <typename T, int R>
-__device__ __forceinline__ void smem_round2(T *sh, T *sl, int b) {
-  constexpr int G = (1 << FCfg<T>::LOGT) >> R;
-  for (int g = threadIdx.x; g < G; g += kFNT) {
-    const int e0 = (g & ((1 << b) - 1)) | ((g >> b) << (b + R));
-    T vh[1 << R], vl[1 << R];
-#pragma unroll
-    for (int q = 0; q < (1 << R); ++q) {
-      vh[q] = sh[fpad<T>(e0 | (q << b))];
-      vl[q] = sl[fpad<T>(e0 | (q << b))];
-    }
-#pragma unroll
-    for (int h = 0; h < R; ++h)
-#pragma unroll
-      for (int q = 0; q < (1 << R); ++q)
-        if (!(q & (1 << h))) cbfly(vh[q], vl[q], vh[q | (1 << h)], vl[q | (1 << h)]);
-#pragma unroll
-    for (int q = 0; q < (1 << R); ++q) {
-      sh[fpad<T>(e0 | (q << b))] = vh[q];
-      sl[fpad<T>(e0 | (q << b))] = vl[q];
-    }
-  }
-}
-
-// tile_wht on compensated pairs (hi, lo); shl: a second padded tile for the lo parts.
-template <typename T>
-__device__ __forceinline__ void tile_wht2(T (&vh)[FCfg<T>::L], T (&vl)[FCfg<T>::L], T *sh, T *shl, int c) {
-  constexpr int L = FCfg<T>::L, LOGL = FCfg<T>::LOGL;
-#pragma unroll
-  for (int h = 0; h < LOGL; ++h) {
-    if (kLOGNT + h >= c) {
-#pragma unroll
-      for (int q = 0; q < L; ++q)
-        if (!(q & (1 << h))) cbfly(vh[q], vl[q], vh[q | (1 << h)], vl[q | (1 << h)]);
-    }
-  }
-  if (c < kLOGNT) {
-#pragma unroll
-    for (int l = 0; l < L; ++l) {
-      sh[fpad<T>(threadIdx.x + (l << kLOGNT))] = vh[l];
-      shl[fpad<T>(threadIdx.x + (l << kLOGNT))] = vl[l];
-    }
-    __syncthreads();
-    for (int b = c; b < kLOGNT; b += 4) {
-      const int r = (kLOGNT - b) < 4 ? (kLOGNT - b) : 4;
-      if (r == 4) smem_round2<T, 4>(sh, shl, b);
-      else if (r == 3) smem_round2<T, 3>(sh, shl, b);
-      else if (r == 2) smem_round2<T, 2>(sh, shl, b);
-      else smem_round2<T, 1>(sh, shl, b);
-      __syncthreads();
-    }
-#pragma unroll
-    for (int l = 0; l < L; ++l) {
-      vh[l] = sh[fpad<T>(threadIdx.x + (l << kLOGNT))];
-      vl[l] = shl[fpad<T>(threadIdx.x + (l << kLOGNT))];
-    }
-    __syncthreads();
-  }
-}
-
 // ---------------------------------------------------------- register-tiled WHT
 // Three thread layouts of a 2^LOGT-element tile (L = 2^LOGL elements per thread,
 // 256 threads):
@@ -229,9 +104,13 @@ template <typename T> struct Lay {
   static constexpr int PADE = 16 / sizeof(T);  // 4 words per row of L elements
   static constexpr int VEC = 16 / sizeof(T);   // elements per 128-bit access
 };
+// FP32: the padded tile.  FP64: three planes of 32-bit words (the 96-bit butterflies below,
+// kW96Plane words each) and 8 words of scratch; the FP64 tile of the fallback fits in them.
+constexpr int kW96Plane = 4096 + 4 * (4096 / 32) + 16 * (4096 / 256);
 template <typename T>
 __host__ __device__ constexpr size_t xtile_bytes() {
-  return (size_t)((1 << FCfg<T>::LOGT) + Lay<T>::PADE * ((1 << FCfg<T>::LOGT) >> FCfg<T>::LOGL)) * sizeof(T);
+  return sizeof(T) == 8 ? (size_t)(3 * kW96Plane + 8) * sizeof(uint32_t)
+                        : (size_t)((1 << FCfg<T>::LOGT) + Lay<T>::PADE * ((1 << FCfg<T>::LOGT) >> FCfg<T>::LOGL)) * sizeof(T);
 }
 template <typename T>
 __device__ __forceinline__ int xpad(int e) { return e + Lay<T>::PADE * (e >> Lay<T>::LOGL); }
@@ -382,9 +261,125 @@ __device__ __forceinline__ void xw_L1w_to_L0(float (&v)[32], float *sm) {
   __syncthreads();
 }
 
+// ------------------------------------------------ FP64 tiles in 96-bit integers (qk_wht96.cuh)
+// The layouts are those above; element e sits at word e + 4 (e >> 5) + 16 (e >> 8) of its plane:
+// conflict-free for L0 (32 consecutive elements per warp), L1 (128-bit accesses, rows of 16
+// words) and L2 (two runs of 16 elements, 256 apart).
+__device__ __forceinline__ int w96_index(int e) { return e + 4 * (e >> 5) + 16 * (e >> 8); }
+
+template <int LAYOUT>
+__device__ __forceinline__ int w96_at(int l) {  // word of the thread's element l of a layout (L1: of its 4 l)
+  const int t = threadIdx.x;
+  if (LAYOUT == 0) return w96_index(t) + l * (256 + 32 + 16);
+  if (LAYOUT == 1) return w96_index(16 * t) + 4 * l;
+  // bits 4 and 5.. of e: 16 l moves within the run of 256, no carry into bit 8
+  return w96_index((t & 15) + ((t >> 4) << 8)) + 16 * l + 4 * (l >> 1);
+}
+
+template <int FROM, int TO>
+__device__ __forceinline__ void w96_xpose(I96 (&x)[16], uint32_t *sm) {
+  uint32_t *p0 = sm, *p1 = sm + kW96Plane, *p2 = sm + 2 * kW96Plane;
+  if constexpr (FROM == 1) {
+#pragma unroll
+    for (int l = 0; l < 4; ++l) {
+      const int w = w96_at<1>(l);
+      *reinterpret_cast<uint4 *>(p0 + w) = make_uint4(x[4 * l].a, x[4 * l + 1].a, x[4 * l + 2].a, x[4 * l + 3].a);
+      *reinterpret_cast<uint4 *>(p1 + w) = make_uint4(x[4 * l].b, x[4 * l + 1].b, x[4 * l + 2].b, x[4 * l + 3].b);
+      *reinterpret_cast<uint4 *>(p2 + w) = make_uint4(x[4 * l].c, x[4 * l + 1].c, x[4 * l + 2].c, x[4 * l + 3].c);
+    }
+  } else {
+#pragma unroll
+    for (int l = 0; l < 16; ++l) {
+      const int w = w96_at<FROM>(l);
+      p0[w] = x[l].a, p1[w] = x[l].b, p2[w] = x[l].c;
+    }
+  }
+  __syncthreads();
+  if constexpr (TO == 1) {
+#pragma unroll
+    for (int l = 0; l < 4; ++l) {
+      const int w = w96_at<1>(l);
+      const uint4 a = *reinterpret_cast<const uint4 *>(p0 + w), b = *reinterpret_cast<const uint4 *>(p1 + w),
+                  c = *reinterpret_cast<const uint4 *>(p2 + w);
+      x[4 * l] = {a.x, b.x, c.x}, x[4 * l + 1] = {a.y, b.y, c.y};
+      x[4 * l + 2] = {a.z, b.z, c.z}, x[4 * l + 3] = {a.w, b.w, c.w};
+    }
+  } else {
+#pragma unroll
+    for (int l = 0; l < 16; ++l) {
+      const int w = w96_at<TO>(l);
+      x[l].a = p0[w], x[l].b = p1[w], x[l].c = p2[w];
+    }
+  }
+  __syncthreads();
+}
+
+// Butterflies on the register bits h whose tile bit (bit0 + h) lies in [lo, hi).
+__device__ __forceinline__ void w96_stages(I96 (&x)[16], int bit0, int lo, int hi) {
+#pragma unroll
+  for (int h = 0; h < 4; ++h)
+    if (bit0 + h >= lo && bit0 + h < hi) {
+#pragma unroll
+      for (int q = 0; q < 16; ++q)
+        if (!(q & (1 << h))) {
+          const I96 a = x[q], b = x[q | (1 << h)];
+          x[q] = i96_add(a, b), x[q | (1 << h)] = i96_sub(a, b);
+        }
+    }
+}
+
+// Tile values into integers over the tile's largest exponent E; false: take the FP64 path.
+// Every thread of the CTA calls it (one barrier).
+__device__ __forceinline__ bool w96_load(const double (&v)[16], I96 (&x)[16], uint32_t *sm, uint32_t &E) {
+  uint32_t hm = 0;
+#pragma unroll
+  for (int l = 0; l < 16; ++l) {
+    const uint32_t h = (uint32_t)__double2hiint(v[l]) & 0x7FFFFFFFu;
+    hm = h > hm ? h : hm;
+  }
+  E = block_max_exp(hm, sm + 3 * kW96Plane);
+  if (E < kW96MinExp || E > kW96MaxExp) return false;
+#pragma unroll
+  for (int l = 0; l < 16; ++l) x[l] = i96_from(v[l], E);
+  return true;
+}
+
+// The tile's sum, in integers and rounded once (FP64 compensated sums outside their exponent
+// range); valid in thread 0.  sm: the transform tile.
+__device__ __forceinline__ double w96_sum(const double (&v)[16], uint32_t *sm) {
+  I96 x[16];
+  uint32_t E;
+  if (!w96_load(v, x, sm, E)) {
+    double s = 0.0, e = 0.0;
+#pragma unroll
+    for (int l = 0; l < 16; ++l) ff_add(s, e, v[l]);
+    const double r = block_sum_c(s, e, reinterpret_cast<double *>(sm));
+    __syncthreads();
+    return r;
+  }
+#pragma unroll
+  for (int l = 1; l < 16; ++l) x[0] = i96_add(x[0], x[l]);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+    x[0] = i96_add(x[0], I96{__shfl_xor_sync(0xffffffffu, x[0].a, o), __shfl_xor_sync(0xffffffffu, x[0].b, o),
+                             __shfl_xor_sync(0xffffffffu, x[0].c, o)});
+  if ((threadIdx.x & 31) == 0) {
+    uint32_t *p = sm + 3 * (threadIdx.x >> 5);
+    p[0] = x[0].a, p[1] = x[0].b, p[2] = x[0].c;
+  }
+  __syncthreads();
+  double r = 0.0;
+  if (threadIdx.x == 0) {
+    for (int q = 1; q < kFNT / 32; ++q) x[0] = i96_add(x[0], I96{sm[3 * q], sm[3 * q + 1], sm[3 * q + 2]});
+    r = i96_to(x[0], E);
+  }
+  __syncthreads();
+  return r;
+}
+
 // Full tile WHT (bits [0, LOGT)): from L0 to L2 (dir 0) or from L2 to L0 (dir 1).
 template <typename T>
-__device__ __forceinline__ void xwht_full(T (&v)[FCfg<T>::L], T *sm, int dir) {
+__device__ __forceinline__ void xwht_full_fp(T (&v)[FCfg<T>::L], T *sm, int dir) {
   constexpr int LOGL = Lay<T>::LOGL, LOGT = Lay<T>::LOGT;
   if constexpr (sizeof(T) == 4) {  // warp-major tile: the same butterflies in the same order
     if (dir == 0) {
@@ -419,7 +414,7 @@ __device__ __forceinline__ void xwht_full(T (&v)[FCfg<T>::L], T *sm, int dir) {
 
 // Column-tile WHT on bits [c, LOGT), c >= LOGL: from L0 to L2 (dir 0) or L2 to L0 (dir 1).
 template <typename T>
-__device__ __forceinline__ void xwht_col(T (&v)[FCfg<T>::L], T *sm, int c, int dir) {
+__device__ __forceinline__ void xwht_col_fp(T (&v)[FCfg<T>::L], T *sm, int c, int dir) {
   constexpr int LOGL = Lay<T>::LOGL, LOGT = Lay<T>::LOGT;
   if (dir == 0) {
     reg_stages<T>(v, 8, c, LOGT);
@@ -430,6 +425,69 @@ __device__ __forceinline__ void xwht_col(T (&v)[FCfg<T>::L], T *sm, int c, int d
     xpose<T>(v, sm, 2, 0);
     reg_stages<T>(v, 8, c, LOGT);
   }
+}
+
+// The FP64 butterflies of a tile outside the integer path's exponent range (out of line: rare).
+static __device__ __noinline__ void xwht64_rare(double *v, double *sm, int c, int dir) {
+  double x[16];
+#pragma unroll
+  for (int l = 0; l < 16; ++l) x[l] = v[l];
+  if (c == 0) xwht_full_fp<double>(x, sm, dir);
+  else xwht_col_fp<double>(x, sm, c, dir);
+#pragma unroll
+  for (int l = 0; l < 16; ++l) v[l] = x[l];
+}
+
+// Full tile WHT (bits [0, LOGT)) from L0 to L2 (dir 0) or from L2 to L0 (dir 1), and
+// column-tile WHT (bits [c, LOGT)); FP64 tiles in 96-bit integers.
+__device__ __forceinline__ void xwht64(double (&v)[16], double *smd, int c, int dir) {
+  uint32_t *sm = reinterpret_cast<uint32_t *>(smd);
+  I96 x[16];
+  uint32_t E;
+  if (!w96_load(v, x, sm, E)) {
+    double tmp[16];
+#pragma unroll
+    for (int l = 0; l < 16; ++l) tmp[l] = v[l];
+    xwht64_rare(tmp, smd, c, dir);
+#pragma unroll
+    for (int l = 0; l < 16; ++l) v[l] = tmp[l];
+    return;
+  }
+  if (c == 0) {
+    if (dir == 0) {
+      w96_stages(x, 8, 8, 12);
+      w96_xpose<0, 1>(x, sm);
+      w96_stages(x, 0, 0, 4);
+      w96_xpose<1, 2>(x, sm);
+      w96_stages(x, 4, 4, 8);
+    } else {
+      w96_stages(x, 4, 4, 8);
+      w96_xpose<2, 1>(x, sm);
+      w96_stages(x, 0, 0, 4);
+      w96_xpose<1, 0>(x, sm);
+      w96_stages(x, 8, 8, 12);
+    }
+  } else if (dir == 0) {
+    w96_stages(x, 8, c, 12);
+    w96_xpose<0, 2>(x, sm);
+    w96_stages(x, 4, c, 8);
+  } else {
+    w96_stages(x, 4, c, 8);
+    w96_xpose<2, 0>(x, sm);
+    w96_stages(x, 8, c, 12);
+  }
+#pragma unroll
+  for (int l = 0; l < 16; ++l) v[l] = i96_to(x[l], E);
+}
+template <typename T>
+__device__ __forceinline__ void xwht_full(T (&v)[FCfg<T>::L], T *sm, int dir) {
+  if constexpr (sizeof(T) == 8) xwht64(v, sm, 0, dir);
+  else xwht_full_fp<T>(v, sm, dir);
+}
+template <typename T>
+__device__ __forceinline__ void xwht_col(T (&v)[FCfg<T>::L], T *sm, int c, int dir) {
+  if constexpr (sizeof(T) == 8) xwht64(v, sm, c, dir);
+  else xwht_col_fp<T>(v, sm, c, dir);
 }
 
 // Packed FP32 pairs (sm_100+ f32x2 adds): the same roundings as the scalar operations.
@@ -551,16 +609,38 @@ __device__ __forceinline__ void xwht_col2(T (&vh)[FCfg<T>::L], T (&vl)[FCfg<T>::
 
 // log lambda for the log-determinant: FP32 tiles take the hardware log2 approximation
 // (absolute error ~2^-22 per term, about 1e-8 relative on a log det summed over 2^20
-// eigenvalues even if every term erred the same way; the sum itself is FP64), FP64 tiles
-// the full-precision log.  1 / lambda likewise: the FP32 tiles' reciprocal estimate plus one
-// Newton step (within 1 ulp); the solve's exact-residual correction below absorbs it.
-__device__ __forceinline__ float fused_log(float v) { return __logf(v); }
-__device__ __forceinline__ double fused_log(double v) { return log(v); }
+// eigenvalues even if every term erred the same way; the sum itself is FP64).  1 / lambda: the
+// reciprocal estimate plus one Newton step (within 1 ulp); the solve's exact-residual
+// correction below absorbs it.
 __device__ __forceinline__ float fused_rcp(float v) {
   const float r = rcp_approx(v);
   return fmaf(fmaf(-v, r, 1.f), r, r);
 }
-__device__ __forceinline__ double fused_rcp(double v) { return 1.0 / v; }
+__device__ __forceinline__ double fused_rcp(double v) { return rcp64(v); }
+// Sum of logs of a thread's eigenvalues.  FP64: the log of the product of the mantissas (16
+// factors below 2) and the sum of the exponents: one multiplication per eigenvalue and one log
+// per thread, where a log is some 30 FP64 instructions; eigenvalues that are not positive normal
+// numbers add their own log.
+template <typename T> struct LogSum;
+template <> struct LogSum<float> {
+  float s = 0.f;
+  __device__ __forceinline__ void add(float v) { s += __logf(v); }
+  __device__ __forceinline__ float total() const { return s; }
+};
+template <> struct LogSum<double> {
+  double prod = 1.0, s = 0.0;
+  int ex = 0;
+  __device__ __forceinline__ void add(double v) {
+    const uint32_t hi = (uint32_t)__double2hiint(v);
+    if (hi - 0x100000u >= 0x7FE00000u) {
+      s += log(v);
+      return;
+    }
+    ex += (int)(hi >> 20) - 1023;
+    prod *= __hiloint2double((int)((hi & 0xFFFFFu) | 0x3FF00000u), __double2loint(v));
+  }
+  __device__ __forceinline__ double total() const { return s + fma((double)ex, 0.69314718055994530942, log(prod)); }
+};
 
 // ------------------------------------------------------------------ phase A
 template <typename T, int FAM, int ALPHA, bool COMP, bool WIDE>
@@ -610,15 +690,23 @@ __device__ __forceinline__ void fused_A_item(const FTask &ft, uint32_t r, uint32
       PTL[e_of<T>(2, t, l)] = pl[l];
     }
   } else {
-    T ps = T(0), pe = T(0);  // compensated thread partial: the sum cancels
+    if constexpr (sizeof(T) == 8) {
 #pragma unroll
-    for (int l = 0; l < L; ++l) {
-      P[t + (l << kLOGNT)] = p[l];  // phase C's k_1 needs p to FP32 precision only
-      ff_add(ps, pe, p[l]);
+      for (int l = 0; l < L; ++l) P[t + (l << kLOGNT)] = p[l];
+      const double sps = w96_sum(p, reinterpret_cast<uint32_t *>(sm));
+      if (t == 0) ft.sp[(uint64_t)r * ft.tiles + tile] = sps;
+      xwht_full_fp<T>(p, sm, 0);  // L0 -> L2, FP64 butterflies (the eigenvalues' rounding)
+    } else {
+      T ps = T(0), pe = T(0);  // compensated thread partial: the sum cancels
+#pragma unroll
+      for (int l = 0; l < L; ++l) {
+        P[t + (l << kLOGNT)] = p[l];  // phase C's k_1 needs p to FP32 precision only
+        ff_add(ps, pe, p[l]);
+      }
+      const double sps = block_sum_c(ps, pe, red);
+      if (t == 0) ft.sp[(uint64_t)r * ft.tiles + tile] = sps;
+      xwht_full<T>(p, sm, 0);  // L0 -> L2
     }
-    const double sps = block_sum_c(ps, pe, red);
-    if (t == 0) ft.sp[(uint64_t)r * ft.tiles + tile] = sps;
-    xwht_full<T>(p, sm, 0);  // L0 -> L2
 #pragma unroll
     for (int l = 0; l < L; ++l) PT[e_of<T>(2, t, l)] = p[l];
   }
@@ -628,7 +716,7 @@ __device__ __forceinline__ void fused_A_item(const FTask &ft, uint32_t r, uint32
     T yv[L];
 #pragma unroll
     for (int l = 0; l < L; ++l) yv[l] = Y[t + (l << kLOGNT)];
-    if constexpr (!COMP) {
+    if constexpr (!COMP && sizeof(T) == 4) {
       T ys = T(0), ye = T(0);
 #pragma unroll
       for (int l = 0; l < L; ++l) ff_add(ys, ye, yv[l]);
@@ -651,6 +739,7 @@ __device__ __forceinline__ void fused_A_item(const FTask &ft, uint32_t r, uint32
       }
     } else {
       xwht_full<T>(yv, sm, 0);
+      if (sizeof(T) == 8 && t == 0) ft.sy[v * ft.tiles + tile] = yv[0];  // element 0: the sum rounded once
 #pragma unroll
       for (int l = 0; l < L; ++l) YT[e_of<T>(2, t, l)] = yv[l];
     }
@@ -658,20 +747,27 @@ __device__ __forceinline__ void fused_A_item(const FTask &ft, uint32_t r, uint32
 }
 
 template <typename T, int FAM, int ALPHA, bool COMP, bool WIDE>
-__global__ void __launch_bounds__(kFNT, WIDE ? 1 : 3) k_fused_A(FTask ft) {
+__global__ void __launch_bounds__(kFNT, WIDE ? 1 : (sizeof(T) == 8 ? 2 : 3)) k_fused_A(FTask ft) {
   extern __shared__ __align__(16) unsigned char smem[];
   fused_A_item<T, FAM, ALPHA, COMP, WIDE>(ft, blockIdx.y, blockIdx.x, smem);
 }
 
 // ------------------------------------------------------------------ phase B
+// Shared bytes: the transform tile, lambda, (FP32) g / the lo tile, reduction scratch.  FP64
+// keeps g in registers, so that two CTAs fit an SM.
+template <typename T>
+__host__ __device__ constexpr size_t fused_B_smem() {
+  return (sizeof(T) == 8 ? xtile_bytes<T>() + (sizeof(T) << FCfg<T>::LOGT) : 3 * xtile_bytes<T>()) + 32 * sizeof(double);
+}
+
 template <typename T, bool COMP, bool WIDE>
 __device__ __forceinline__ void fused_B_item(const FTask &ft, uint32_t r, uint32_t tau, unsigned char *smem,
                                              uint32_t *status) {
   constexpr int LOGT = FCfg<T>::LOGT, L = FCfg<T>::L;
   T *sm = reinterpret_cast<T *>(smem);
-  T *lmv = reinterpret_cast<T *>(smem + xtile_bytes<T>());      // lambda (own entries)
-  T *gst = reinterpret_cast<T *>(smem + 2 * xtile_bytes<T>());  // g (own entries) / lo tile
-  double *red = reinterpret_cast<double *>(smem + 3 * xtile_bytes<T>());
+  T *lmv = reinterpret_cast<T *>(smem + xtile_bytes<T>());      // lambda, FP64: 1 / lambda (own entries)
+  T *gst = reinterpret_cast<T *>(smem + 2 * xtile_bytes<T>());  // FP32: g (own entries) / lo tile
+  double *red = reinterpret_cast<double *>(smem + fused_B_smem<T>()) - 32;
   const int c = ft.cB, t = threadIdx.x;
   const uint64_t n = 1ull << ft.job.m;
   // element (t, l) of the tile is w = (row << LOGT) | (tau << c) | col, e = t + 256 l
@@ -694,11 +790,11 @@ __device__ __forceinline__ void fused_B_item(const FTask &ft, uint32_t r, uint32
     for (int l = 0; l < L; ++l) laml[l] = __ldcg(&PTL[wi0(l)]);
     xwht_col2<T>(lam, laml, sm, gst, c, 0);  // L0 -> L2, compensated (gst: the lo tile)
   } else {
-    xwht_col<T>(lam, sm, c, 0);  // L0 -> L2
+    xwht_col_fp<T>(lam, sm, c, 0);  // L0 -> L2
   }
   const T zeta = (T)ft.job.zeta, eta = (T)ft.eta, zn = (T)(ft.job.zeta * (double)n);
   bool bad = false;
-  T lds = T(0);
+  LogSum<T> lds;
   double *LAM = ft.lam ? ft.lam + (uint64_t)r * n : nullptr;
   bool floored = false;
 #pragma unroll
@@ -730,12 +826,13 @@ __device__ __forceinline__ void fused_B_item(const FTask &ft, uint32_t r, uint32
       if (LAM) LAM[wi2(l)] = f2d_exact(v);
     }
     bad |= !(v > T(0));
-    lds += fused_log(v);
-    lmv[t + (l << kLOGNT)] = v;  // each thread reads back only its own entries
+    lds.add(v);
+    // each thread reads back only its own entries; FP64 (no refinement) needs 1 / lambda alone
+    lmv[t + (l << kLOGNT)] = sizeof(T) == 8 ? fused_rcp(v) : v;
   }
   if (bad && status) atomicOr(status, (uint32_t)QK_STATUS_NOTPD);
   if (floored && status) atomicOr(status, (uint32_t)QK_STATUS_FLOOR);
-  const double ldsum = block_sum_c(lds, T(0), red);
+  const double ldsum = block_sum_c(lds.total(), T(0), red);
   if (t == 0) ft.ld[(uint64_t)r * ft.tiles + tau] = ldsum;
   const T inv_n = T(1) / (T)n;
   for (uint32_t q = 0; q < ft.nrhs; ++q) {
@@ -755,11 +852,12 @@ __device__ __forceinline__ void fused_B_item(const FTask &ft, uint32_t r, uint32
       xwht_col<T>(y, sm, c, 0);
     }
     T quad = T(0), gs = T(0);
+    T greg[sizeof(T) == 8 ? L : 1];
 #pragma unroll
     for (int l = 0; l < L; ++l) {
       const int e = t + (l << kLOGNT);  // this thread's own entries only
       const T lw = lmv[e];
-      const T il = fused_rcp(lw);
+      const T il = sizeof(T) == 8 ? lw : fused_rcp(lw);
       const T sc = inv_n * il;          // 1 / (n lambda_w)
       T ch = y[l] * sc;                 // c^_w = Y_w / (n lambda_w)
       const T a = ch * y[l];            // Y_w^2 / (n lambda_w)
@@ -776,7 +874,8 @@ __device__ __forceinline__ void fused_B_item(const FTask &ft, uint32_t r, uint32
         ch = fmadd(rho + ylo[l], sc, ch);
       }
       y[l] = ch;
-      gst[e] = gg;
+      if constexpr (sizeof(T) == 8) greg[l] = gg;
+      else gst[e] = gg;
     }
     // inverse high bits of c^, then of g: one copy of the transform's code for both (the
     // kernel's time goes to instruction fetch more than to arithmetic)
@@ -784,7 +883,10 @@ __device__ __forceinline__ void fused_B_item(const FTask &ft, uint32_t r, uint32
     for (int k = 0; k < 2; ++k) {
       if (k) {
 #pragma unroll
-        for (int l = 0; l < L; ++l) y[l] = gst[t + (l << kLOGNT)];
+        for (int l = 0; l < L; ++l) {
+          if constexpr (sizeof(T) == 8) y[l] = greg[l];
+          else y[l] = gst[t + (l << kLOGNT)];
+        }
       }
       xwht_col<T>(y, sm, c, 1);  // L2 -> L0
       T *dst = k ? GT : YT;
@@ -923,32 +1025,40 @@ static __global__ void __launch_bounds__(kFNT, 2) k_fused_C64(FTask ft) {
 }
 
 // ------------------------------------------------------------------ final
-__device__ __forceinline__ void fused_final_item(const FTask &ft, uint32_t v) {
-  __shared__ double sh[32];
+// The partial sums of vector v added up: its MLL outputs (`scalars`) and entries j0 .. j1 - 1 of
+// its 2 d gradient sums, a warp per entry (each sum in the same order whichever CTA forms it).
+__device__ __forceinline__ void fused_final_item(const FTask &ft, uint32_t v, uint32_t j0, uint32_t j1, bool scalars) {
+  __shared__ double sh[5][8];
+  __shared__ double res[5];
   const uint32_t r = v / ft.nrhs;
   const uint32_t tiles = ft.tiles, d = ft.job.d;
   const double n = (double)(1ull << ft.job.m), zeta = ft.job.zeta;
-  double q = 0, gsum = 0, ld = 0, sp = 0, sy = 0;
+  double s[5] = {0, 0, 0, 0, 0};  // quadratic form, sum g, log det, sum p, sum y
   for (uint32_t b = threadIdx.x; b < tiles; b += blockDim.x) {
-    q += __ldcg(&ft.qg[((uint64_t)v * tiles + b) * 2 + 0]);
-    gsum += __ldcg(&ft.qg[((uint64_t)v * tiles + b) * 2 + 1]);
-    ld += __ldcg(&ft.ld[(uint64_t)r * tiles + b]);
-    sp += __ldcg(&ft.sp[(uint64_t)r * tiles + b]);
-    sy += __ldcg(&ft.sy[(uint64_t)v * tiles + b]);
+    if (scalars) {
+      s[0] += __ldcg(&ft.qg[((uint64_t)v * tiles + b) * 2 + 0]);
+      s[1] += __ldcg(&ft.qg[((uint64_t)v * tiles + b) * 2 + 1]);
+      s[2] += __ldcg(&ft.ld[(uint64_t)r * tiles + b]);
+    }
+    s[3] += __ldcg(&ft.sp[(uint64_t)r * tiles + b]);
+    s[4] += __ldcg(&ft.sy[(uint64_t)v * tiles + b]);
   }
-  q = block_sum(q, sh);
-  gsum = block_sum(gsum, sh);
-  ld = block_sum(ld, sh);
-  sp = block_sum(sp, sh);
-  sy = block_sum(sy, sh);
-  __shared__ double res[5];
-  if (threadIdx.x == 0) {
-    res[0] = q, res[1] = gsum, res[2] = ld, res[3] = sp, res[4] = sy;
+#pragma unroll
+  for (int k = 0; k < 5; ++k) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s[k] += __shfl_xor_sync(0xffffffffu, s[k], o);
+    if ((threadIdx.x & 31) == 0) sh[k][threadIdx.x >> 5] = s[k];
+  }
+  __syncthreads();
+  if (threadIdx.x < 5) {
+    double t = 0.0;
+    for (int q = 0; q < (int)(blockDim.x >> 5); ++q) t += sh[threadIdx.x][q];
+    res[threadIdx.x] = t;
   }
   __syncthreads();
   const double lam0 = zeta * (n + res[3]) + ft.eta;  // lambda_0 from the FP64 sum of p
   const double mfac = -zeta * res[4] / (lam0 * lam0);
-  if (threadIdx.x == 0) {
+  if (scalars && threadIdx.x == 0) {
     double *o = ft.out + (uint64_t)v * QK_MLL_NOUT;
     o[QK_MLL_QUAD] = res[0];
     o[QK_MLL_LOGDET] = res[2];
@@ -959,7 +1069,7 @@ __device__ __forceinline__ void fused_final_item(const FTask &ft, uint32_t v) {
   if (!ft.grad) return;
   double *g = ft.grad + (uint64_t)v * (2 * d + 2);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (uint32_t j = warp; j < 2 * d; j += blockDim.x >> 5) {
+  for (uint32_t j = j0 + warp; j < j1; j += blockDim.x >> 5) {
     double s = 0.0;
     for (uint32_t b = lane; b < ft.gblocks; b += 32) s += __ldcg(&ft.gr[((uint64_t)v * ft.gblocks + b) * 2 * d + j]);
 #pragma unroll
@@ -969,13 +1079,17 @@ __device__ __forceinline__ void fused_final_item(const FTask &ft, uint32_t v) {
       else g[d + 1 + (j - d)] = mfac * s;
     }
   }
-  if (threadIdx.x == 0) {
+  if (scalars && threadIdx.x == 0) {
     g[d] = res[1];
     g[2 * d + 1] = mfac;
   }
 }
 
-static __global__ void __launch_bounds__(256) k_fused_final(FTask ft) { fused_final_item(ft, blockIdx.x); }
+// CTA (v, y): 8 gradient entries of vector v, one per warp; y = 0 the MLL outputs as well.
+static __global__ void __launch_bounds__(256) k_fused_final(FTask ft) {
+  const uint32_t j0 = 8 * blockIdx.y, d2 = 2 * ft.job.d;
+  fused_final_item(ft, blockIdx.x, j0, j0 + 8 < d2 ? j0 + 8 : d2, blockIdx.y == 0);
+}
 
 // -------------------------------------- persistent whole-pipeline schedule (one launch)
 // Every randomization of every task is a unit u with four kinds of work items: A tiles,
@@ -1093,7 +1207,7 @@ __global__ void __launch_bounds__(kFNT, 2) k_fused_persist(PSched ps) {
       if constexpr (sizeof(T) == 8) fused_C64_item<ALPHA>(pu.ft, idx, smem);
       else fused_C_item<FAM, ALPHA>(pu.ft, idx / pu.tiles, idx % pu.tiles, smem);
     } else {
-      fused_final_item(pu.ft, idx);
+      fused_final_item(pu.ft, idx, 0, 2 * pu.ft.job.d, true);
     }
     __syncthreads();  // every thread's stores (and shared-memory reads) are done
     if (t == 0)
@@ -1108,7 +1222,7 @@ int launch_fused_t(const FTask &ft, cudaStream_t st, LaunchTimer *tm) {
   const size_t colb = align256(col_smem_bytes<L>(d));
   // phase A keeps a second tile for the lo parts when compensating
   const size_t smA = colb + xtile_bytes<T>() + 32 * sizeof(double);
-  const size_t smB = 3 * xtile_bytes<T>() + 32 * sizeof(double);
+  const size_t smB = fused_B_smem<T>();
   smem_optin<k_fused_A<T, FAM, ALPHA, COMP, WIDE>>(smA);
   smem_optin<k_fused_B<T, COMP, WIDE>>(smB);
   if (tm) tm->begin("k_fused_A", st);
@@ -1123,6 +1237,7 @@ int launch_fused_t(const FTask &ft, cudaStream_t st, LaunchTimer *tm) {
   if (ft.c || ft.grad) {
     if (tm) tm->begin("k_fused_C", st);
     if constexpr (sizeof(T) == 8) {
+      smem_optin<k_fused_C64>(xtile_bytes<double>());
       k_fused_C64<<<dim3(ft.tiles, R * ft.nrhs), kFNT, xtile_bytes<double>(), st>>>(ft);
     } else {
       const size_t smC = colb + xtile_bytes<T>() + (size_t)(kFNT / 32) * 2 * d * sizeof(double);
@@ -1141,7 +1256,7 @@ int launch_fused_t(const FTask &ft, cudaStream_t st, LaunchTimer *tm) {
     }
   }
   if (tm) tm->begin("k_fused_final", st);
-  k_fused_final<<<R * ft.nrhs, 256, 0, st>>>(ft);
+  k_fused_final<<<dim3(R * ft.nrhs, ft.grad ? (2 * d + 7) / 8 : 1), 256, 0, st>>>(ft);
   if (tm) tm->end(st);
   return check_launch("fused final");
 }
@@ -1162,7 +1277,7 @@ int persist_launch_t(const PSched &ps, uint32_t dmax, cudaStream_t st) {
   constexpr int L = FCfg<T>::L;
   const size_t colb = align256(col_smem_bytes<L>(dmax));
   const size_t smA = colb + xtile_bytes<T>() + 32 * sizeof(double);
-  const size_t smB = 3 * xtile_bytes<T>() + 32 * sizeof(double);
+  const size_t smB = fused_B_smem<T>();
   const size_t smC = sizeof(T) == 8 ? grad64_smem(dmax, QK_MAX_M, 8)  // above its transforms' xtile_bytes (in smA)
                                     : colb + xtile_bytes<T>() + (size_t)(kFNT / 32) * 2 * dmax * sizeof(double);
   size_t sm = smA > smB ? smA : smB;

@@ -67,6 +67,8 @@ bool fused_supported(const qk_task &t, int dtype);
 bool tiled_wht_supported(uint32_t m, int dtype);
 int tiled_wht(void *x, uint32_t m, uint64_t nvec, int dtype, double scale, cudaStream_t st,
               size_t chunk_bytes = ~(size_t)0);
+// One pass of the multi-pass FP64 transform in 96-bit integers (2^c columns, row bits from s).
+int wht64_pass(double *x, int m, int s, int c, uint64_t blocks, double scale, cudaStream_t st);
 // Persistent single-launch batched WHT (qk_fused.cu) and its tuner (qk_tune.cu).
 constexpr uint32_t kSpinLimit = 1u << 23;  // ~1 s of 128 ns sleeps
 size_t persist_wht_ws_bytes(uint64_t nvec);

@@ -1,0 +1,85 @@
+// Quotients without FP64 divisions (GB300: about 2 FP64 lanes per SM and cycle): reciprocals and
+// quotients to about one FP64 rounding from the FP32 reciprocal estimate, and the FP32 scaling by
+// an FP64 eigenvalue in float-float arithmetic.
+#pragma once
+
+#include "qk_common.cuh"
+
+namespace qk {
+
+// Approximate reciprocal (PTX rcp.approx.ftz.f32, max 1 ulp; subnormals flush to 0): 1/0 = inf.
+__device__ __forceinline__ float rcp_approx(float a) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
+  return r;
+}
+// a / b in FP64 without the FP64 divide (GB300 has about two FP64 lanes per SM and cycle):
+// from the FP32 reciprocal estimate r of b (its leading 24 bits, relative error e below
+// 2^-22), q0 = a r, then q0 (1 + e + e^2) with e = 1 - b r rounded once: what is left is e^3,
+// below 2^-66, so the result is within 2 ulp of the rounded quotient (checked against the
+// divide by qk_ratio_selftest).  Four FP64 instructions.  False for b outside
+// 2^-100 .. 2^100 in magnitude (zero, subnormal, inf and NaN included).
+__device__ __forceinline__ bool ratio_fast(double a, double b, double &q) {
+  const uint32_t hi = (uint32_t)__double2hiint(b), lo = (uint32_t)__double2loint(b);
+  const uint32_t ex = (hi >> 20) & 0x7FFu;
+  if (ex - 923u > 200u) return false;
+  const uint32_t fb = (hi & 0x80000000u) | ((ex - 896u) << 23) | ((hi & 0xFFFFFu) << 3) | (lo >> 29);
+  const double r = f2d_exact(rcp_approx(__uint_as_float(fb)));
+  const double e = fma(-b, r, 1.0);
+  const double q0 = a * r;
+  q = fma(q0, fma(e, e, e), q0);
+  return true;
+}
+__device__ __forceinline__ double ratio(double a, double b) {
+  double q;
+  return ratio_fast(a, b, q) ? q : a / b;
+}
+
+// 1 / b as ratio_fast(1, b): one rounding, 3 FP64 instructions.
+__device__ __forceinline__ double rcp64(double b) {
+  const uint32_t hi = (uint32_t)__double2hiint(b), lo = (uint32_t)__double2loint(b);
+  const uint32_t ex = (hi >> 20) & 0x7FFu;
+  if (ex - 923u > 200u) return 1.0 / b;
+  const uint32_t fb = (hi & 0x80000000u) | ((ex - 896u) << 23) | ((hi & 0xFFFFFu) << 3) | (lo >> 29);
+  const double r = f2d_exact(rcp_approx(__uint_as_float(fb)));
+  const double e = fma(-b, r, 1.0);
+  return fma(r, fma(e, e, e), r);
+}
+
+// 1 / b correctly rounded: one more Newton step, whose residual is exact and whose last operation
+// is one rounding (Markstein 1990: correct unless b's mantissa is all ones, which takes the
+// divide).  For the lattices' spectral step, where sums over cancelling terms near a small
+// nugget show the last bit.
+__device__ __forceinline__ double rcp64_exact(double b) {
+  const uint32_t hi = (uint32_t)__double2hiint(b), lo = (uint32_t)__double2loint(b);
+  const uint32_t ex = (hi >> 20) & 0x7FFu;
+  if (ex - 923u > 200u || ((hi & 0xFFFFFu) == 0xFFFFFu && lo == 0xFFFFFFFFu)) return 1.0 / b;
+  const double r = rcp64(b);
+  return fma(r, fma(-b, r, 1.0), r);
+}
+
+// x / lambda fac (inverse) or x lambda fac, fac a power of two.  FP32: lambda as a float pair (its
+// leading 24 bits and the rest, by integer operations), the quotient or product to about 2^-44
+// before it is rounded to FP32: the FP64 division's result without FP64 instructions; x or
+// lambda outside a wide middle range takes FP64.
+__device__ __forceinline__ double scale_lambda(double x, double lam, double fac, bool inverse) {
+  return x * (inverse ? fac * rcp64(lam) : fac * lam);
+}
+__device__ __forceinline__ float scale_lambda(float x, double lam, double fac, bool inverse) {
+  const uint32_t hi = (uint32_t)__double2hiint(lam), lo = (uint32_t)__double2loint(lam);
+  const uint32_t ex = (hi >> 20) & 0x7FFu, xe = (__float_as_uint(x) >> 23) & 0xFFu;
+  if (ex - 983u > 80u || (hi & 0x80000000u) || (xe - 87u > 80u && x != 0.f))
+    return (float)((double)x * (inverse ? fac / lam : fac * lam));
+  const float lh = __uint_as_float(((ex - 896u) << 23) | ((hi & 0xFFFFFu) << 3) | (lo >> 29));
+  const float ll = __uint2float_rn(lo & 0x1FFFFFFFu) * __uint_as_float((ex - 948u) << 23);
+  float a = lh, b = ll;
+  if (inverse) {
+    a = rcp_approx(lh);
+    const float e = __fmaf_rn(-ll, a, __fmaf_rn(-lh, a, 1.f));
+    b = __fmul_rn(a, __fmaf_rn(e, e, e));
+  }
+  const float p = __fmul_rn(x, a);
+  return __fadd_rn(p, __fmaf_rn(x, b, __fmaf_rn(x, a, -p))) * (float)fac;
+}
+
+}  // namespace qk
