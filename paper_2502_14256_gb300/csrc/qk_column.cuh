@@ -33,7 +33,7 @@ __device__ __forceinline__ uint32_t xor_columns(const uint32_t *col, uint32_t v)
 }
 
 // DSI kernels as polynomials in the converted word fz = (T)Z with coefficients that
-// depend only on beta, i.e. on clz(Z) (the Theorem of Sec. 5.3; x = fz 2^-32):
+// depend only on beta, i.e. on Z's leading bit (the Theorem of Sec. 5.3; x = fz 2^-32):
 //   order 1: K = 1 - 3 t1                         (1 at Z = 0)
 //   order 2: K = (3/2 - 5/2 t1) - beta 2^-32 fz; FP64 rows hold (3/2 - 5/2 t1 + beta, -beta),
 //            both exact, and take X = 1 + fz 2^-32 (mantissa bits, no conversion): the same
@@ -41,8 +41,10 @@ __device__ __forceinline__ uint32_t xor_columns(const uint32_t *col, uint32_t v)
 //   order 3: K = (-1 + 43/18 (1 - t2)) - 5 (1 - t1) 2^-32 fz + beta 2^-64 fz^2
 //   order 4: K = (-1 + 701/294 (1 - t3)) - 43/9 (1 - t2) 2^-32 fz + 5 (1 - t1) 2^-64 fz^2
 //                - 2/3 beta 2^-96 fz^3 - beta/24 S'(Z)
-// Row r = clz(Z) in 0..32 (r = 32 is Z = 0: beta = t = 0); rows are padded to a
-// power-of-two stride so that each lookup is one (or two) vector loads.
+// Row r = 1 + the position of Z's leading bit, 0..32 (r = 0 is Z = 0: beta = t = 0), so that the
+// row's address is one multiply-add of what the find-leading-one instruction returns (-1 for
+// Z = 0; clz would take a subtraction more per factor); rows are padded to a power-of-two
+// stride so that each lookup is one (or two) vector loads.
 // S'(Z) = sum of 8^-a over set digits x_{a+1} is read from a 256-entry byte table:
 // S' = T[b0] + 2^-24 T[b1] + 2^-48 T[b2] + ... for the bytes b0, b1, ... of Z.
 constexpr int kTabRows = 33, kTabNC = 8, kOctRows = 256;
@@ -101,12 +103,12 @@ __host__ __device__ constexpr DsiTable<T> make_dsi_table() {
   DsiTable<T> tab{};
   constexpr int S = tab_stride(ALPHA);
   for (int q = 0; q < kTabRows; ++q) {
-    const int beta = q < 32 ? q + 1 : 0;
-    const double t1 = q < 32 ? pow2neg(beta) : 0.0, t2 = t1 * t1, t3 = t2 * t1;
+    const int beta = q ? 33 - q : 0;
+    const double t1 = q ? pow2neg(beta) : 0.0, t2 = t1 * t1, t3 = t2 * t1;
     const double b = (double)beta;
     double A = 0, B = 0, C = 0, D = 0, E = 0;
     if (ALPHA == 1) {
-      A = q < 32 ? 1.0 - 3.0 * t1 : 1.0;
+      A = q ? 1.0 - 3.0 * t1 : 1.0;
     } else if (ALPHA == 2) {
       A = 1.5 - 2.5 * t1;
       B = -b * pow2neg(32);
@@ -156,12 +158,12 @@ template <int ALPHA>
 __host__ __device__ constexpr DsiTableFF make_dsi_table_ff() {
   DsiTableFF tab{};
   for (int q = 0; q < kTabRows; ++q) {
-    const int beta = q < 32 ? q + 1 : 0;
-    const double t1 = q < 32 ? pow2neg(beta) : 0.0, t2 = t1 * t1, t3 = t2 * t1;
+    const int beta = q ? 33 - q : 0;
+    const double t1 = q ? pow2neg(beta) : 0.0, t2 = t1 * t1, t3 = t2 * t1;
     const double b = (double)beta;
     double co[5] = {0, 0, 0, 0, 0};
     if (ALPHA == 1) {
-      co[0] = q < 32 ? 1.0 - 3.0 * t1 : 1.0;
+      co[0] = q ? 1.0 - 3.0 * t1 : 1.0;
     } else if (ALPHA == 2) {
       co[0] = 1.5 - 2.5 * t1;
       co[1] = -b * pow2neg(32);
@@ -209,6 +211,12 @@ __device__ void build_dsi_tab(T *tab) {
   for (int q = threadIdx.x; q < kDsiTabLen; q += kColNT) tab[q] = src[q];
 }
 
+// 1 + the position of the leading one bit, 0 for Z = 0.
+__device__ __forceinline__ int lead_row(uint32_t Z) {
+  int r;
+  asm("bfind.u32 %0, %1;" : "=r"(r) : "r"(Z));
+  return r + 1;
+}
 __device__ __forceinline__ float word_to(float, uint32_t Z) { return __uint2float_rn(Z); }
 __device__ __forceinline__ double word_to(double, uint32_t Z) { return u32_to_double(Z, 0); }  // exact
 
@@ -216,7 +224,7 @@ __device__ __forceinline__ double word_to(double, uint32_t Z) { return u32_to_do
 template <typename T, int ALPHA>
 __device__ __forceinline__ T dsi_tab_eval(const T *tab, uint32_t Z) {
   constexpr int S = tab_stride(ALPHA);
-  const T *row = tab + __clz(Z) * S;
+  const T *row = tab + lead_row(Z) * S;
   if constexpr (ALPHA == 1) {
     return row[0];
   } else if constexpr (ALPHA == 2 && sizeof(T) == 8) {
@@ -380,7 +388,7 @@ __device__ __forceinline__ FF<F2> word_ff2(uint32_t Z0, uint32_t Z1) {
 // least 2^-21, above the second part, so one fast TwoSum normalises it.
 template <int ALPHA>
 __device__ __forceinline__ FF<F2> dsi_ff2(const float *tab, uint32_t Z0, uint32_t Z1) {
-  const float *r0 = tab + __clz(Z0) * kFFStride, *r1 = tab + __clz(Z1) * kFFStride;
+  const float *r0 = tab + lead_row(Z0) * kFFStride, *r1 = tab + lead_row(Z1) * kFFStride;
   const float4 a0 = *reinterpret_cast<const float4 *>(r0), a1 = *reinterpret_cast<const float4 *>(r1);
   const FF<F2> A = {vpack(a0.x, a1.x), vpack(a0.y, a1.y)};
   if constexpr (ALPHA == 1) {
