@@ -17,6 +17,8 @@
 
 #include "qk_common.cuh"
 #include "qk_internal.h"
+#include "qk_netops.h"
+#include "qk_quotient.cuh"
 #include "qk_transform.cuh"
 
 namespace qk {
@@ -35,16 +37,6 @@ template <> __device__ __forceinline__ float from_real<float>(double v) { return
 template <> __device__ __forceinline__ double from_real<double>(double v) { return v; }
 template <> __device__ __forceinline__ float2 from_real<float2>(double v) { return make_float2((float)v, 0.f); }
 template <> __device__ __forceinline__ double2 from_real<double2>(double v) { return make_double2(v, 0.0); }
-template <typename E> __device__ __forceinline__ E mul_real(E v, double s);
-template <> __device__ __forceinline__ float mul_real<float>(float v, double s) { return (float)((double)v * s); }
-template <> __device__ __forceinline__ double mul_real<double>(double v, double s) { return v * s; }
-template <> __device__ __forceinline__ float2 mul_real<float2>(float2 v, double s) {
-  return make_float2((float)((double)v.x * s), (float)((double)v.y * s));
-}
-template <> __device__ __forceinline__ double2 mul_real<double2>(double2 v, double s) {
-  return make_double2(v.x * s, v.y * s);
-}
-
 __device__ __forceinline__ uint64_t gtid() { return (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; }
 __device__ __forceinline__ uint64_t gstride() { return (uint64_t)gridDim.x * blockDim.x; }
 
@@ -99,15 +91,14 @@ __global__ void k_lam_final(const E *__restrict__ X, double *__restrict__ lam, u
   if (floored && status) atomicOr(status, (uint32_t)QK_STATUS_FLOOR);
 }
 
-// X[v][w] *= fac / lambda[v / nrhs][w] (mode 0) or fac * lambda (mode 1), in FP64.
+// X[v][w] *= fac / lambda[v / nrhs][w] (mode 0) or fac * lambda (mode 1), fac a power of two.
 template <typename E>
 __global__ void k_scale_lam(E *__restrict__ X, const double *__restrict__ lam, uint64_t total, int m,
                             uint32_t nrhs, double fac, int mode) {
   const uint64_t mask = (1ull << m) - 1;
   for (uint64_t i = gtid(); i < total; i += gstride()) {
     const uint64_t v = i >> m, w = i & mask;
-    const double l = lam[((v / nrhs) << m) + w];
-    X[i] = mul_real(X[i], mode == 0 ? fac / l : fac * l);
+    X[i] = scale_lambda(X[i], lam[((v / nrhs) << m) + w], fac, mode == 0);
   }
 }
 
@@ -117,9 +108,9 @@ __global__ void k_residual(const T *__restrict__ y, const E *__restrict__ Kc, T 
   for (uint64_t i = gtid(); i < count; i += gstride()) r[i] = (T)((double)y[i] - re(Kc[i]) * scale);
 }
 
-template <typename T>
-__global__ void k_add(T *__restrict__ c, const T *__restrict__ dc, uint64_t count) {
-  for (uint64_t i = gtid(); i < count; i += gstride()) c[i] += dc[i];
+template <typename E, typename T>
+__global__ void k_add(T *__restrict__ c, const E *__restrict__ dc, uint64_t count) {
+  for (uint64_t i = gtid(); i < count; i += gstride()) c[i] += (T)re(dc[i]);
 }
 
 constexpr int kRedNT = 256;
@@ -153,9 +144,9 @@ __global__ void k_mll_spectral(E *__restrict__ X, const double *__restrict__ lam
   for (uint64_t w = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; w < n; w += (uint64_t)gridDim.x * blockDim.x) {
     const E Y = xv[w];
     const double l = lr[w];
-    const double a = abs2(Y) * inv_n / l;
+    const double il = rcp64(l), a = abs2(Y) * (inv_n * il);
     q += a;
-    const double g = 0.5 * (a - 1.0) / l;
+    const double g = (0.5 * (a - 1.0)) * il;
     gs += g;
     xv[w] = from_real<E>(g);
   }
@@ -278,8 +269,8 @@ __global__ void k_scale_pairs(E *__restrict__ X, const double *__restrict__ lam,
     for (int h = 0; h < 2; ++h) {
       const uint64_t v = 2 * q + h < nvec ? 2 * q + h : 2 * q;  // an absent half scales a zero
       const double *lr = lam + ((v / nrhs) << m);
-      sk[h] = mode == 0 ? fac / lr[k] : fac * lr[k];
-      skk[h] = mode == 0 ? fac / lr[kk] : fac * lr[kk];
+      sk[h] = fac * (mode == 0 ? rcp64_exact(lr[k]) : lr[k]);
+      skk[h] = fac * (mode == 0 ? rcp64_exact(lr[kk]) : lr[kk]);
     }
     const double2 ck = make_double2(a.x * sk[0], a.y * sk[0]), dk = make_double2(b.x * sk[1], b.y * sk[1]);
     const double2 ckk = make_double2(a.x * skk[0], -a.y * skk[0]), dkk = make_double2(b.x * skk[1], -b.y * skk[1]);
@@ -331,9 +322,9 @@ __global__ void k_mll_spectral_pairs(const E *X, const double *__restrict__ lam,
       ck[h][0] = ck[h][1] = ckk[h][0] = ckk[h][1] = 0.0;
       if (v >= nvec) continue;
       const double *lr = lam + ((v / nrhs) << m);
-      // one division per eigenvalue; inv_n is a power of two, so sk = inv_n / lambda exactly
-      // as k_scale_pairs rounds it (the same solve as qk_solve, bit for bit)
-      const double rk = 1.0 / lr[k], rkk = 1.0 / lr[kk];
+      // one reciprocal per eigenvalue; inv_n is a power of two, so sk is inv_n / lambda as
+      // k_scale_pairs rounds it (the same solve as qk_solve, bit for bit)
+      const double rk = rcp64_exact(lr[k]), rkk = rcp64_exact(lr[kk]);
       const double sk = inv_n * rk, skk = inv_n * rkk;
       const double y2 = y[h].x * y[h].x + y[h].y * y[h].y;
       const double ak = y2 * sk;
@@ -374,14 +365,40 @@ __global__ void k_mll_spectral_pairs(const E *X, const double *__restrict__ lam,
   }
 }
 
+// Partial sums of log lambda.  FP64: log(lambda_1 lambda_2 ...) from the product of the mantissas
+// (one FP64 multiplication per eigenvalue instead of a log of some 30 instructions; relative
+// error about sqrt(count) 2^-53 of the product, so absolute in its log) and the sum of the
+// exponents, the logarithm taken every 512 factors; an eigenvalue that is not a positive
+// normal number adds its own logarithm.
 template <bool FAST_LOG>
 __global__ void k_logdet(const double *__restrict__ lam, int m, double *__restrict__ part) {
   __shared__ double sh[32];
   const uint64_t n = 1ull << m;
   const double *lr = lam + (uint64_t)blockIdx.y * n;
   double s = 0.0;
-  for (uint64_t w = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; w < n; w += (uint64_t)gridDim.x * blockDim.x)
-    s += FAST_LOG ? (double)logf((float)lr[w]) : log(lr[w]);
+  const uint64_t step = (uint64_t)gridDim.x * blockDim.x;
+  if (FAST_LOG) {
+    for (uint64_t w = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; w < n; w += step) s += (double)logf((float)lr[w]);
+  } else {
+    double prod = 1.0;
+    long long ex = 0;
+    int k = 0;
+    for (uint64_t w = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; w < n; w += step) {
+      const double l = lr[w];
+      const uint32_t hi = (uint32_t)__double2hiint(l);
+      if (hi - 0x100000u >= 0x7FE00000u) {  // zero, subnormal, negative, infinite or NaN
+        s += log(l);
+        continue;
+      }
+      ex += (int)(hi >> 20) - 1023;
+      prod *= __hiloint2double((int)((hi & 0xFFFFFu) | 0x3FF00000u), __double2loint(l));
+      if (++k == 512) {
+        s += log(prod);
+        prod = 1.0, k = 0;
+      }
+    }
+    s += fma((double)ex, 0.69314718055994530942, log(prod));
+  }
   const double t = block_sum(s, sh);
   if (threadIdx.x == 0) part[(uint64_t)blockIdx.y * gridDim.x + blockIdx.x] = t;
 }
@@ -394,66 +411,73 @@ struct FinalArgs {
   double *out, *grad;
 };
 
-constexpr int kFinNT = 256;
+constexpr int kFinNT = 256, kFinQ = 16;  // gradient entries per CTA, 16 groups of blocks each
 
-// One CTA per vector: the partial sums of the spectral step, the log-determinant, y and the
-// gradient sweep added up (threads over the blocks, then over (entry, block group)).
+// CTA (v, 0): the partial sums of the spectral step, the log-determinant and y of vector v added
+// up; CTA (v, y > 0): entries [16 (y - 1), 16 y) of its gradient, thread t taking entry t % 16
+// over the blocks t / 16 mod 16.  (One CTA per vector took 52 us at 1024 blocks of 64 entries.)
 __global__ void __launch_bounds__(kFinNT) k_mll_final(FinalArgs a) {
   __shared__ double sh[32];
   __shared__ double gsh[kFinNT];
+  __shared__ double s_sumy;
   const uint32_t v = blockIdx.x, t = threadIdx.x;
   const uint32_t r = v / a.nrhs;
   const double n = (double)(1ull << a.m);
-  double quad = 0.0, gsum = 0.0, ld = 0.0, sy = 0.0;
-  for (uint32_t b = t; b < a.bspec; b += kFinNT) {
-    quad += a.spec_part[((uint64_t)v * a.bspec + b) * 2 + 0];
-    gsum += a.spec_part[((uint64_t)v * a.bspec + b) * 2 + 1];
-  }
-  for (uint32_t b = t; b < a.blog; b += kFinNT) ld += a.log_part[(uint64_t)r * a.blog + b];
+  double sy = 0.0;
   for (uint32_t b = t; b < a.by0; b += kFinNT) sy += a.y0[(uint64_t)v * a.by0 + b];
-  quad = block_sum(quad, sh);
-  gsum = block_sum(gsum, sh);
-  ld = block_sum(ld, sh);
   sy = block_sum(sy, sh);
-  __shared__ double s_sumy;
   if (t == 0) s_sumy = sy;
   __syncthreads();
-  const double sumy = s_sumy;
-  const double lam0 = a.lam[(uint64_t)r << a.m];
-  if (t == 0) {
-    double *o = a.out + (uint64_t)v * QK_MLL_NOUT;
-    o[QK_MLL_QUAD] = quad;
-    o[QK_MLL_LOGDET] = ld;
-    o[QK_MLL_MLL] = -0.5 * quad - 0.5 * ld - 0.5 * n * 1.8378770664093454836;  // log(2 pi)
-    o[QK_MLL_MEAN] = a.zeta * sumy / lam0;
-    o[QK_MLL_VAR] = a.zeta * ((lam0 - a.zeta * n) / lam0);
-  }
-  if (!a.grad) return;
-  double *g = a.grad + (uint64_t)v * (2 * a.d + 2);
+  const double sumy = s_sumy, lam0 = a.lam[(uint64_t)r << a.m];
   const double mfac = -a.zeta * sumy / (lam0 * lam0);
-  if (t == 0) {
-    g[a.d] = gsum;
-    g[2 * a.d + 1] = mfac;
-  }
-  // entries q in [0, 2d): thread t takes entry q0 + t % nq over the blocks b = t / nq mod ng
-  const uint32_t nq2 = 2 * a.d;
-  const uint32_t nq = nq2 < (uint32_t)kFinNT ? nq2 : (uint32_t)kFinNT, ng = kFinNT / nq;
-  const double *gp = a.grad_part + (uint64_t)v * a.bgrad * nq2;
-  for (uint32_t q0 = 0; q0 < nq2; q0 += nq) {
-    const uint32_t q = q0 + t % nq, grp = t / nq;
-    double s = 0.0;
-    if (grp < ng && q < nq2)
-      for (uint32_t b = grp; b < a.bgrad; b += ng) s += gp[(uint64_t)b * nq2 + q];
-    gsh[t] = s;
-    __syncthreads();
-    if (t < nq && q < nq2) {
-      double tot = 0.0;
-      for (uint32_t k = 0; k < ng; ++k) tot += gsh[k * nq + t];
-      if (q < a.d) g[q] = tot;
-      else g[a.d + 1 + (q - a.d)] = mfac * tot;
+  double *g = a.grad + (uint64_t)v * (2 * a.d + 2);
+  if (blockIdx.y == 0) {
+    double quad = 0.0, gsum = 0.0, ld = 0.0;
+    for (uint32_t b = t; b < a.bspec; b += kFinNT) {
+      quad += a.spec_part[((uint64_t)v * a.bspec + b) * 2 + 0];
+      gsum += a.spec_part[((uint64_t)v * a.bspec + b) * 2 + 1];
     }
-    __syncthreads();
+    for (uint32_t b = t; b < a.blog; b += kFinNT) ld += a.log_part[(uint64_t)r * a.blog + b];
+    quad = block_sum(quad, sh);
+    gsum = block_sum(gsum, sh);
+    ld = block_sum(ld, sh);
+    if (t == 0) {
+      double *o = a.out + (uint64_t)v * QK_MLL_NOUT;
+      o[QK_MLL_QUAD] = quad;
+      o[QK_MLL_LOGDET] = ld;
+      o[QK_MLL_MLL] = -0.5 * quad - 0.5 * ld - 0.5 * n * 1.8378770664093454836;  // log(2 pi)
+      o[QK_MLL_MEAN] = a.zeta * sumy / lam0;
+      o[QK_MLL_VAR] = a.zeta * ((lam0 - a.zeta * n) / lam0);
+      if (a.grad) {
+        g[a.d] = gsum;
+        g[2 * a.d + 1] = mfac;
+      }
+    }
+    return;
   }
+  const uint32_t nq2 = 2 * a.d, q = (blockIdx.y - 1) * kFinQ + t % kFinQ, grp = t / kFinQ;
+  constexpr uint32_t NG = kFinNT / kFinQ;
+  const double *gp = a.grad_part + (uint64_t)v * a.bgrad * nq2 + q;
+  double s0 = 0.0, s1 = 0.0;
+  if (q < nq2) {
+    uint32_t b = grp;
+    for (; b + NG < a.bgrad; b += 2 * NG) s0 += gp[(uint64_t)b * nq2], s1 += gp[(uint64_t)(b + NG) * nq2];
+    if (b < a.bgrad) s0 += gp[(uint64_t)b * nq2];
+  }
+  gsh[t] = s0 + s1;
+  __syncthreads();
+  if (t < (uint32_t)kFinQ && q < nq2) {
+    double tot = 0.0;
+    for (uint32_t k = 0; k < NG; ++k) tot += gsh[k * kFinQ + t];
+    if (q < a.d) g[q] = tot;
+    else g[a.d + 1 + (q - a.d)] = mfac * tot;
+  }
+}
+
+static int launch_mll_final(const FinalArgs &fa, cudaStream_t st) {
+  const unsigned gy = 1 + (fa.grad ? (2 * fa.d + kFinQ - 1) / kFinQ : 0);
+  k_mll_final<<<dim3(fa.nvec, gy), kFinNT, 0, st>>>(fa);
+  return check_launch("mll final");
 }
 
 // ------------------------------------------------------------ host helpers
@@ -463,9 +487,12 @@ static unsigned grid_for(uint64_t count) {
   return (unsigned)(b < 1 ? 1 : (b > cap ? cap : b));
 }
 
-template <typename E, int KIND>
+// KEEP: the transforms of first columns (run_transform).
+template <typename E, int KIND, bool KEEP = false>
 static int xform(E *x, int m, uint64_t nvec, double scale, cudaStream_t st) {
-  return run_transform<KIND, E>(x, m, 1ull << m, nvec, scale, st);
+  if constexpr (!KEEP && KIND == XF_WHT && std::is_same<E, double>::value)
+    if (tiled_wht_supported((uint32_t)m, QK_F64)) return tiled_wht(x, (uint32_t)m, nvec, QK_F64, scale, st);
+  return run_transform<KIND, E, KEEP>(x, m, 1ull << m, nvec, scale, st);
 }
 
 template <typename E> struct IsCplx { static constexpr bool value = false; };
@@ -474,11 +501,11 @@ template <> struct IsCplx<double2> { static constexpr bool value = true; };
 
 // Forward transform (in place): WHT for real elements (nets), FFTBR (DIT) for
 // complex elements (lattices); the element type encodes the family.
-template <typename E>
+template <typename E, bool KEEP = false>
 static int fwd(int family, E *x, int m, uint64_t nvec, cudaStream_t st) {
   (void)family;
-  if constexpr (IsCplx<E>::value) return xform<E, XF_DIT>(x, m, nvec, 1.0, st);
-  else return xform<E, XF_WHT>(x, m, nvec, 1.0, st);
+  if constexpr (IsCplx<E>::value) return xform<E, XF_DIT, KEEP>(x, m, nvec, 1.0, st);
+  else return xform<E, XF_WHT, KEEP>(x, m, nvec, 1.0, st);
 }
 template <typename E>
 static int inv(int family, E *x, int m, uint64_t nvec, double scale, cudaStream_t st) {
@@ -539,12 +566,14 @@ static int eigs_t(int family, uint32_t m, uint32_t batch, int form, const void *
                   double *lam, void *ws, uint32_t *status, cudaStream_t st) {
   const uint64_t cnt = (uint64_t)batch << m;
   E *X = (E *)ws;
+  const double zmul = form == QK_COL_P ? zeta : 1.0;
+  const double dc = form == QK_COL_P ? zeta * (double)(1ull << m) : 0.0;
+  if (net_ops_supported(m, batch, sizeof(E) == 8))
+    return net_eigs<E>(m, batch, (const E *)col, X, zmul, dc, eta, nullptr, lam, status, st);
   k_load_real<T, E><<<grid_for(cnt), 256, 0, st>>>((const T *)col, X, cnt);
   int rc = check_launch("eigs load");
   if (rc) return rc;
-  if ((rc = fwd<E>(family, X, m, batch, st))) return rc;
-  const double zmul = form == QK_COL_P ? zeta : 1.0;
-  const double dc = form == QK_COL_P ? zeta * (double)(1ull << m) : 0.0;
+  if ((rc = fwd<E, true>(family, X, m, batch, st))) return rc;
   k_lam_final<E><<<grid_for(cnt), 256, 0, st>>>(X, lam, cnt, (int)m, zmul, dc, eta, status);
   return check_launch("eigs finalize");
 }
@@ -613,12 +642,15 @@ static int eigs_extend_t(int family, uint32_t m, uint32_t batch, int form, const
                          double eta, const double *lam_old, double *lam, void *ws, uint32_t *status, cudaStream_t st) {
   const uint64_t cnt = (uint64_t)batch << m;
   E *X = (E *)ws;
+  const double zmul = form == QK_COL_P ? zeta : 1.0;
+  const double dc = form == QK_COL_P ? zeta * (double)(1ull << m) : 0.0;
+  if constexpr (!IsCplx<E>::value)
+    if (net_ops_supported(m, batch, sizeof(E) == 8))
+      return net_eigs<E>(m, batch, (const E *)col_new, X, zmul, dc, eta, lam_old, lam, status, st);
   k_load_real<T, E><<<grid_for(cnt), 256, 0, st>>>((const T *)col_new, X, cnt);
   int rc = check_launch("eigs extend load");
   if (rc) return rc;
-  if ((rc = fwd<E>(family, X, m, batch, st))) return rc;
-  const double zmul = form == QK_COL_P ? zeta : 1.0;
-  const double dc = form == QK_COL_P ? zeta * (double)(1ull << m) : 0.0;
+  if ((rc = fwd<E, true>(family, X, m, batch, st))) return rc;
   k_lam_extend<E><<<grid_for(cnt), 256, 0, st>>>(X, lam_old, lam, cnt, (int)m, zmul, dc, eta, status);
   return check_launch("eigs extend");
 }
@@ -681,7 +713,7 @@ static int eigs_si_t(uint32_t m, uint32_t batch, int form, const void *col, doub
   k_load_pairs<T, E><<<grid_for(cnt), 256, 0, st>>>((const T *)col, X, batch, (int)m);
   int rc = check_launch("eigs load");
   if (rc) return rc;
-  if ((rc = xform<E, XF_DIT>(X, (int)m, np, 1.0, st))) return rc;
+  if ((rc = xform<E, XF_DIT, true>(X, (int)m, np, 1.0, st))) return rc;
   const double zmul = form == QK_COL_P ? zeta : 1.0;
   const double dc = form == QK_COL_P ? zeta * (double)(1ull << m) : 0.0;
   k_lam_pairs<E><<<grid_for(cnt), 256, 0, st>>>(X, lam, batch, (int)m, zmul, dc, eta, status);
@@ -702,20 +734,25 @@ int op_eigs(int family, uint32_t m, uint32_t batch, int dtype, int form, const v
                          : eigs_si_t<float, float2>(m, batch, form, col, zeta, eta, lam, ws, status, st);
 }
 
-// c = K^-1 y (mode 0) or K y (mode 1) in precision of E; X is scratch of nvec * n E.
+// Nets: out = op(K^-1 in) (mode 0) or op(K in) (mode 1) with transforms in E (op: NET_SET,
+// NET_ADD, or NET_RESIDUAL out = y - K in); X is scratch of nvec * n E.
 template <typename T, typename E>
-static int apply_t(int family, uint32_t m, uint32_t nvec, uint32_t nrhs, const double *lam, const T *y, T *c,
-                   E *X, int mode, cudaStream_t st) {
+static int apply_t(int family, uint32_t m, uint32_t nvec, uint32_t nrhs, const double *lam, const T *in, const T *y, T *out,
+                   E *X, int mode, int op, cudaStream_t st) {
+  if (net_ops_supported(m, nvec, sizeof(E) == 8))
+    return net_apply<E, T>(m, nvec, nrhs, lam, in, y, out, X, mode == 0, op, st);
   const uint64_t cnt = (uint64_t)nvec << m;
   const double n = (double)(1ull << m);
-  k_load_real<T, E><<<grid_for(cnt), 256, 0, st>>>(y, X, cnt);
+  k_load_real<T, E><<<grid_for(cnt), 256, 0, st>>>(in, X, cnt);
   int rc = check_launch("solve load");
   if (rc) return rc;
   if ((rc = fwd<E>(family, X, m, nvec, st))) return rc;
   k_scale_lam<E><<<grid_for(cnt), 256, 0, st>>>(X, lam, cnt, (int)m, nrhs, 1.0 / n, mode);
   if ((rc = check_launch("solve scale"))) return rc;
   if ((rc = inv<E>(family, X, m, nvec, 1.0, st))) return rc;
-  k_store_real<E, T><<<grid_for(cnt), 256, 0, st>>>(X, c, cnt, 1.0);
+  if (op == NET_RESIDUAL) k_residual<E, T><<<grid_for(cnt), 256, 0, st>>>(y, X, out, cnt, 1.0);
+  else if (op == NET_ADD) k_add<E, T><<<grid_for(cnt), 256, 0, st>>>(out, X, cnt);
+  else k_store_real<E, T><<<grid_for(cnt), 256, 0, st>>>(X, out, cnt, 1.0);
   return check_launch("solve store");
 }
 
@@ -730,24 +767,13 @@ static int solve_t(int family, uint32_t m, uint32_t batch, uint32_t nrhs, const 
   E64 *X64 = (E64 *)p;
   p += align256(sizeof(E64) * cnt);
   T *tmp = (T *)p;
-  int rc = apply_t<T, E>(family, m, nvec, nrhs, lam, y, c, X, 0, st);
-  if (rc) return rc;
-  const double n = (double)(1ull << m);
-  for (int it = 0; it < refine; ++it) {
-    // residual r = y - K c with FP64 transforms
-    k_load_real<T, E64><<<grid_for(cnt), 256, 0, st>>>(c, X64, cnt);
-    if ((rc = check_launch("refine load"))) return rc;
-    if ((rc = fwd<E64>(family, X64, m, nvec, st))) return rc;
-    k_scale_lam<E64><<<grid_for(cnt), 256, 0, st>>>(X64, lam, cnt, (int)m, nrhs, 1.0 / n, 1);
-    if ((rc = check_launch("refine scale"))) return rc;
-    if ((rc = inv<E64>(family, X64, m, nvec, 1.0, st))) return rc;
-    k_residual<E64, T><<<grid_for(cnt), 256, 0, st>>>(y, X64, tmp, cnt, 1.0);
-    if ((rc = check_launch("refine residual"))) return rc;
-    if ((rc = apply_t<T, E>(family, m, nvec, nrhs, lam, tmp, tmp, X, 0, st))) return rc;
-    k_add<T><<<grid_for(cnt), 256, 0, st>>>(c, tmp, cnt);
-    if ((rc = check_launch("refine add"))) return rc;
+  int rc = apply_t<T, E>(family, m, nvec, nrhs, lam, y, y, c, X, 0, NET_SET, st);
+  for (int it = 0; it < refine && !rc; ++it) {
+    // residual r = y - K c with FP64 transforms, then c += K^-1 r
+    if ((rc = apply_t<T, E64>(family, m, nvec, nrhs, lam, c, y, tmp, X64, 1, NET_RESIDUAL, st))) return rc;
+    rc = apply_t<T, E>(family, m, nvec, nrhs, lam, tmp, y, c, X, 0, NET_ADD, st);
   }
-  return QK_OK;
+  return rc;
 }
 
 // Lattices: c = K^-1 y (mode 0) or K y (mode 1) on pairs of vectors; X: (nvec + 1) / 2
@@ -793,7 +819,7 @@ static int solve_si_t(uint32_t m, uint32_t batch, uint32_t nrhs, const double *l
     k_residual_pairs<E64, T><<<grid_for(np << m), 256, 0, st>>>(y, X64, tmp, nvec, (int)m, 1.0);
     if ((rc = check_launch("refine residual"))) return rc;
     if ((rc = apply_si_t<T, E>(m, nvec, nrhs, lam, tmp, tmp, X, 0, st))) return rc;
-    k_add<T><<<grid_for(cnt), 256, 0, st>>>(c, tmp, cnt);
+    k_add<T, T><<<grid_for(cnt), 256, 0, st>>>(c, tmp, cnt);
     if ((rc = check_launch("refine add"))) return rc;
   }
   return QK_OK;
@@ -807,14 +833,9 @@ int op_solve(int family, uint32_t m, uint32_t batch, uint32_t nrhs, int dtype, c
       return solve_si_t<double, double2, double2>(m, batch, nrhs, lam, (const double *)y, (double *)c, refine, ws, st);
     return solve_si_t<float, float2, double2>(m, batch, nrhs, lam, (const float *)y, (float *)c, refine, ws, st);
   }
-  if (family == QK_DSI) {
-    if (dtype == QK_F64)
-      return solve_t<double, double, double>(family, m, batch, nrhs, lam, (const double *)y, (double *)c, refine, ws, st);
-    return solve_t<float, float, double>(family, m, batch, nrhs, lam, (const float *)y, (float *)c, refine, ws, st);
-  }
   if (dtype == QK_F64)
-    return solve_t<double, double2, double2>(family, m, batch, nrhs, lam, (const double *)y, (double *)c, refine, ws, st);
-  return solve_t<float, float2, double2>(family, m, batch, nrhs, lam, (const float *)y, (float *)c, refine, ws, st);
+    return solve_t<double, double, double>(family, m, batch, nrhs, lam, (const double *)y, (double *)c, refine, ws, st);
+  return solve_t<float, float, double>(family, m, batch, nrhs, lam, (const float *)y, (float *)c, refine, ws, st);
 }
 
 // X <- the unnormalised forward transform (H, or the DFT of the data in linear order) of
@@ -843,11 +864,9 @@ int op_matvec(int family, uint32_t m, uint32_t batch, uint32_t nrhs, int dtype, 
   if (family == QK_SI)
     return dtype == QK_F64 ? apply_si_t<double, double2>(m, nvec, nrhs, lam, (const double *)y, (double *)u, (double2 *)ws, 1, st)
                            : apply_si_t<float, float2>(m, nvec, nrhs, lam, (const float *)y, (float *)u, (float2 *)ws, 1, st);
-  if (family == QK_DSI)
-    return dtype == QK_F64 ? apply_t<double, double>(family, m, nvec, nrhs, lam, (const double *)y, (double *)u, (double *)ws, 1, st)
-                           : apply_t<float, float>(family, m, nvec, nrhs, lam, (const float *)y, (float *)u, (float *)ws, 1, st);
-  return dtype == QK_F64 ? apply_t<double, double2>(family, m, nvec, nrhs, lam, (const double *)y, (double *)u, (double2 *)ws, 1, st)
-                         : apply_t<float, float2>(family, m, nvec, nrhs, lam, (const float *)y, (float *)u, (float2 *)ws, 1, st);
+  if (dtype == QK_F64)
+    return apply_t<double, double>(family, m, nvec, nrhs, lam, (const double *)y, (const double *)y, (double *)u, (double *)ws, 1, NET_SET, st);
+  return apply_t<float, float>(family, m, nvec, nrhs, lam, (const float *)y, (const float *)y, (float *)u, (float *)ws, 1, NET_SET, st);
 }
 
 template <typename T, typename E>
@@ -876,23 +895,28 @@ static int mll_t(const ColJob &job, uint32_t nrhs, const double *lam, const T *y
   p += align256((uint64_t)nvec * bs * sizeof(double));
   double *grad_part = (double *)p;
 
-  k_load_real<T, E><<<grid_for(cnt), 256, 0, st>>>(y, X, cnt);
-  int rc = check_launch("mll load");
-  if (rc) return rc;
-  k_sum_rows<T><<<dim3(spec_blocks(m), nvec), 256, 0, st>>>(y, (int)m, y0);
-  if ((rc = check_launch("mll sum y"))) return rc;
-  if ((rc = fwd<E>(job.family, X, (int)m, nvec, st))) return rc;
-  k_mll_spectral<E><<<dim3(bs, nvec), kRedNT, 0, st>>>(X, lam, (int)m, nrhs, spec_part, y0);
-  if ((rc = check_launch("mll spectral"))) return rc;
+  const bool fused = net_ops_supported(m, nvec, sizeof(E) == 8);
+  const uint32_t bspec = fused ? net_mll_blocks(m, sizeof(E) == 8) : bs;  // partial sums per vector (<= bs)
+  int rc;
+  if (fused) {
+    if ((rc = net_mll<E, T>(m, nvec, nrhs, lam, y, X, spec_part, y0, grad ? u : nullptr, st))) return rc;
+  } else {
+    k_load_real<T, E><<<grid_for(cnt), 256, 0, st>>>(y, X, cnt);
+    if ((rc = check_launch("mll load"))) return rc;
+    k_sum_rows<T><<<dim3(spec_blocks(m), nvec), 256, 0, st>>>(y, (int)m, y0);
+    if ((rc = check_launch("mll sum y"))) return rc;
+    if ((rc = fwd<E>(job.family, X, (int)m, nvec, st))) return rc;
+    k_mll_spectral<E><<<dim3(bs, nvec), kRedNT, 0, st>>>(X, lam, (int)m, nrhs, spec_part, y0);
+    if ((rc = check_launch("mll spectral"))) return rc;
+  }
   if (dtype == QK_F64)
     k_logdet<false><<<dim3(bs, job.nr), kRedNT, 0, st>>>(lam, (int)m, log_part);
   else  // FP32 logs of FP32-rounded eigenvalues: each log is off by ~eps32 (absolute)
     k_logdet<true><<<dim3(bs, job.nr), kRedNT, 0, st>>>(lam, (int)m, log_part);
   if ((rc = check_launch("mll logdet"))) return rc;
   if (grad) {
-    // u = H g (nets) or the DFT of g read back in natural order (lattices); real.
-    if ((rc = inv<E>(job.family, X, (int)m, nvec, 1.0, st))) return rc;
-    if (SEP_U) {
+    if (!fused && (rc = inv<E>(job.family, X, (int)m, nvec, 1.0, st))) return rc;  // u = H g
+    if (SEP_U && !fused) {
       k_store_real<E, T><<<grid_for(cnt), 256, 0, st>>>(X, u, cnt, 1.0);
       if ((rc = check_launch("mll u"))) return rc;
     }
@@ -902,7 +926,7 @@ static int mll_t(const ColJob &job, uint32_t nrhs, const double *lam, const T *y
   fa.nvec = nvec;
   fa.nrhs = nrhs;
   fa.d = job.d;
-  fa.bspec = bs;
+  fa.bspec = bspec;
   fa.blog = bs;
   fa.bgrad = grad_blocks(m, sizeof(T) == 8);
   fa.m = (int)m;
@@ -912,11 +936,10 @@ static int mll_t(const ColJob &job, uint32_t nrhs, const double *lam, const T *y
   fa.log_part = log_part;
   fa.grad_part = grad_part;
   fa.y0 = y0;
-  fa.by0 = bs;
+  fa.by0 = bspec;
   fa.out = out;
   fa.grad = grad;
-  k_mll_final<<<nvec, kFinNT, 0, st>>>(fa);
-  return check_launch("mll final");
+  return launch_mll_final(fa, st);
 }
 
 // Lattices: MLL, gradient and (with c) the solve on pairs of vectors.  Forward transforms in
@@ -1016,8 +1039,7 @@ static int mll_si_t(const ColJob &job, uint32_t nrhs, const double *lam, const T
   fa.by0 = bs;
   fa.out = out;
   fa.grad = grad;
-  k_mll_final<<<(unsigned)nvec, kFinNT, 0, st>>>(fa);
-  return check_launch("mll final");
+  return launch_mll_final(fa, st);
 }
 
 // MLL, gradient and solve of lattice tasks in one pass (dtype QK_F64, QK_F32W or QK_F32):

@@ -23,6 +23,7 @@
 #include <vector>
 
 #include "qk_common.cuh"
+#include "qk_internal.h"
 
 namespace qk {
 
@@ -242,11 +243,49 @@ __device__ __forceinline__ TileMap make_tilemap(const PassDesc &p, int LOGE, uin
   return t;
 }
 
+// The FFT round on bits 0 .. R-1 of the index: every group's twiddle is 1, so the butterflies
+// keep constant roots only, 10 multiplications for 16 elements instead of 32 and a sincospi
+// (the same values: a product with 1, 0 or -i is exact).
+__device__ __forceinline__ float2 cmul_i(float2 a, int sign) { return sign < 0 ? make_float2(a.y, -a.x) : make_float2(-a.y, a.x); }
+__device__ __forceinline__ double2 cmul_i(double2 a, int sign) { return sign < 0 ? make_double2(a.y, -a.x) : make_double2(-a.y, a.x); }
+__device__ __forceinline__ FFC cmul_i(FFC a, int sign) {  // packed (re, im): im is the high half
+  const unsigned long long m = sign < 0 ? 0x8000000000000000ull : 0x0000000080000000ull;
+  return {F2{vswap(a.h).v ^ m}, F2{vswap(a.l).v ^ m}};
+}
+template <int KIND, int R, typename E>
+__device__ __forceinline__ void radix_round_first(E (&v)[1 << R]) {
+  using S = typename ScalarOf<E>::type;
+  constexpr int SIGN = KIND == XF_DIT ? -1 : 1;
+  auto root = [&](E a, int k) -> E {  // a e^{sign i pi k / 8}
+    if (k == 0) return a;
+    if (k == 4) return cmul_i(a, SIGN);
+    return cmul(a, root8<E>(k, S(SIGN)));
+  };
+#pragma unroll
+  for (int i = 0; i < R; ++i) {
+    const int h = KIND == XF_DIT ? i : R - 1 - i;
+#pragma unroll
+    for (int q = 0; q < (1 << R); ++q)
+      if (!(q & (1 << h))) {
+        const int k = (q & ((1 << h) - 1)) << (3 - h);
+        const E a = v[q], b = KIND == XF_DIT ? root(v[q | (1 << h)], k) : v[q | (1 << h)];
+        v[q] = a + b;
+        v[q | (1 << h)] = KIND == XF_DIT ? a - b : root(a - b, k);
+      }
+  }
+}
+
 // Radix-2^R butterflies over R row bits starting at tile bit position `pos`
 // (global bit gb0), on the 2^R elements v[] of one group.
 template <int KIND, int R, typename E>
 __device__ __forceinline__ void radix_round(E (&v)[1 << R], uint64_t glow, int gb0) {
   using S = typename ScalarOf<E>::type;
+  if constexpr (KIND != XF_WHT) {
+    if (gb0 == 0) {
+      radix_round_first<KIND, R, E>(v);
+      return;
+    }
+  }
   if constexpr (KIND == XF_WHT) {
 #pragma unroll
     for (int h = 0; h < R; ++h) {
@@ -580,8 +619,10 @@ inline size_t pass_smem() {
   return (size_t)((1 << LOGE) + ((1 << LOGE) >> PAD)) * sizeof(E);
 }
 
-// Run a complete transform of `nvec` vectors of length 2^m, in place.
-template <int KIND, typename E>
+// Run a complete transform of `nvec` vectors of length 2^m, in place.  KEEP: the FP64 WHT in FP64
+// butterflies (first columns: with a small nugget the rounding of the small eigenvalues decides
+// the outputs' digits); otherwise its passes run in integers.
+template <int KIND, typename E, bool KEEP = false>
 int run_transform(E *x, int m, uint64_t vstride, uint64_t nvec, double scale, cudaStream_t st) {
   constexpr int NT = 256;
   std::vector<PassDesc> passes = plan_passes<E>(m, vstride, nvec);
@@ -608,6 +649,13 @@ int run_transform(E *x, int m, uint64_t vstride, uint64_t nvec, double scale, cu
           default: k_fft_reg<KIND, 12><<<(unsigned)blocks, NT, smem, st>>>(x, p); break;
         }
         int rc = check_launch("transform pass (registers)");
+        if (rc) return rc;
+        continue;
+      }
+    }
+    if constexpr (!KEEP && KIND == XF_WHT && std::is_same<E, double>::value) {
+      if (!p.small && p.c + p.k == 12 && p.vstride == (1ull << m)) {
+        int rc = wht64_pass(x, m, p.s, p.c, blocks, p.scale, st);
         if (rc) return rc;
         continue;
       }
