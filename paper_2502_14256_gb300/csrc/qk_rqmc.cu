@@ -15,7 +15,7 @@
 
 namespace qk {
 
-constexpr int kIntNT = 256, kIntRL = 8, kIntNP = kIntNT * kIntRL;  // points per CTA tile
+constexpr int kIntRL = 8;  // consecutive points per thread
 
 template <typename T>
 __device__ __forceinline__ T t_exp(T v) {
@@ -27,118 +27,231 @@ __device__ __forceinline__ T t_cos(T v) {
   if constexpr (sizeof(T) == 8) return cos(v);
   else return cosf(v);
 }
-template <typename T>
-__device__ __forceinline__ T t_pow(T a, T b) {
-  if constexpr (sizeof(T) == 8) return pow(a, b);
-  else return powf(a, b);
-}
 
-// Coordinate x = X 2^-32 of a word, or its baker transform 1 - 2|x - 1/2| = X' 2^-32 with
-// X' = 2X (X < 2^31) or 2^33 - 2X (exact as a 33-bit integer), converted once to T.
+// Coordinate x = X 2^-32 of a word, or its baker transform 1 - 2|x - 1/2| = X' 2^-31 with
+// X' = X (X < 2^31) or 2^32 - X, converted once to T.
+__device__ __forceinline__ uint32_t baker_word(uint32_t X) { return (int32_t)X < 0 ? 0u - X : X; }
 template <typename T>
 __device__ __forceinline__ T coord(uint32_t X, bool baker) {
-  if (!baker) {
-    if constexpr (sizeof(T) == 8) return (double)X * 0x1p-32;
-    else return __uint2float_rn(X) * 0x1p-32f;
-  }
-  const uint64_t Xb = X < 0x80000000u ? 2ull * X : (1ull << 33) - 2ull * X;
-  if constexpr (sizeof(T) == 8) return (double)Xb * 0x1p-32;
-  else return __ull2float_rn(Xb) * 0x1p-32f;
+  if constexpr (sizeof(T) == 8) return baker ? u32_to_double(baker_word(X), 31) : u32_to_double(X, 32);
+  else return baker ? __uint2float_rn(baker_word(X)) * 0x1p-31f : __uint2float_rn(X) * 0x1p-32f;
 }
 
+// Points of 64-bit mantissas: value m 2^(e - 63), m >= 2^63 or m = 0 (e then meaningless).
+// A product keeps 63 bits; used where FP64 would spend its few lanes per SM on every dimension.
+struct M64 {
+  uint64_t m;
+  int e;
+};
+__device__ __forceinline__ M64 m64_mul(M64 a, M64 b) {
+  uint64_t p = __umul64hi(a.m, b.m);  // in [2^62, 2^64) for nonzero factors
+  const int up = (p >> 63) ? 1 : 0;
+  return {up ? p : p << 1, a.e + b.e + up};
+}
+__device__ __forceinline__ M64 m64_from(uint64_t v, int t) {  // v 2^-t
+  const int c = __clzll((long long)v);
+  return {v << (c & 63), 63 - c - t};
+}
+__device__ __forceinline__ double m64_to_double(M64 a) {  // rounded once; |a.e| below the FP64 range
+  return u64_to_double(a.m, 63 - a.e);
+}
+
+// Per-dimension constants of the integrands, FP64 (d doubles), and for FP64 evaluation of the Genz
+// functions the coefficients as fixed-point words (hi, lo): c = (hi 2^24 + lo) 2^-S.
+struct FConst {
+  double *cf;
+  uint2 *fx;
+};
+constexpr int kGenzShiftOsc = 53, kGenzShiftCp = 57;  // sum c = 4.5 and 0.25: sum hi < 2^32
+
 // Running state of one point over its dimensions: the first two coordinates, a product
-// (G-function) and a linear form (Genz).
+// (G-function) and a linear form (Genz).  FP32: plain FP32 arithmetic.
 template <typename T>
 struct FState {
   T x1, x2, prod, lin;
 };
+// FP64: exact integers instead of FP64 sums and products (GB300: about 2 FP64 lanes per SM and
+// cycle, a 32 x 32 + 64 bit multiply-add issues an order of magnitude faster).  Genz: sum c_j x_j
+// from 57-bit fixed-point coefficients in two 64-bit accumulators (no rounding per
+// dimension); G-function: |4x_j - 2| - a_j = N 2^-32 is an integer N, the product of the N
+// keeps 63 bits.
+template <>
+struct FState<double> {
+  uint32_t w1, w2;
+  uint64_t hi, lo;
+  M64 prod;
+  uint32_t neg;
+};
 
 template <typename T>
-__device__ __forceinline__ void fstate_add(FState<T> &s, int f, uint32_t j, T x, const double *cf) {
+__device__ __forceinline__ void fstate_init(FState<T> &s) {
+  if constexpr (sizeof(T) == 8) {
+    s.w1 = s.w2 = s.neg = 0, s.hi = s.lo = 0, s.prod = {1ull << 63, 0};
+  } else {
+    s = FState<T>{T(0), T(0), T(1), T(0)};
+  }
+}
+
+__device__ __forceinline__ void fstate_add(FState<float> &s, int f, uint32_t j, uint32_t X, bool baker, const FConst &k) {
+  const float x = coord<float>(X, baker);
   if (j == 0) s.x1 = x;
   if (j == 1) s.x2 = x;
   if (f == QK_F_GFUN) {
-    const T a = (T)cf[j];
-    s.prod *= (fabs(T(4) * x - T(2)) - a) / (T(1) + a);
+    const float a = (float)k.cf[j];
+    s.prod *= (fabsf(4.f * x - 2.f) - a) / (1.f + a);
   } else if (f == QK_F_GENZ_OSC || f == QK_F_GENZ_CP) {
-    s.lin = fmadd((T)cf[j], x, s.lin);
+    s.lin = fmadd((float)k.cf[j], x, s.lin);
+  }
+}
+__device__ __forceinline__ void fstate_add(FState<double> &s, int f, uint32_t j, uint32_t X, bool baker, const FConst &k) {
+  if (j == 0) s.w1 = X;
+  if (j == 1) s.w2 = X;
+  if (f == QK_F_GFUN) {
+    // |4x - 2| 2^32 (a multiple of 4 or 8, below 2^34) minus a_j 2^32 = (j - 1) 2^31 (0-based j)
+    const int64_t v = baker ? ((int64_t)baker_word(X) << 3) - (1ll << 33) : ((int64_t)X << 2) - (1ll << 33);
+    const int64_t N = (v < 0 ? -v : v) - (((int64_t)j - 1) << 31);
+    s.neg ^= N < 0 ? 1u : 0u;
+    s.prod = m64_mul(s.prod, m64_from((uint64_t)(N < 0 ? -N : N), 32));
+  } else if (f == QK_F_GENZ_OSC || f == QK_F_GENZ_CP) {
+    const uint2 c = k.fx[j];
+    const uint32_t W = baker ? baker_word(X) : X;
+    s.hi += (uint64_t)c.x * W;  // sum hi_j < 2^32, W < 2^32: no overflow
+    s.lo += (uint64_t)c.y * W;  // 2^24 2^32 d, d <= 256
   }
 }
 
 template <typename T>
-__device__ __forceinline__ T fstate_value(const FState<T> &s, int f, uint32_t d) {
-  switch (f) {
-    case QK_F_SIMPLE1: return s.x1 * t_exp(s.x1) - T(1);
-    case QK_F_SIMPLE2: return s.x2 * t_exp(s.x1 * s.x2) / T(0.71828182845904523536) - T(1);  // e - 2
-    case QK_F_OAKLEY: {
-      const T t1 = (s.x1 - T(0.5)) / T(50), t2 = (s.x2 - T(0.5)) / T(50);
-      return T(5) + t1 + t2 + T(2) * t_cos(t1) + T(2) * t_cos(t2);
-    }
-    case QK_F_GFUN: return s.prod;
-    case QK_F_GENZ_OSC: return t_cos(s.lin);  // cos(-s) = cos(s)
-    default: return t_pow(T(1) + s.lin, -(T)(d + 1));
+__device__ __forceinline__ T simple_value(int f, T x1, T x2) {
+  if (f == QK_F_SIMPLE1) return x1 * t_exp(x1) - T(1);
+  if (f == QK_F_SIMPLE2) return x2 * t_exp(x1 * x2) / T(0.71828182845904523536) - T(1);  // e - 2
+  const T t1 = (x1 - T(0.5)) / T(50), t2 = (x2 - T(0.5)) / T(50);  // Oakley
+  return T(5) + t1 + t2 + T(2) * t_cos(t1) + T(2) * t_cos(t2);
+}
+__device__ __forceinline__ float fstate_value(const FState<float> &s, int f, uint32_t d, bool, const M64 &) {
+  if (f == QK_F_GFUN) return s.prod;
+  if (f == QK_F_GENZ_OSC) return cosf(s.lin);  // cos(-s) = cos(s)
+  if (f == QK_F_GENZ_CP) return powf(1.f + s.lin, -(float)(d + 1));
+  return simple_value<float>(f, s.x1, s.x2);
+}
+__device__ __forceinline__ double fstate_value(const FState<double> &s, int f, uint32_t d, bool baker, const M64 &ginv) {
+  const int wb = baker ? 31 : 32;
+  if (f == QK_F_GFUN) {
+    const double v = s.prod.m ? m64_to_double(m64_mul(s.prod, ginv)) : 0.0;
+    return s.neg ? -v : v;
   }
+  if (f == QK_F_GENZ_OSC)
+    return cos(fma(u64_to_double(s.hi, 0), 0x1p24, u64_to_double(s.lo, 0)) * exp2neg(0.0, kGenzShiftOsc + wb));
+  if (f == QK_F_GENZ_CP) {
+    // (1 + s)^-(d + 1): 1 + s = m 2^-63 with s below 1/4, the power by squaring on 64-bit
+    // mantissas (relative error below (d + 1) 2^-62), one FP64 reciprocal
+    const int sh = kGenzShiftCp - 24 + wb - 63;  // hi 2^(24 - S - wb) in units of 2^-63
+    M64 b{(1ull << 63) + ((s.hi + (s.lo >> 24)) >> sh), 0}, r{1ull << 63, 0};
+    for (uint32_t k = d + 1;; k >>= 1) {
+      if (k & 1u) r = m64_mul(r, b);
+      if (k <= 1u) break;
+      b = m64_mul(b, b);
+    }
+    return rcp64(m64_to_double(r));
+  }
+  return simple_value<double>(f, coord<double>(s.w1, baker), coord<double>(s.w2, baker));
 }
 
 // y[r][i] = f(x_i) for the points at positions i0 + [0, n) of randomization r0 + blockIdx.y.
-// A CTA covers kIntNP consecutive positions aligned to kIntNP; a thread makes kIntRL
-// consecutive points dimension by dimension (nets: seeded from the XOR tables of the tile,
-// lane and warp bits, then one XOR per point with a column known at compile time, as in
-// point generation; lattices: brev(i) g + D).
-template <typename T, bool NET>
-__global__ void __launch_bounds__(kIntNT) k_integrand(uint32_t d, int order, const uint32_t *__restrict__ Ct,
-                                                      const uint32_t *__restrict__ g, const uint32_t *__restrict__ D,
-                                                      uint32_t r0, uint64_t i0, uint64_t n, int f, int baker,
-                                                      T *__restrict__ y) {
+// A CTA of NT threads covers NT kIntRL consecutive positions aligned to that; a thread makes
+// kIntRL consecutive points dimension by dimension (nets: seeded from the XOR tables of the
+// tile, lane and warp bits, then one XOR per point with a column known at compile time, as in
+// point generation; lattices: brev(i) g + D).  NT = 64 where tiles of 2048 points would leave
+// a wave partly empty (10 x 2^15 points: 160 tiles on 152 SMs).
+template <typename T, bool NET, int NT>
+__global__ void __launch_bounds__(NT) k_integrand(uint32_t d, int order, const uint32_t *__restrict__ Ct,
+                                                  const uint32_t *__restrict__ g, const uint32_t *__restrict__ D,
+                                                  uint32_t r0, uint64_t i0, uint64_t n, int f, int baker,
+                                                  T *__restrict__ y) {
+  constexpr int NP = NT * kIntRL, NW = NT / 32;
   extern __shared__ __align__(16) unsigned char ism[];
-  double *cf = reinterpret_cast<double *>(ism);                  // (d) coefficients
-  uint32_t *ztile = reinterpret_cast<uint32_t *>(cf + d);        // (d) tile words, shift included
-  uint32_t *zlane = ztile + d;                                   // (32 d) nets
-  uint32_t *zwarp = zlane + 32 * d;                              // (8 d) nets
-  uint32_t *steps = zwarp + (kIntNT / 32) * d;                   // (3 d) nets: step columns
+  __shared__ double sh[32];
+  __shared__ double s_scale;
+  __shared__ M64 s_ginv;
+  FConst fc;
+  fc.cf = reinterpret_cast<double *>(ism);                        // (d) coefficients
+  fc.fx = reinterpret_cast<uint2 *>(fc.cf + d);                   // (d) fixed-point coefficients
+  uint32_t *ztile = reinterpret_cast<uint32_t *>(fc.fx + d);      // (d) tile words, shift included
+  uint32_t *zlane = ztile + d;                                    // (32 d) nets
+  uint32_t *zwarp = zlane + 32 * d;                               // (NW d) nets
+  uint32_t *steps = zwarp + NW * d;                               // (3 d) nets: step columns
   const uint32_t rl = blockIdx.y, r = r0 + rl;
-  const uint64_t base = ((i0 / kIntNP) + blockIdx.x) * kIntNP;  // < 2^32
+  const uint64_t base = ((i0 / NP) + blockIdx.x) * NP;  // < 2^32
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   // coefficients (FP64): Genz oscillatory / corner peak (Sec. 6), G-function a_j = (j - 2)/2
-  if (t == 0) {
-    if (f == QK_F_GENZ_OSC || f == QK_F_GENZ_CP) {
-      double sum = 0.0;
-      for (uint32_t j = 0; j < d; ++j) {
-        const double ct = f == QK_F_GENZ_OSC ? exp((double)(j + 1) * log(1e-8) / (double)d)
-                                             : 1.0 / ((double)(j + 1) * (double)(j + 1));
-        cf[j] = ct;
-        sum += ct;
+  if (f == QK_F_GENZ_OSC || f == QK_F_GENZ_CP) {
+    double sum = 0.0;
+    for (uint32_t j = t; j < d; j += NT) {
+      const double ct = f == QK_F_GENZ_OSC ? exp((double)(j + 1) * log(1e-8) / (double)d)
+                                           : 1.0 / ((double)(j + 1) * (double)(j + 1));
+      fc.cf[j] = ct;
+      sum += ct;
+    }
+    sum = block_sum(sum, sh);
+    if (t == 0) s_scale = (f == QK_F_GENZ_OSC ? 4.5 : 0.25) / sum;
+    __syncthreads();
+    const double fix = exp2neg(0.0, -(f == QK_F_GENZ_OSC ? kGenzShiftOsc : kGenzShiftCp));
+    for (uint32_t j = t; j < d; j += NT) {
+      const double c = fc.cf[j] * s_scale;
+      const uint64_t q = (uint64_t)__double2ull_rn(c * fix);
+      fc.cf[j] = c;
+      fc.fx[j] = make_uint2((uint32_t)(q >> 24), (uint32_t)q & 0xFFFFFFu);
+    }
+  } else {
+    for (uint32_t j = t; j < d; j += NT) fc.cf[j] = ((double)(j + 1) - 2.0) / 2.0;
+    if (f == QK_F_GFUN && sizeof(T) == 8 && t == 0) {
+      // 1 / prod_j (1 + a_j) = 2^d / d! : 64-bit mantissas, the reciprocal from a long division
+      M64 p{1ull << 63, 0};
+      for (uint32_t j = 2; j <= d; ++j) p = m64_mul(p, m64_from(j, 0));
+      // floor(2^126 / m) for m in [2^63, 2^64): bit by bit
+      uint64_t q = 0, rem = 1ull << 62;  // remainder of 2^62 after 0 quotient bits, then 64 steps of 2 rem
+      for (int k = 0; k < 64; ++k) {
+        const bool top = rem >> 63;
+        rem <<= 1;
+        q <<= 1;
+        if (top || rem >= p.m) rem -= p.m, q |= 1;
       }
-      const double scale = (f == QK_F_GENZ_OSC ? 4.5 : 0.25) / sum;
-      for (uint32_t j = 0; j < d; ++j) cf[j] *= scale;
-    } else {
-      for (uint32_t j = 0; j < d; ++j) cf[j] = ((double)(j + 1) - 2.0) / 2.0;
+      const M64 inv = m64_from(q, 63);  // 2^63 / m in (1/2, 1]
+      s_ginv = {inv.m, inv.e - p.e + (int)d};
     }
   }
   if constexpr (NET) {
     const uint32_t *Cr = Ct + (size_t)r * d * 32;
-    for (uint32_t q = t; q < 32 * d; q += kIntNT) {
-      const uint32_t j = q >> 5, ln = q & 31;
-      zlane[q] = xor_columns(Cr + j * 32, order_map(order, ln * kIntRL));
+    for (uint32_t q = t; q < 32 * d; q += NT) {
+      const uint32_t j = q >> 5, v = order_map(order, (q & 31) * kIntRL);
+      uint32_t acc = 0;
+#pragma unroll
+      for (int k = 2; k < 8; ++k)  // digits 3..7 of the position (and 2 in Gray order): independent loads
+        if ((v >> k) & 1u) acc ^= Cr[j * 32 + k];
+      zlane[q] = acc;
     }
-    for (uint32_t q = t; q < (kIntNT / 32) * d; q += kIntNT) {
+    for (uint32_t q = t; q < NW * d; q += NT) {
       const uint32_t w = q / d, j = q - w * d;
       zwarp[w * d + j] = xor_columns(Cr + j * 32, order_map(order, (w * 32) * kIntRL));
     }
-    for (uint32_t j = t; j < d; j += kIntNT) {
-      ztile[j] = xor_columns(Cr + j * 32, order_map(order, (uint32_t)base)) ^ (D ? D[(size_t)r * d + j] : 0u);
+    for (uint32_t j = t; j < d; j += NT) {
+      const uint32_t v = order_map(order, (uint32_t)base);
+      uint32_t acc = D ? D[(size_t)r * d + j] : 0u;
+#pragma unroll
+      for (int k = 0; k < 32; ++k)
+        if ((v >> k) & 1u) acc ^= Cr[j * 32 + k];
+      ztile[j] = acc;
       const uint32_t c0 = Cr[j * 32], c1 = Cr[j * 32 + 1], c2 = Cr[j * 32 + 2];
       steps[3 * j] = c0;
       steps[3 * j + 1] = order == QK_GRAY ? c1 : (c0 ^ c1);
       steps[3 * j + 2] = order == QK_GRAY ? c2 : (c0 ^ c1 ^ c2);
     }
   } else {
-    for (uint32_t j = t; j < d; j += kIntNT) ztile[j] = D ? D[(size_t)r * d + j] : 0u;
+    for (uint32_t j = t; j < d; j += NT) ztile[j] = D ? D[(size_t)r * d + j] : 0u;
   }
   __syncthreads();
   FState<T> st[kIntRL];
 #pragma unroll
-  for (int k = 0; k < kIntRL; ++k) st[k] = FState<T>{T(0), T(0), T(1), T(0)};
+  for (int k = 0; k < kIntRL; ++k) fstate_init<T>(st[k]);
   const uint32_t i_first = (uint32_t)base + (uint32_t)t * kIntRL;
   for (uint32_t j = 0; j < d; ++j) {
     uint32_t w[kIntRL];
@@ -159,60 +272,116 @@ __global__ void __launch_bounds__(kIntNT) k_integrand(uint32_t d, int order, con
       for (int k = 0; k < kIntRL; ++k) w[k] = __brev(i_first + k) * gj + dj;
     }
 #pragma unroll
-    for (int k = 0; k < kIntRL; ++k) fstate_add(st[k], f, j, coord<T>(w[k], baker != 0), cf);
+    for (int k = 0; k < kIntRL; ++k) fstate_add(st[k], f, j, w[k], baker != 0, fc);
   }
   T *yr = y + (size_t)rl * n;
+  const M64 ginv = s_ginv;
 #pragma unroll
   for (int k = 0; k < kIntRL; ++k) {
     const uint64_t i = (uint64_t)i_first + k;
-    if (i >= i0 && i < i0 + n) yr[i - i0] = fstate_value(st[k], f, d);
+    if (i >= i0 && i < i0 + n) yr[i - i0] = fstate_value(st[k], f, d, baker != 0, ginv);
   }
 }
 
-template <typename T>
+template <typename T, int NT>
 static int launch_integrand_t(const qk_pointset *ps, uint32_t r0, uint32_t nr, uint64_t i0, uint64_t n, int f,
                               int baker, T *y, cudaStream_t st) {
   const uint32_t d = ps->d;
-  const uint64_t tiles = (i0 + n - 1) / kIntNP - i0 / kIntNP + 1;
-  const size_t smem = sizeof(double) * d + sizeof(uint32_t) * ((size_t)d + 32 * d + (kIntNT / 32) * d + 3 * d);
+  constexpr int NP = NT * kIntRL;
+  const uint64_t tiles = (i0 + n - 1) / NP - i0 / NP + 1;
+  const size_t smem = 2 * sizeof(double) * d + sizeof(uint32_t) * ((size_t)d + 32 * d + (NT / 32) * d + 3 * d);
   const bool net = ps->kind == QK_NET_B2;
-  if (net) smem_optin<k_integrand<T, true>>(smem);
-  else smem_optin<k_integrand<T, false>>(smem);
+  if (net) smem_optin<k_integrand<T, true, NT>>(smem);
+  else smem_optin<k_integrand<T, false, NT>>(smem);
   for (uint32_t rc = 0; rc < nr; rc += 65535) {  // grid.y limit
     const uint32_t cnt = nr - rc < 65535 ? nr - rc : 65535;
     dim3 grid((unsigned)tiles, cnt);
     T *yc = y + (size_t)rc * n;
     if (net)
-      k_integrand<T, true><<<grid, kIntNT, smem, st>>>(d, ps->order, ps->Ct, nullptr, ps->D, r0 + rc, i0, n, f, baker, yc);
+      k_integrand<T, true, NT><<<grid, NT, smem, st>>>(d, ps->order, ps->Ct, nullptr, ps->D, r0 + rc, i0, n, f, baker, yc);
     else
-      k_integrand<T, false><<<grid, kIntNT, smem, st>>>(d, ps->order, nullptr, ps->g, ps->D, r0 + rc, i0, n, f, baker, yc);
+      k_integrand<T, false, NT><<<grid, NT, smem, st>>>(d, ps->order, nullptr, ps->g, ps->D, r0 + rc, i0, n, f, baker, yc);
     int rc_ = check_launch("qk_integrand");
     if (rc_) return rc_;
   }
   return QK_OK;
 }
-
-// ------------------------------------------------------------- RQMC estimate
-// Per randomization: the FP64 sum of y over the n points (one CTA per randomization).
 template <typename T>
-__global__ void __launch_bounds__(1024) k_row_means(const T *__restrict__ y, uint64_t n, double *__restrict__ mu_r) {
-  __shared__ double sh[32];
-  const T *yr = y + (size_t)blockIdx.x * n;
-  double s = 0.0;
-  for (uint64_t i = threadIdx.x; i < n; i += blockDim.x) s += (double)yr[i];
-  const double tot = block_sum(s, sh);
-  if (threadIdx.x == 0) mu_r[blockIdx.x] = tot / (double)n;
+static int launch_integrand(const qk_pointset *ps, uint32_t r0, uint32_t nr, uint64_t i0, uint64_t n, int f, int baker,
+                            T *y, cudaStream_t st) {
+  // tiles of 2048 points from eight CTAs per SM on, of 512 below
+  return (n / (256 * kIntRL)) * nr >= 8ull * sm_count() ? launch_integrand_t<T, 256>(ps, r0, nr, i0, n, f, baker, y, st)
+                                                        : launch_integrand_t<T, 64>(ps, r0, nr, i0, n, f, baker, y, st);
 }
 
-// out = [mu, sigma, half width, t, mu_1 .. mu_R]: mu_r already in out[4 ..].
+// ------------------------------------------------------------- row sums and the RQMC estimate
+// Sums of the rows of a (rows, n) array by a cluster of kRowCta CTAs per row (no scratch to
+// leave partial sums in: they meet in the first CTA's shared memory).  One CTA per row took
+// 14 us for 10 rows of 2^15 doubles; rows are many times longer than a CTA.
+constexpr int kRowCta = 8, kRowNT = 512;
+
+// FP64 sum over this cluster's row of f(i) for i < n; valid in thread 0 of the cluster's rank 0.
+template <typename F>
+__device__ __forceinline__ double cluster_row_sum(uint64_t n, F f) {
+  __shared__ double sh[32];
+  __shared__ double part[kRowCta];
+  uint32_t rank;
+  asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+  double s0 = 0.0, s1 = 0.0;
+  const uint64_t step = (uint64_t)kRowCta * kRowNT;
+  uint64_t i = (uint64_t)rank * kRowNT + threadIdx.x;
+  for (; i + step < n; i += 2 * step) s0 += f(i), s1 += f(i + step);
+  if (i < n) s0 += f(i);
+  const double s = block_sum(s0 + s1, sh);
+  if (threadIdx.x == 0) {
+    uint32_t local = (uint32_t)__cvta_generic_to_shared(&part[rank]), remote;
+    asm("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(remote) : "r"(local));
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(remote), "d"(s) : "memory");
+  }
+  // every CTA of the cluster arrives and waits: the parts are in place, no CTA has left before
+  asm volatile("barrier.cluster.arrive.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
+  double tot = 0.0;
+  if (rank == 0 && threadIdx.x == 0)
+    for (int k = 0; k < kRowCta; ++k) tot += part[k];
+  return tot;
+}
+__device__ __forceinline__ bool cluster_first() {
+  uint32_t rank;
+  asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+  return rank == 0 && threadIdx.x == 0;
+}
+
+// launch(r0, cnt): rows r0 .. r0 + cnt - 1, cnt * kRowCta CTAs (kept below the grid limit).
+template <typename F>
+static void by_rows(uint64_t rows, F launch) {
+  for (uint64_t r0 = 0; r0 < rows; r0 += 1u << 27) launch(r0, (unsigned)(rows - r0 < (1u << 27) ? rows - r0 : 1u << 27));
+}
+
+template <typename T>
+__global__ void __cluster_dims__(kRowCta, 1, 1) __launch_bounds__(kRowNT) k_row_means(const T *__restrict__ y, uint64_t n,
+                                                                                     double *__restrict__ mu_r) {
+  const uint64_t row = blockIdx.x / kRowCta;
+  const T *yr = y + row * n;
+  const double tot = cluster_row_sum(n, [&](uint64_t i) { return f2d_exact(yr[i]); });
+  if (cluster_first()) mu_r[row] = tot / (double)n;
+}
+
+// out = [mu, sigma, half width, t, mu_1 .. mu_R]: mu_r already in out[4 ..].  One warp.
 __global__ void k_rqmc_final(uint32_t R, double t_star, double *__restrict__ out) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
   const double *mu_r = out + 4;
+  const uint32_t lane = threadIdx.x;
+  auto warp_total = [](double v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+  };
   double mu = 0.0;
-  for (uint32_t r = 0; r < R; ++r) mu += mu_r[r];
-  mu /= (double)R;
+  for (uint32_t r = lane; r < R; r += 32) mu += mu_r[r];
+  mu = warp_total(mu) / (double)R;
   double ss = 0.0;
-  for (uint32_t r = 0; r < R; ++r) ss += (mu_r[r] - mu) * (mu_r[r] - mu);
+  for (uint32_t r = lane; r < R; r += 32) ss += (mu_r[r] - mu) * (mu_r[r] - mu);
+  ss = warp_total(ss);
+  if (lane) return;
   const double sigma = sqrt(ss / (double)(R - 1));
   out[0] = mu;
   out[1] = sigma;
@@ -294,17 +463,16 @@ static double student_t_quantile(double df, double p) {
 // (kappa_i = int K(u, x_i) du = zeta and int int K = zeta: each one-dimensional K_alpha
 // integrates to zero).  out (batch, 3) = [equal, optimal, optimal weight value].
 template <typename T>
-__global__ void __launch_bounds__(1024) k_discrepancy_closed(const T *__restrict__ col, int form, uint64_t n, double zeta,
-                                                             double *__restrict__ out) {
-  __shared__ double sh[32];
-  const T *cr = col + (size_t)blockIdx.x * n;
-  double s = 0.0;
-  for (uint64_t i = threadIdx.x; i < n; i += blockDim.x)
-    s += form == QK_COL_P ? (double)cr[i] : (double)cr[i] / zeta - 1.0;
-  const double S = block_sum(s, sh);
-  if (threadIdx.x == 0) {
+__global__ void __cluster_dims__(kRowCta, 1, 1) __launch_bounds__(kRowNT) k_discrepancy_closed(const T *__restrict__ col, int form,
+                                                                                              uint64_t n, double zeta,
+                                                                                              double *__restrict__ out) {
+  const uint64_t row = blockIdx.x / kRowCta;
+  const T *cr = col + row * n;
+  const double S = form == QK_COL_P ? cluster_row_sum(n, [&](uint64_t i) { return f2d_exact(cr[i]); })
+                                    : cluster_row_sum(n, [&](uint64_t i) { return (double)cr[i] / zeta - 1.0; });
+  if (cluster_first()) {
     const double nn = (double)n;
-    double *o = out + (size_t)blockIdx.x * 3;
+    double *o = out + row * 3;
     o[0] = zeta * S / nn;
     o[1] = zeta * S / (nn + S);
     o[2] = 1.0 / (nn + S);  // zeta / lambda_0
@@ -334,13 +502,12 @@ __global__ void k_quad_lambda(const E *__restrict__ X, const double *__restrict_
 }
 
 template <typename T>
-__global__ void __launch_bounds__(1024) k_weight_sums(const T *__restrict__ w, uint64_t n, double *__restrict__ out) {
-  __shared__ double sh[32];
-  const T *wr = w + (size_t)blockIdx.x * n;
-  double s = 0.0;
-  for (uint64_t i = threadIdx.x; i < n; i += blockDim.x) s += (double)wr[i];
-  const double tot = block_sum(s, sh);
-  if (threadIdx.x == 0) out[blockIdx.x] = tot;
+__global__ void __cluster_dims__(kRowCta, 1, 1) __launch_bounds__(kRowNT) k_weight_sums(const T *__restrict__ w, uint64_t n,
+                                                                                       double *__restrict__ out) {
+  const uint64_t row = blockIdx.x / kRowCta;
+  const T *wr = w + row * n;
+  const double tot = cluster_row_sum(n, [&](uint64_t i) { return f2d_exact(wr[i]); });
+  if (cluster_first()) out[row] = tot;
 }
 
 __global__ void k_discrepancy_final(uint32_t nvec, uint32_t blocks, double zeta, const double *__restrict__ part,
@@ -365,7 +532,7 @@ static int discrepancy_weights_t(int family, uint32_t m, uint32_t batch, uint32_
   double *part = (double *)p;
   p += align256(sizeof(double) * nvec * kDiscBlocks);
   double *wsum = (double *)p;
-  k_weight_sums<T><<<nvec, 1024, 0, st>>>(w, n, wsum);
+  by_rows(nvec, [&](uint64_t r0, unsigned c) { k_weight_sums<T><<<c * kRowCta, kRowNT, 0, st>>>(w + r0 * n, n, wsum + r0); });
   int rc = check_launch("discrepancy weight sums");
   if (rc) return rc;
   // unnormalised forward transform of the weights (the solve's first half)
@@ -418,8 +585,8 @@ int qk_integrand(const qk_pointset *ps, uint32_t r0, uint32_t nr, uint64_t i0, u
   if (n == 0 || nr == 0) return QK_OK;
   if (!y) return fail(QK_EINVAL, "qk_integrand: y is NULL");
   const cudaStream_t st = (cudaStream_t)stream;
-  return dtype == QK_F64 ? launch_integrand_t<double>(ps, r0, nr, i0, n, f, baker, (double *)y, st)
-                         : launch_integrand_t<float>(ps, r0, nr, i0, n, f, baker, (float *)y, st);
+  return dtype == QK_F64 ? launch_integrand<double>(ps, r0, nr, i0, n, f, baker, (double *)y, st)
+                         : launch_integrand<float>(ps, r0, nr, i0, n, f, baker, (float *)y, st);
 }
 
 int qk_rqmc(uint32_t R, uint64_t n, int32_t dtype, const void *y, double tau, double *out, qk_stream stream) {
@@ -431,8 +598,10 @@ int qk_rqmc(uint32_t R, uint64_t n, int32_t dtype, const void *y, double tau, do
   if (!y || !out) return fail(QK_EINVAL, "qk_rqmc: NULL array");
   const double t_star = student_t_quantile((double)(R - 1), 1.0 - 0.5 * tau);
   const cudaStream_t st = (cudaStream_t)stream;
-  if (dtype == QK_F64) k_row_means<double><<<R, 1024, 0, st>>>((const double *)y, n, out + 4);
-  else k_row_means<float><<<R, 1024, 0, st>>>((const float *)y, n, out + 4);
+  by_rows(R, [&](uint64_t r0, unsigned c) {
+    if (dtype == QK_F64) k_row_means<double><<<c * kRowCta, kRowNT, 0, st>>>((const double *)y + r0 * n, n, out + 4 + r0);
+    else k_row_means<float><<<c * kRowCta, kRowNT, 0, st>>>((const float *)y + r0 * n, n, out + 4 + r0);
+  });
   QK_TRY(check_launch("rqmc means"));
   k_rqmc_final<<<1, 32, 0, st>>>(R, t_star, out);
   return check_launch("rqmc interval");
@@ -450,8 +619,12 @@ int qk_discrepancy(int32_t family, uint32_t m, uint32_t batch, int32_t dtype, in
   if (!col || !out) return fail(QK_EINVAL, "qk_discrepancy: NULL array");
   const cudaStream_t st = (cudaStream_t)stream;
   const uint64_t n = 1ull << m;
-  if (dtype == QK_F64) k_discrepancy_closed<double><<<batch, 1024, 0, st>>>((const double *)col, form, n, zeta, out);
-  else k_discrepancy_closed<float><<<batch, 1024, 0, st>>>((const float *)col, form, n, zeta, out);
+  by_rows(batch, [&](uint64_t r0, unsigned c) {
+    if (dtype == QK_F64)
+      k_discrepancy_closed<double><<<c * kRowCta, kRowNT, 0, st>>>((const double *)col + r0 * n, form, n, zeta, out + 3 * r0);
+    else
+      k_discrepancy_closed<float><<<c * kRowCta, kRowNT, 0, st>>>((const float *)col + r0 * n, form, n, zeta, out + 3 * r0);
+  });
   return check_launch("qk_discrepancy");
 }
 
