@@ -11,6 +11,8 @@ applies the chain rule from c_j and eta to the parameters.
 """
 from __future__ import annotations
 
+import math
+
 import torch
 
 from . import qk
@@ -30,8 +32,10 @@ class BayesCubatureMLL(torch.autograd.Function):
         nr, nrhs, n = y.shape
         if n != 1 << m:
             raise ValueError(f"y has {n} points per right-hand side, 2^{m} expected")
-        c = (gamma * torch.exp(log_ls)).to(torch.float64).contiguous()
-        eta = float(torch.exp(log_eta))
+        ls = torch.exp(log_ls)
+        c = (gamma * ls).to(torch.float64).contiguous()
+        le = float(log_eta)  # the one host read before the launches
+        eta = math.inf if le > 709.782712893384 else math.exp(le)
         kern = qk.kernel(family, alpha, c, zeta)
         col = torch.empty((nr, n), dtype=y.dtype, device=y.device)
         qk.kernel_col(ps, kern, r0, nr, m, col, form=qk.QK_COL_P)
@@ -45,19 +49,25 @@ class BayesCubatureMLL(torch.autograd.Function):
         qk.mll(ps, kern, r0, nr, m, nrhs, eta, lam, y.contiguous(), out, grad, status=status)
         qk.read_status(status)
         if want_grad:
-            ctx.save_for_backward(grad, c, torch.exp(log_ls), torch.exp(log_eta))
-        ctx.d = d
+            ctx.save_for_backward(grad, c, ls)
+        ctx.d, ctx.eta = d, eta
         return out[..., qk.QK_MLL_MLL].clone(), out[..., qk.QK_MLL_MEAN].clone()
 
     @staticmethod
     def backward(ctx, g_mll, g_mean):
-        grad, c, ls, eta = ctx.saved_tensors
-        d = ctx.d
-        g_mll = torch.zeros_like(grad[..., 0]) if g_mll is None else g_mll.to(torch.float64)
-        g_mean = torch.zeros_like(grad[..., 0]) if g_mean is None else g_mean.to(torch.float64)
-        dc = (g_mll[..., None] * grad[..., :d] + g_mean[..., None] * grad[..., d + 1:2 * d + 1]).sum(dim=(0, 1))
-        deta = (g_mll * grad[..., d] + g_mean * grad[..., 2 * d + 1]).sum()
-        return dc * ls, dc * c, deta * eta, None, None
+        # the block is [dMLL/dc, dMLL/deta | dMEAN/dc, dMEAN/deta]: both halves contracted at once
+        grad, c, ls = ctx.saved_tensors
+        d, total = ctx.d, None
+        for g, half in ((g_mll, grad[..., :d + 1]), (g_mean, grad[..., d + 1:])):
+            if g is None:
+                continue
+            g = g.to(torch.float64)[..., None]
+            total = g * half if total is None else torch.addcmul(total, g, half)
+        if total is None:
+            total = torch.zeros_like(grad[..., :d + 1])
+        total = total.sum(dim=(0, 1))
+        dc = total[:d]
+        return dc * ls, dc * c, total[d] * ctx.eta, None, None
 
 
 def mll_and_mean(gamma, log_ls, log_eta, y, ps, family: int, alpha: int, m: int, zeta: float = 1.0, r0: int = 0):

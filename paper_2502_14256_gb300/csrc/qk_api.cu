@@ -335,14 +335,17 @@ int qk_mll(const qk_pointset *ps, const qk_kernel *k, uint32_t r0, uint32_t nr, 
 int qk_read_status(uint32_t *status, qk_stream stream) {
   g_err[0] = 0;
   if (!status) return QK_OK;
-  cudaError_t e = cudaStreamSynchronize((cudaStream_t)stream);
-  if (e != cudaSuccess) return cuda_fail(e, "qk_read_status sync");
+  // one copy and one wait; the word is cleared only where a bit is set
   uint32_t h = 0;
-  e = cudaMemcpy(&h, status, sizeof(h), cudaMemcpyDeviceToHost);
+  cudaError_t e = cudaMemcpyAsync(&h, status, sizeof(h), cudaMemcpyDeviceToHost, (cudaStream_t)stream);
   if (e != cudaSuccess) return cuda_fail(e, "qk_read_status copy");
-  const uint32_t zero = 0;
-  e = cudaMemcpy(status, &zero, sizeof(zero), cudaMemcpyHostToDevice);
-  if (e != cudaSuccess) return cuda_fail(e, "qk_read_status clear");
+  e = cudaStreamSynchronize((cudaStream_t)stream);
+  if (e != cudaSuccess) return cuda_fail(e, "qk_read_status sync");
+  if (h) {
+    e = cudaMemsetAsync(status, 0, sizeof(h), (cudaStream_t)stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize((cudaStream_t)stream);
+    if (e != cudaSuccess) return cuda_fail(e, "qk_read_status clear");
+  }
   if (h & QK_STATUS_TIMEOUT) return fail(QK_ETIMEOUT, "a bounded device wait expired");
   if (h & QK_STATUS_NOTPD) return fail(QK_ENOTPD, "an eigenvalue was <= 0: K is not positive definite");
   return QK_OK;
