@@ -61,10 +61,11 @@ int launch_lms(uint32_t d, uint32_t R, const uint32_t *C, const uint32_t *S, uin
 //   lattices: brev(i) g is additive over the fields: X = F + A(it) + T, T = brev(tile) g + D,
 // i.e. one XOR or add per word and a 16-byte store per four, no shared-memory staging and no
 // barrier between tiles (32 x 1000003 x 13 words: see the launch below).
-// Groups are aligned to 16 bytes in memory: where a randomization's tiles start phi words past
-// such a boundary, the groups shift down by phi; thread 0's first phi words then belong to the
-// end of the group region before (for its first group: to the tile's end), and it stores word by
-// word.  So do the tiles cut by the range's ends.
+// Warps' stores start on 128-byte lines (a line written in two parts by two warps costs L2 a
+// merge): where a randomization's tiles start phi words past such a boundary, the groups shift
+// down by phi; the first phi words of the shifted groups then belong to the region before (for
+// the first group: to the tile's end), their values lagging one group.  One thread at most
+// stores its first and last words one by one; so do the tiles cut by the range's ends.
 constexpr int kGenNT = 256;
 
 // log2 of the tile's points: NTA = 2^(lognp - 5) d threads, the largest that fit a CTA.
@@ -122,11 +123,11 @@ __global__ void __launch_bounds__(kGenNT) k_points(uint32_t d, int order, const 
       // start before i0)
       const uint64_t first = ((uint64_t)rl * n - i0 + base) * d;
       out = X + (int64_t)first;
-      phi = ((uint32_t)first + (uint32_t)((uintptr_t)X >> 2)) & 3u;
+      phi = ((uint32_t)first + (uint32_t)((uintptr_t)X >> 2)) & 31u;
       if (active) {
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-          const uint32_t e = 4 * t + k >= phi ? 4 * t + k - phi : words / 8 - phi + k;
+          const uint32_t e = 4 * t + k >= phi ? 4 * t + k - phi : words / 8 - phi + 4 * t + k;
           const uint32_t p = e / d, j = e - p * d;
           E[k] = e;
           uint32_t f = 0, z = 0;
@@ -158,12 +159,11 @@ __global__ void __launch_bounds__(kGenNT) k_points(uint32_t d, int order, const 
     if (active) {
       const uint64_t lo = base > i0 ? base : i0, hi = base + NP < i0 + n ? base + NP : i0 + n;
       const uint32_t elo = (uint32_t)(lo - base) * d, ehi = (uint32_t)(hi - base) * d;
-      const bool split = t == 0 && phi != 0;
+      const uint32_t lag = phi > 4 * t ? (phi - 4 * t < 4 ? phi - 4 * t : 4) : 0;  // this thread's lagging words
       uint32_t V[4];
 #pragma unroll
       for (int k = 0; k < 4; ++k) V[k] = gen_add<NET>(F[k], T[k]);
       if (elo == 0 && ehi == words) {
-        // thread 0's words below phi belong to the region before: their values lag one group
         uint32_t *dst = out + (int32_t)(4 * t - phi);
         uint32_t prev[4] = {0, 0, 0, 0};
 #pragma unroll
@@ -175,27 +175,28 @@ __global__ void __launch_bounds__(kGenNT) k_points(uint32_t d, int order, const 
 #pragma unroll
             for (int b = 0; b < 3; ++b)
               if (it & (1 << b)) v[k] = gen_add<NET>(v[k], A[b][k]);
-            o[k] = split && (uint32_t)k < phi ? prev[k] : v[k];
+            o[k] = (uint32_t)k < lag ? prev[k] : v[k];
             prev[k] = v[k];
           }
-          if (it == 0 && split) {
+          if (it > 0 || lag == 0) {
+            *reinterpret_cast<uint4 *>(dst + 4 * NTA * it) = make_uint4(o[0], o[1], o[2], o[3]);
+          } else {
 #pragma unroll
             for (int k = 1; k < 4; ++k)
-              if ((uint32_t)k >= phi) dst[k] = o[k];
-          } else {
-            *reinterpret_cast<uint4 *>(dst + 4 * NTA * it) = make_uint4(o[0], o[1], o[2], o[3]);
+              if ((uint32_t)k >= lag) dst[k] = o[k];
           }
         }
-        if (split) {
+        if (lag) {
+          uint32_t *tail = dst + words;
 #pragma unroll
-          for (int k = 0; k < 3; ++k)
-            if ((uint32_t)k < phi) out[words - phi + k] = prev[k];
+          for (int k = 0; k < 4; ++k)
+            if ((uint32_t)k < lag) tail[k] = prev[k];
         }
       } else {
         for (uint32_t it = 0; it < 8; ++it) {
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
-            const uint32_t q = split && (uint32_t)k < phi ? (it + 7) & 7 : it, e = E[k] + 4 * NTA * q;
+            const uint32_t q = (uint32_t)k < lag ? (it + 7) & 7 : it, e = E[k] + 4 * NTA * q;
             uint32_t v = V[k];
 #pragma unroll
             for (int b = 0; b < 3; ++b)
