@@ -126,15 +126,50 @@ __device__ __forceinline__ double block_sum_c(float s, float e, double *sh) {
 }
 __device__ __forceinline__ double block_sum_c(double s, double e, double *sh) { return block_sum(s + e, sh); }
 
-// Exact float -> double by integer operations for normal values (the FP64 conversion
-// unit is as slow as the FP64 adder on GB300); zero, subnormal, inf and NaN inputs take
-// the hardware conversion.
-__device__ __forceinline__ double f2d_exact(float v) {
-  const uint32_t u = __float_as_uint(v), ex = (u >> 23) & 0xFFu;
-  if (ex == 0u || ex == 0xFFu) return (double)v;
-  const uint32_t hi = (u & 0x80000000u) | ((ex + 896u) << 20) | ((u & 0x7FFFFFu) >> 3);
+// Exact float -> double by integer operations for zero and normal values (the FP64 conversion
+// unit is as slow as the FP64 adder on GB300, and occupies it even where a predicate turns it
+// off): f2d_normal; f2d_special(v) is true for the others (subnormal, infinite, NaN), which
+// take the hardware conversion (f2d_exact tests for itself).
+__device__ __forceinline__ bool f2d_special(float v) {
+  const uint32_t u = __float_as_uint(v) & 0x7FFFFFFFu;
+  return u - 1u < 0x7FFFFFu || u >= 0x7F800000u;
+}
+__device__ __forceinline__ double f2d_normal(float v) {
+  const uint32_t u = __float_as_uint(v), e = u & 0x7FFFFFFFu;
+  const uint32_t hi = (u & 0x80000000u) | (e ? (e >> 3) + 0x38000000u : 0u);
   return __hiloint2double((int)hi, (int)(u << 29));
 }
+__device__ __forceinline__ double f2d_exact(float v) {
+  if (f2d_special(v)) return (double)v;
+  return f2d_normal(v);
+}
+__device__ __forceinline__ bool f2d_special(double) { return false; }
+__device__ __forceinline__ double f2d_normal(double v) { return v; }
+// The same conversions with the special values converted out of line, for loops over elements
+// (a call is a branch; a predicated conversion would occupy the FP64 unit all the same).
+static __device__ __noinline__ double f2d_rare(float v) { return (double)v; }
+static __device__ __noinline__ float d2f_rare(double v) { return (float)v; }
+__device__ __forceinline__ double f2d_int(float v) { return f2d_special(v) ? f2d_rare(v) : f2d_normal(v); }
+__device__ __forceinline__ double f2d_int(double v) { return v; }
+// v 2^k, -64 <= k <= 64, on the exponent field where v and the result are normal.
+static __device__ __noinline__ double scale_pow2_rare(double v, int k) { return ldexp(v, k); }
+__device__ __forceinline__ double scale_pow2(double v, int k) {
+  const uint32_t hi = (uint32_t)__double2hiint(v), ex = (hi >> 20) & 0x7FFu;
+  if (ex - 65u > 1916u) return scale_pow2_rare(v, k);
+  return __hiloint2double((int)(hi + ((uint32_t)k << 20)), __double2loint(v));
+}
+// (float)v, to nearest even, by integer operations where it is zero or a normal FP32 number.
+__device__ __forceinline__ float d2f_int(double v) {
+  const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v), ex = (hi >> 20) & 0x7FFu;
+  if (ex - 898u > 250u) return (hi << 1 | lo) ? d2f_rare(v) : __uint_as_float(hi);
+  const uint32_t m = ((ex - 896u) << 23) | ((hi & 0xFFFFFu) << 3) | (lo >> 29), rem = lo & 0x1FFFFFFFu;
+  return __uint_as_float((hi & 0x80000000u) | (m + (rem > 0x10000000u || (rem == 0x10000000u && (m & 1u)))));
+}
+// 8 bytes from global to shared memory without a register in between.
+__device__ __forceinline__ void cp_async8(void *dst, const void *src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 __device__ __forceinline__ double f2d_exact(double v) { return v; }
 
 __device__ __forceinline__ uint32_t ld_acquire_u32(const uint32_t *p) {

@@ -146,9 +146,14 @@ __global__ void __launch_bounds__(kHoNT) k_kernel_col_ho(uint32_t d, int order, 
                                                          T *__restrict__ out) {
   extern __shared__ __align__(16) unsigned char csm[];
   double *wd = reinterpret_cast<double *>(csm);
-  uint64_t *zlane = reinterpret_cast<uint64_t *>(wd + d);  // [j][lane]
+  // FP64: the coefficient rows of qk_grad.cuh (1 to 4 FP64 instructions per factor where the
+  // closed form takes 6 to 12)
+  double *tab = wd + ((d + 1) & ~1u);
+  uint64_t *zlane = reinterpret_cast<uint64_t *>(tab + (sizeof(T) == 8 ? kHoRows * kHoNC : 0));  // [j][lane]
   uint64_t *zwarp = zlane + 32 * d;                         // [warp][j]
   uint64_t *zl = zwarp + (kHoNT / 32) * d;                  // [j][l]
+  if constexpr (sizeof(T) == 8)
+    for (uint32_t q = threadIdx.x; q < kHoRows * kHoNC; q += kHoNT) tab[q] = g_dsi_d64[ALPHA - 1].v[q];
   const uint32_t rl = blockIdx.y;
   const uint64_t n = 1ull << m;
   const uint64_t tile_base = (uint64_t)blockIdx.x * (kHoNT * kHoColL);
@@ -175,7 +180,11 @@ __global__ void __launch_bounds__(kHoNT) k_kernel_col_ho(uint32_t d, int order, 
     const T wj = (T)wd[j];
     const uint64_t b = zlane[j * 32 + lane] ^ zwarp[warp * d + j];
 #pragma unroll
-    for (int l = 0; l < kHoColL; ++l) p[l] = pm1_step(p[l], wj * dsi_factor64<T, ALPHA>(b ^ zl[j * kHoColL + l]));
+    for (int l = 0; l < kHoColL; ++l) {
+      const uint64_t Z = b ^ zl[j * kHoColL + l];
+      if constexpr (sizeof(T) == 8) p[l] = pm1_step(p[l], wj * dsi_tab_eval64<ALPHA>(tab, Z));
+      else p[l] = pm1_step(p[l], wj * dsi_factor64<T, ALPHA>(Z));
+    }
   }
 #pragma unroll
   for (int l = 0; l < kHoColL; ++l) {
@@ -189,7 +198,8 @@ static int launch_col_ho_t(const qk_hopointset *ps, const qk_kernel *k, uint32_t
                            T *out, cudaStream_t st) {
   const uint32_t d = ps->d;
   const uint64_t n = 1ull << m;
-  const size_t smem = sizeof(double) * d + sizeof(uint64_t) * ((size_t)32 * d + (kHoNT / 32) * d + kHoColL * d);
+  const size_t smem = sizeof(double) * (((d + 1) & ~1u) + (sizeof(T) == 8 ? kHoRows * kHoNC : 0)) +
+                      sizeof(uint64_t) * ((size_t)32 * d + (kHoNT / 32) * d + kHoColL * d);
   smem_optin<k_kernel_col_ho<T, ALPHA>>(smem);
   for (uint32_t rc = 0; rc < nr; rc += 65535) {
     const uint32_t cnt = nr - rc < 65535 ? nr - rc : 65535;

@@ -124,9 +124,16 @@ __global__ void k_sum_rows(const T *__restrict__ y, int m, double *__restrict__ 
   const uint64_t n = 1ull << m, chunk = (n + gridDim.x - 1) / gridDim.x;
   const uint64_t lo = (uint64_t)blockIdx.x * chunk, hi = lo + chunk < n ? lo + chunk : n;
   const T *yv = y + (uint64_t)blockIdx.y * n;
-  double s = 0.0;
-  for (uint64_t i = lo + threadIdx.x; i < hi; i += blockDim.x) s += (double)yv[i];
-  const double t = block_sum(s, sh);
+  double t;
+  if constexpr (sizeof(T) == 4) {  // float-float (about 2^-46): no FP64 instructions per element
+    float s = 0.f, e = 0.f;
+    for (uint64_t i = lo + threadIdx.x; i < hi; i += blockDim.x) ff_merge(s, e, yv[i], 0.f);
+    t = block_sum_c(s, e, sh);
+  } else {
+    double s = 0.0;
+    for (uint64_t i = lo + threadIdx.x; i < hi; i += blockDim.x) s += yv[i];
+    t = block_sum(s, sh);
+  }
   if (threadIdx.x == 0) out[(uint64_t)blockIdx.y * gridDim.x + blockIdx.x] = t;
 }
 
@@ -189,6 +196,13 @@ __device__ __forceinline__ double cim(double2 z) { return z.y; }
 __device__ __forceinline__ double cre(FFC z) { return ffc_re(z); }
 __device__ __forceinline__ double cim(FFC z) { return ffc_im(z); }
 
+// A pair of data values as an element: FP32 data in float-float have no low parts.
+template <typename E, typename T>
+__device__ __forceinline__ E pair_elem(T a, T b) {
+  if constexpr (std::is_same<E, FFC>::value && sizeof(T) == 4) return E{vpack(a, b), vsplat(0.f)};
+  else return cplx<E>((double)a, (double)b);
+}
+
 // out[q] = in[2q] + i in[2q+1] (real vectors of T, n = 2^m each)
 template <typename T, typename E>
 __global__ void k_load_pairs(const T *__restrict__ in, E *__restrict__ out, uint64_t nvec, int m) {
@@ -196,7 +210,7 @@ __global__ void k_load_pairs(const T *__restrict__ in, E *__restrict__ out, uint
   for (uint64_t i = gtid(); i < total; i += gstride()) {
     const uint64_t q = i >> m, w = i & mask;
     const uint64_t vb = 2 * q + 1;
-    out[i] = cplx<E>((double)in[((2 * q) << m) + w], vb < nvec ? (double)in[(vb << m) + w] : 0.0);
+    out[i] = pair_elem<E, T>(in[((2 * q) << m) + w], vb < nvec ? in[(vb << m) + w] : T(0));
   }
 }
 
@@ -309,6 +323,8 @@ __global__ void k_mll_spectral_pairs(const E *X, const double *__restrict__ lam,
   EO *cq = C ? C + (q << m) : nullptr;
   const double inv_n = 1.0 / (double)n;
   double qs[2] = {0.0, 0.0}, gs[2] = {0.0, 0.0};
+  auto sweep = [&](auto nv) {
+  constexpr int NVEC = decltype(nv)::value;  // vectors of this pair: an odd batch's last has one
   for (uint64_t k = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; k <= half;
        k += (uint64_t)gridDim.x * blockDim.x) {
     const uint64_t kk = (n - k) & (n - 1);
@@ -320,7 +336,7 @@ __global__ void k_mll_spectral_pairs(const E *X, const double *__restrict__ lam,
       const uint64_t v = 2 * q + h;
       gk[h] = gkk[h] = 0.0;
       ck[h][0] = ck[h][1] = ckk[h][0] = ckk[h][1] = 0.0;
-      if (v >= nvec) continue;
+      if (h >= NVEC) continue;
       const double *lr = lam + ((v / nrhs) << m);
       // one reciprocal per eigenvalue; inv_n is a power of two, so sk is inv_n / lambda as
       // k_scale_pairs rounds it (the same solve as qk_solve, bit for bit)
@@ -353,6 +369,9 @@ __global__ void k_mll_spectral_pairs(const E *X, const double *__restrict__ lam,
       }
     }
   }
+  };
+  if (2 * q + 1 < nvec) sweep(std::integral_constant<int, 2>());
+  else sweep(std::integral_constant<int, 1>());
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     const double sq = block_sum(qs[h], sh);
@@ -378,7 +397,12 @@ __global__ void k_logdet(const double *__restrict__ lam, int m, double *__restri
   double s = 0.0;
   const uint64_t step = (uint64_t)gridDim.x * blockDim.x;
   if (FAST_LOG) {
-    for (uint64_t w = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; w < n; w += step) s += (double)logf((float)lr[w]);
+    // each logarithm as a float, their sum as a float-float pair (FP64 sums of floats to 2^-46)
+    float fs = 0.f, fe = 0.f;
+    for (uint64_t w = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; w < n; w += step) ff_merge(fs, fe, logf(d2f_int(lr[w])), 0.f);
+    const double t = block_sum_c(fs, fe, sh);
+    if (threadIdx.x == 0) part[(uint64_t)blockIdx.y * gridDim.x + blockIdx.x] = t;
+    return;
   } else {
     double prod = 1.0;
     long long ex = 0;
