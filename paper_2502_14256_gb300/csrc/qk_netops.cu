@@ -23,19 +23,36 @@
 
 namespace qk {
 
-// lambda = zmul x + dc [w = 0] + eta with the floor and the sign test of qk_eigs.
+// lambda = zmul x + dc [w = 0] + eta with the floor and the sign test of qk_eigs, and the doubling
+// update lambda' = lambda +- t, t = zmul x + dc [w = 0].  The common form costs one FP64 fma per
+// value: eta > 0, x zero or normal; the floor compares as integers (the order of positive
+// doubles; a value below eta, negative or NaN becomes eta, and is then positive).  A thread that
+// holds w = 0 or a special x, and every thread where eta <= 0, repeats its elements in the
+// general form behind a branch: an FP64 instruction that a predicate turns off still takes its
+// time on GB300 (measured: 6 instead of 2 per element and update).
 struct LamArgs {
   double zmul, dc, eta;
   uint32_t *status;
 };
+__device__ __forceinline__ double lam_floor_int(double v, double eta, bool &floored) {
+  const long long b = __double_as_longlong(v);
+  if (b >= __double_as_longlong(eta) && b <= 0x7FF0000000000000ll) return v;
+  floored = true;
+  return eta;
+}
 template <typename T>
-__device__ __forceinline__ double lam_value(T x, bool w0, const LamArgs &a, bool &bad, bool &floored) {
-  const double xd = f2d_exact(x);
-  // positive finite x away from w = 0 with zmul, eta > 0: lambda >= eta > 0, neither test fires
-  const uint32_t h = (uint32_t)__double2hiint(xd);
-  if (a.zmul > 0.0 && a.eta > 0.0 && !w0 && h - 1u < 0x7FEFFFFFu) return fma(a.zmul, xd, a.eta);
-  double v = fma(a.zmul, xd, a.eta);
-  if (w0) v += a.dc;
+__device__ __forceinline__ double lam_fast(T x, const LamArgs &a, bool &rare, bool &floored) {
+  rare |= f2d_special(x);
+  return lam_floor_int(fma(a.zmul, f2d_normal(x), a.eta), a.eta, floored);
+}
+template <typename T>
+__device__ __forceinline__ void lam_pair_fast(T x, double old, const LamArgs &a, double (&v)[2], bool &rare, bool &floored) {
+  const double xd = f2d_normal(x);
+  rare |= f2d_special(x);
+  v[0] = lam_floor_int(fma(a.zmul, xd, old), a.eta, floored);
+  v[1] = lam_floor_int(fma(-a.zmul, xd, old), a.eta, floored);
+}
+__device__ __forceinline__ double lam_floor(double v, const LamArgs &a, bool &bad, bool &floored) {
   if (a.eta > 0.0 && !(v >= a.eta)) {  // K + eta I has no eigenvalue below eta: rounding
     v = a.eta;
     floored = true;
@@ -43,53 +60,55 @@ __device__ __forceinline__ double lam_value(T x, bool w0, const LamArgs &a, bool
   bad |= !(v > 0.0);
   return v;
 }
-// The doubling update: lambda' = lambda + t and lambda - t, t = zmul x + dc [w = 0] (one fma each).
-// Values of at least eta > 0 (compared as integers: the order of positive doubles) need no test.
+template <typename T>
+__device__ __forceinline__ double lam_value(T x, bool w0, const LamArgs &a, bool &bad, bool &floored) {
+  double v = fma(a.zmul, f2d_exact(x), a.eta);
+  if (w0) v += a.dc;
+  return lam_floor(v, a, bad, floored);
+}
 template <typename T>
 __device__ __forceinline__ void lam_pair(T x, double old, bool w0, const LamArgs &a, double (&v)[2], bool &bad, bool &floored) {
-  const double xd = f2d_exact(x);
-  if (w0) {
-    const double t = fma(a.zmul, xd, a.dc);
-    v[0] = old + t, v[1] = old - t;
-  } else {
-    v[0] = fma(a.zmul, xd, old), v[1] = fma(-a.zmul, xd, old);
-  }
-  const long long lo = __double_as_longlong(a.eta), inf = 0x7FF0000000000000ll;
-#pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    const long long b = __double_as_longlong(v[h]);
-    if (lo > 0 && b >= lo && b <= inf) continue;
-    if (a.eta > 0.0 && !(v[h] >= a.eta)) {
-      v[h] = a.eta;
-      floored = true;
-    }
-    bad |= !(v[h] > 0.0);
-  }
+  const double t = fma(a.zmul, f2d_exact(x), w0 ? a.dc : 0.0);
+  v[0] = lam_floor(old + t, a, bad, floored), v[1] = lam_floor(old - t, a, bad, floored);
 }
 __device__ __forceinline__ void lam_flags(const LamArgs &a, bool bad, bool floored) {
   if (bad && a.status) atomicOr(a.status, (uint32_t)QK_STATUS_NOTPD);
   if (floored && a.status) atomicOr(a.status, (uint32_t)QK_STATUS_FLOOR);
 }
 
+// Data into the transform's precision, and back.
+template <typename T, typename TIO>
+__device__ __forceinline__ T widen(TIO v) {
+  if constexpr (sizeof(T) == 8) return f2d_int(v);
+  else return v;
+}
+template <typename TIO, typename T>
+__device__ __forceinline__ TIO narrow(T v) {
+  if constexpr (sizeof(TIO) == 4 && sizeof(T) == 8) return d2f_int(v);
+  else return v;
+}
+
 // MLL spectral step of one frequency: adds to the quadratic form and to sum g, returns g.
 __device__ __forceinline__ double mll_g(double Y, double lam, double inv_n, double &quad, double &gs) {
-  const double il = rcp64(lam), a = Y * Y * (inv_n * il), g = (0.5 * (a - 1.0)) * il;
+  const double il = rcp64(lam), a = Y * Y * (inv_n * il), h = 0.5 * il, g = fma(a, h, -h);
   quad += a;
   gs += g;
   return g;
 }
 
-template <typename TO>
-__device__ __forceinline__ void store_op(TO *out, uint64_t i, double v, int op, const TO *y) {
-  if (op == NET_SET) out[i] = (TO)v;
-  else if (op == NET_ADD) out[i] += (TO)v;
-  else out[i] = (TO)((double)y[i] - v);  // NET_RESIDUAL
+// What is stored for a result v where `prev` is the value there (NET_ADD) or y's (NET_RESIDUAL).
+__device__ __forceinline__ float op_value(float v, float prev, int op) {
+  if (op == NET_SET) return v;
+  if (op == NET_ADD) return prev + v;
+  return d2f_int(f2d_int(prev) - f2d_int(v));
 }
-template <typename TO>
-__device__ __forceinline__ void store_op(TO *out, uint64_t i, float v, int op, const TO *y) {
-  if (op == NET_SET) out[i] = (TO)v;
-  else if (op == NET_ADD) out[i] += (TO)v;
-  else out[i] = (TO)((double)y[i] - (double)v);
+__device__ __forceinline__ float op_value(double v, float prev, int op) {
+  if (op == NET_RESIDUAL) return d2f_int(f2d_int(prev) - v);
+  const float f = d2f_int(v);
+  return op == NET_SET ? f : prev + f;
+}
+__device__ __forceinline__ double op_value(double v, double prev, int op) {
+  return op == NET_SET ? v : op == NET_ADD ? prev + v : prev - v;
 }
 
 // ------------------------------------------------------------ one CTA per vector
@@ -229,7 +248,24 @@ __global__ void __launch_bounds__(sizeof(T) == 8 ? 256 : 512) k_net_eigs_small(c
 #pragma unroll
   for (int i = 0; i < 16; ++i) x[i] = t + i * NT < n ? col[off + t + i * NT] : T(0);
   small_wht<T, 16, true>(x, m, smem);
-  bool bad = false, floored = false;
+  bool rare = t == 0 || !(a.eta > 0.0), bad = false, floored = false;  // t == 0: w = 0
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    const int e = t + i * NT;
+    if (e >= n) continue;
+    if (old) {
+      double v[2];
+      lam_pair_fast(x[i], old[off + e], a, v, rare, floored);
+      lam[2 * off + e] = v[0], lam[2 * off + n + e] = v[1];
+    } else {
+      lam[off + e] = lam_fast(x[i], a, rare, floored);
+    }
+  }
+  if (!rare) {
+    lam_flags(a, false, floored);
+    return;
+  }
+  floored = false;
 #pragma unroll
   for (int i = 0; i < 16; ++i) {
     const int e = t + i * NT;
@@ -257,7 +293,7 @@ __global__ void __launch_bounds__(sizeof(T) == 8 ? 256 : 512) k_net_apply_small(
   const double fac = 1.0 / (double)n;
   T x[16];
 #pragma unroll
-  for (int i = 0; i < 16; ++i) x[i] = t + i * NT < n ? (T)in[off + t + i * NT] : T(0);
+  for (int i = 0; i < 16; ++i) x[i] = t + i * NT < n ? widen<T>(in[off + t + i * NT]) : T(0);
   small_wht<T, 16>(x, m, smem);
 #pragma unroll
   for (int i = 0; i < 16; ++i)
@@ -265,7 +301,10 @@ __global__ void __launch_bounds__(sizeof(T) == 8 ? 256 : 512) k_net_apply_small(
   small_wht<T, 16>(x, m, smem);
 #pragma unroll
   for (int i = 0; i < 16; ++i)
-    if (t + i * NT < n) store_op(out, off + t + i * NT, x[i], op, y);
+    if (t + i * NT < n) {
+      const uint64_t j = off + t + i * NT;
+      out[j] = op_value(x[i], op == NET_SET ? TIO(0) : op == NET_ADD ? out[j] : y[j], op);
+    }
 }
 
 // The MLL's transforms: quadratic form, sum g and sum y (one partial sum per vector), u = H g.
@@ -285,7 +324,7 @@ __global__ void __launch_bounds__(sizeof(T) == 8 ? 256 : 512) k_net_mll_small(co
 #pragma unroll
   for (int i = 0; i < 16; ++i) {
     const TIO v = t + i * NT < n ? y[off + t + i * NT] : TIO(0);
-    x[i] = (T)v;
+    x[i] = widen<T>(v);
     if constexpr (sizeof(TIO) == 4) ff_add(s, e, v);
   }
   small_wht<T, 16>(x, m, smem);
@@ -295,7 +334,7 @@ __global__ void __launch_bounds__(sizeof(T) == 8 ? 256 : 512) k_net_mll_small(co
   double quad = 0.0, gs = 0.0;
 #pragma unroll
   for (int i = 0; i < 16; ++i)
-    if (t + i * NT < n) x[i] = (T)mll_g(f2d_exact(x[i]), lr[t + i * NT], inv_n, quad, gs);
+    if (t + i * NT < n) x[i] = narrow<T>(mll_g(f2d_int(x[i]), lr[t + i * NT], inv_n, quad, gs));
   quad = block_sum(quad, sh);
   gs = block_sum(gs, sh);
   if (t == 0) part[2 * blockIdx.x] = quad, part[2 * blockIdx.x + 1] = gs;
@@ -303,7 +342,7 @@ __global__ void __launch_bounds__(sizeof(T) == 8 ? 256 : 512) k_net_mll_small(co
   small_wht<T, 16>(x, m, smem);
 #pragma unroll
   for (int i = 0; i < 16; ++i)
-    if (t + i * NT < n) u[off + t + i * NT] = (TIO)x[i];
+    if (t + i * NT < n) u[off + t + i * NT] = narrow<TIO>(x[i]);
 }
 
 // --------------------------------------------------------------- two tile passes
@@ -344,7 +383,7 @@ __global__ void __launch_bounds__(kFNT, sizeof(T) == 8 ? 3 : 4) k_net_low_in(con
 #pragma unroll
   for (int l = 0; l < L; ++l) {
     const TIO a = in[base + t + (l << kLOGNT)];
-    v[l] = (T)a;
+    v[l] = widen<T>(a);
     if constexpr (sizeof(TIO) == 4)
       if (ysum) ff_add(s, e, a);
   }
@@ -363,7 +402,7 @@ __global__ void __launch_bounds__(kFNT, sizeof(T) == 8 ? 3 : 4) k_net_low_in(con
 }
 
 template <typename T, typename TIO>
-__global__ void __launch_bounds__(kFNT, sizeof(T) == 8 ? 3 : 4) k_net_low_out(const T *X, const TIO *y, TIO *out, int op) {
+__global__ void __launch_bounds__(kFNT, 3) k_net_low_out(const T *X, const TIO *y, TIO *out, int op) {
   constexpr int LOGT = FCfg<T>::LOGT, L = FCfg<T>::L;
   extern __shared__ __align__(16) unsigned char smem[];
   T *sm = reinterpret_cast<T *>(smem);
@@ -372,9 +411,17 @@ __global__ void __launch_bounds__(kFNT, sizeof(T) == 8 ? 3 : 4) k_net_low_out(co
   T v[L];
 #pragma unroll
   for (int l = 0; l < L; ++l) v[l] = X[base + t + (l << kLOGNT)];
-  xwht_full<T>(v, sm, 0);
+  TIO prev[L];  // read before the transform where the registers allow (FP32 data)
+  const TIO *src = op == NET_ADD ? out : y;
 #pragma unroll
-  for (int l = 0; l < L; ++l) store_op(out, base + e_of<T>(2, t, l), v[l], op, y);
+  for (int l = 0; l < L; ++l) prev[l] = sizeof(TIO) == 4 && op != NET_SET ? src[base + e_of<T>(2, t, l)] : TIO(0);
+  xwht_full<T>(v, sm, 0);
+  if (sizeof(TIO) == 8 && op != NET_SET) {
+#pragma unroll
+    for (int l = 0; l < L; ++l) prev[l] = src[base + e_of<T>(2, t, l)];
+  }
+#pragma unroll
+  for (int l = 0; l < L; ++l) out[base + e_of<T>(2, t, l)] = op_value(v[l], prev[l], op);
 }
 
 // The high bits of one column tile with the operation on the transform's values inside.
@@ -388,11 +435,16 @@ struct MidArgs {
   double *lam_out, *part;
   LamArgs la;
 };
-// The eigenvalues a tile needs are read four at a time, the next four in flight while these are
-// used and the first four during the transform: without it the kernel holds too few loads in
-// flight at 64 registers (n = 2^19, 32 vectors, doubling: 205 us; 84 registers, 3 CTAs per SM).
+// The eigenvalues a tile needs (EXTEND, APPLY, MLL) are copied to shared memory asynchronously
+// behind the transform tile while the transform runs, each thread reading back what it copied:
+// loaded into registers four or eight at a time the kernel waited on them (long_scoreboard 13
+// per issue; 32 x 2^19 doubling: 164 us, now 145).
+template <typename T, int MODE>
+constexpr size_t mid_smem() {
+  return xtile_bytes<T>() + (MODE == 4 || MODE == 1 || MODE == 2 ? sizeof(double) << FCfg<T>::LOGT : 0);
+}
 template <typename T, typename TIO, int MODE>
-__global__ void __launch_bounds__(kFNT, 3) k_net_mid(T *X, TIO *out, MidArgs a) {
+__global__ void __launch_bounds__(kFNT, MODE == 0 || MODE == 3 ? 3 : 2) k_net_mid(T *X, TIO *out, MidArgs a) {
   constexpr int LOGT = FCfg<T>::LOGT, L = FCfg<T>::L;
   constexpr bool KEEP = MODE == MID_EIGS || MODE == MID_EXTEND, UP = kUp<T, KEEP>;
   constexpr int LIN = UP ? 2 : 0, LMID = 2 - LIN, DF = UP ? 1 : 0;  // bits upwards: L2 then L0
@@ -408,47 +460,56 @@ __global__ void __launch_bounds__(kFNT, 3) k_net_mid(T *X, TIO *out, MidArgs a) 
   for (int l = 0; l < L; ++l) x[l] = xv[widx(e_of<T>(LIN, t, l))];
   // with_lam(f): f(l, w, lambda_w) for every element of layout LMID
   constexpr bool NEEDS = MODE == MID_EXTEND || MODE == MID_APPLY || MODE == MID_MLL;
-  constexpr int CH = 4;
   const double *lr = NEEDS ? a.lam + (uint64_t)(MODE == MID_EXTEND ? v : v / a.nrhs) * n : nullptr;
-  double lc[CH];
+  double *sl = reinterpret_cast<double *>(smem + xtile_bytes<T>());  // element (t, l) at t + 256 l
   if constexpr (NEEDS) {
 #pragma unroll
-    for (int i = 0; i < CH; ++i) lc[i] = __ldg(&lr[widx(e_of<T>(LMID, t, i))]);
+    for (int l = 0; l < L; ++l) cp_async8(&sl[t + (l << kLOGNT)], &lr[widx(e_of<T>(LMID, t, l))]);
   }
   auto with_lam = [&](auto f) {
+    cp_async_wait();
 #pragma unroll
-    for (int l0 = 0; l0 < L; l0 += CH) {
-      double ln[CH];
-      if (l0 + CH < L) {
-#pragma unroll
-        for (int i = 0; i < CH; ++i) ln[i] = __ldg(&lr[widx(e_of<T>(LMID, t, l0 + CH + i))]);
-      }
-#pragma unroll
-      for (int i = 0; i < CH; ++i) f(l0 + i, widx(e_of<T>(LMID, t, l0 + i)), lc[i]);
-      if (l0 + CH < L) {
-#pragma unroll
-        for (int i = 0; i < CH; ++i) lc[i] = ln[i];
-      }
-    }
+    for (int l = 0; l < L; ++l) f(l, widx(e_of<T>(LMID, t, l)), sl[t + (l << kLOGNT)]);
   };
   if constexpr (KEEP) xwht_col_fp<T>(x, sm, c, DF);  // LIN -> LMID
   else xwht_col<T>(x, sm, c, DF);
   if constexpr (MODE == MID_EIGS) {
+    double *dst = a.lam_out + (uint64_t)v * n;
+    bool rare = (tau == 0 && t == 0) || !(a.la.eta > 0.0);  // w = 0: element 0 of every layout
     bool bad = false, floored = false;
 #pragma unroll
-    for (int l = 0; l < L; ++l) {
-      const uint32_t w = widx(e_of<T>(LMID, t, l));
-      a.lam_out[(uint64_t)v * n + w] = lam_value(x[l], w == 0, a.la, bad, floored);
+    for (int l = 0; l < L; ++l) dst[widx(e_of<T>(LMID, t, l))] = lam_fast(x[l], a.la, rare, floored);
+    if (rare) {  // through the thread's own slots of the tile: a rolled loop, no registers held for it
+      floored = false;
+#pragma unroll
+      for (int l = 0; l < L; ++l) sm[t + (l << kLOGNT)] = x[l];
+#pragma unroll 1
+      for (int l = 0; l < L; ++l) {
+        const uint32_t w = widx(e_of<T>(LMID, t, l));
+        dst[w] = lam_value(sm[t + (l << kLOGNT)], w == 0, a.la, bad, floored);
+      }
     }
     lam_flags(a.la, bad, floored);
   } else if constexpr (MODE == MID_EXTEND) {
-    bool bad = false, floored = false;
     double *dst = a.lam_out + (uint64_t)v * 2 * n;
+    bool rare = (tau == 0 && t == 0) || !(a.la.eta > 0.0), bad = false, floored = false;
     with_lam([&](int l, uint32_t w, double old) {
       double p[2];
-      lam_pair(x[l], old, w == 0, a.la, p, bad, floored);
+      lam_pair_fast(x[l], old, a.la, p, rare, floored);
       dst[w] = p[0], dst[n + w] = p[1];
     });
+    if (rare) {
+      floored = false;
+#pragma unroll
+      for (int l = 0; l < L; ++l) sm[t + (l << kLOGNT)] = x[l];
+#pragma unroll 1
+      for (int l = 0; l < L; ++l) {
+        const uint32_t w = widx(e_of<T>(LMID, t, l));
+        double p[2];
+        lam_pair(sm[t + (l << kLOGNT)], lr[w], w == 0, a.la, p, bad, floored);
+        dst[w] = p[0], dst[n + w] = p[1];
+      }
+    }
     lam_flags(a.la, bad, floored);
   } else if constexpr (MODE == MID_APPLY) {
     const double fac = 1.0 / (double)n;
@@ -460,7 +521,7 @@ __global__ void __launch_bounds__(kFNT, 3) k_net_mid(T *X, TIO *out, MidArgs a) 
     __shared__ double sh[32];
     const double inv_n = 1.0 / (double)n;
     double quad = 0.0, gs = 0.0;
-    with_lam([&](int l, uint32_t, double lam) { x[l] = (T)mll_g(f2d_exact(x[l]), lam, inv_n, quad, gs); });
+    with_lam([&](int l, uint32_t, double lam) { x[l] = narrow<T>(mll_g(f2d_int(x[l]), lam, inv_n, quad, gs)); });
     if (a.back) xwht_col<T>(x, sm, c, 1 - DF);
 #pragma unroll
     for (int l = 0; l < L; ++l) xv[widx(a.back ? e_of<T>(LIN, t, l) : e_of<T>(LMID, t, l))] = x[l];
@@ -498,8 +559,9 @@ uint32_t net_mll_blocks(uint32_t m, bool fp64) {
 template <typename T, typename TIO, int MODE>
 static int launch_mid(T *X, TIO *out, uint32_t m, uint32_t nvec, MidArgs a, cudaStream_t st) {
   a.m = (int)m, a.c = 2 * FCfg<T>::LOGT - (int)m;
-  smem_optin<k_net_mid<T, TIO, MODE>>(xtile_bytes<T>());
-  k_net_mid<T, TIO, MODE><<<dim3(tiles_of<T>(m), nvec), kFNT, xtile_bytes<T>(), st>>>(X, out, a);
+  constexpr size_t sm = mid_smem<T, MODE>();
+  smem_optin<k_net_mid<T, TIO, MODE>>(sm);
+  k_net_mid<T, TIO, MODE><<<dim3(tiles_of<T>(m), nvec), kFNT, sm, st>>>(X, out, a);
   return check_launch("net transform: high bits");
 }
 template <typename T, typename TIO, bool KEEP = false>
