@@ -190,7 +190,7 @@ __device__ __forceinline__ void grad64_item(const ColJob &job, const typename Gr
         const double K = T.factor(T.word(s0 + i, j));
         const double f = fma(wj, K, 1.0);
         double q;
-        if (!ratio_fast(K, f, q)) {
+        if (!ratio_lean(K, f, q) && !ratio_fast(K, f, q)) {
           if (f == 0.0) {  // the explicit product over the other dimensions; k1 = 0 here
             double dk = job.zeta;
             for (uint32_t jj = 0; jj < d; ++jj) {

@@ -35,6 +35,28 @@ __device__ __forceinline__ double ratio(double a, double b) {
   return ratio_fast(a, b, q) ? q : a / b;
 }
 
+// a / b with three FP64 instructions: the FP32 estimate of 1 / b for b's leading 24 bits and its
+// residual over all of b (about 2^-46 left) become one double r by integer operations, then
+// q0 = a r and its residual, as in Markstein's division: the rounded quotient up to 2^-80 before
+// the last rounding.  The mantissa of 1 / b lies in (1/2, 1); where the correction could carry
+// it over either end (b within 2^-20 of a power of two), or b is outside 2^-100 .. 2^100, false.
+__device__ __forceinline__ bool ratio_lean(double a, double b, double &q) {
+  const uint32_t hi = (uint32_t)__double2hiint(b), lo = (uint32_t)__double2loint(b);
+  const uint32_t ex = (hi >> 20) & 0x7FFu, mt = hi & 0xFFFFFu;
+  if (ex - 923u > 200u || mt - 1u > 0xFFFFDu) return false;
+  const float bh = __uint_as_float(0x3F800000u | (mt << 3) | (lo >> 29));
+  const float bl = __fmul_rn(__uint2float_rn(lo & 0x1FFFFFFFu), 0x1p-52f);
+  const float rm = rcp_approx(bh);  // in (1/2, 1)
+  const float e = __fmaf_rn(-bl, rm, __fmaf_rn(-bh, rm, 1.f));
+  const int32_t dl = __float2int_rn(__fmul_rn(__fmul_rn(e, rm), 0x1p52f));  // units of 2^-52
+  const uint32_t u = __float_as_uint(rm);
+  const uint32_t rh = ((u >> 3) + (896u << 20) - ((ex - 1023u) << 20)) | (hi & 0x80000000u);
+  const double r = __longlong_as_double((long long)((((uint64_t)rh << 32) | (u << 29)) + (uint64_t)((int64_t)dl * 2)));
+  const double q0 = a * r;
+  q = fma(fma(-b, q0, a), r, q0);
+  return true;
+}
+
 // 1 / b as ratio_fast(1, b): one rounding, 3 FP64 instructions.
 __device__ __forceinline__ double rcp64(double b) {
   const uint32_t hi = (uint32_t)__double2hiint(b), lo = (uint32_t)__double2loint(b);
