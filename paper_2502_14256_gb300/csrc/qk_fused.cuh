@@ -819,13 +819,27 @@ __device__ __forceinline__ void fused_B_item(const FTask &ft, uint32_t r, uint32
     } else {
       v = fmadd(zeta, lam[l], eta);
       if (l == 0 && t == 0 && tau == 0) v += zn;  // w = 0 (e = 0 in every layout)
-      if (eta > T(0) && !(v >= eta)) {  // K + eta I has no eigenvalue below eta: rounding
-        v = eta;
-        floored = true;
+      if constexpr (sizeof(T) == 8) {  // K + eta I has no eigenvalue below eta; as integers, the
+        // order of positive doubles: FP64 comparisons take FP64 time, predicated or not
+        const long long b = __double_as_longlong(v), lo = __double_as_longlong(eta);
+        if (lo > 0 && lo <= 0x7FF0000000000000ll && !(b >= lo && b <= 0x7FF0000000000000ll)) {
+          v = eta;
+          floored = true;
+        }
+      } else {
+        if (eta > T(0) && !(v >= eta)) {  // K + eta I has no eigenvalue below eta: rounding
+          v = eta;
+          floored = true;
+        }
       }
       if (LAM) LAM[wi2(l)] = f2d_exact(v);
     }
-    bad |= !(v > T(0));
+    if constexpr (sizeof(T) == 8) {
+      const long long b = __double_as_longlong(v);
+      bad |= !(b > 0 && b <= 0x7FF0000000000000ll);
+    } else {
+      bad |= !(v > T(0));
+    }
     lds.add(v);
     // each thread reads back only its own entries; FP64 (no refinement) needs 1 / lambda alone
     lmv[t + (l << kLOGNT)] = sizeof(T) == 8 ? fused_rcp(v) : v;
@@ -858,11 +872,19 @@ __device__ __forceinline__ void fused_B_item(const FTask &ft, uint32_t r, uint32
       const int e = t + (l << kLOGNT);  // this thread's own entries only
       const T lw = lmv[e];
       const T il = sizeof(T) == 8 ? lw : fused_rcp(lw);
-      const T sc = inv_n * il;          // 1 / (n lambda_w)
+      T sc;                             // 1 / (n lambda_w)
+      if constexpr (sizeof(T) == 8) sc = scale_pow2(il, -(int)ft.job.m);
+      else sc = inv_n * il;
       T ch = y[l] * sc;                 // c^_w = Y_w / (n lambda_w)
       const T a = ch * y[l];            // Y_w^2 / (n lambda_w)
       quad += a;
-      const T gg = T(0.5) * (a - T(1)) * il;
+      T gg;                             // (a - 1) / (2 lambda_w)
+      if constexpr (sizeof(T) == 8) {
+        const T h = scale_pow2(il, -1);
+        gg = fma(a, h, -h);
+      } else {
+        gg = T(0.5) * (a - T(1)) * il;
+      }
       gs += gg;
       if constexpr (COMP) {
         // refinement: the exact residual of the division plus the forward transform's
