@@ -454,8 +454,11 @@ uint32_t grad_blocks(uint32_t m, bool fp64) { return fp64 ? grad64_blocks(m) : c
 
 __global__ void k_ratio_selftest(const double *__restrict__ a, const double *__restrict__ b, double *__restrict__ q,
                                  uint64_t n) {
-  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x)
-    q[i] = ratio(a[i], b[i]);
+  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
+    double v;  // as in the FP64 gradient sweep
+    if (!ratio_lean(a[i], b[i], v)) v = ratio(a[i], b[i]);
+    q[i] = v;
+  }
 }
 
 template <int FAM, int ALPHA>

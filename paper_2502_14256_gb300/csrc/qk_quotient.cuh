@@ -17,7 +17,7 @@ __device__ __forceinline__ float rcp_approx(float a) {
 // from the FP32 reciprocal estimate r of b (its leading 24 bits, relative error e below
 // 2^-22), q0 = a r, then q0 (1 + e + e^2) with e = 1 - b r rounded once: what is left is e^3,
 // below 2^-66, so the result is within 2 ulp of the rounded quotient (checked against the
-// divide by qk_ratio_selftest).  Four FP64 instructions.  False for b outside
+// divide by qk_ratio_selftest, as ratio_lean).  Four FP64 instructions.  False for b outside
 // 2^-100 .. 2^100 in magnitude (zero, subnormal, inf and NaN included).
 __device__ __forceinline__ bool ratio_fast(double a, double b, double &q) {
   const uint32_t hi = (uint32_t)__double2hiint(b), lo = (uint32_t)__double2loint(b);
