@@ -319,16 +319,15 @@ __global__ void __launch_bounds__(sizeof(T) == 8 ? 256 : 512) k_net_mll_small(co
   const double *lr = lam + ((uint64_t)(blockIdx.x / nrhs) << m);
   const double inv_n = 1.0 / (double)n;
   T x[16];
-  float s = 0.f, e = 0.f;  // FP32 data: the sum as a float-float pair
-  double sd = 0.0;
+  double sd = 0.0;  // FP32 data: their sum (one FP64 addition each; the conversion is integer)
 #pragma unroll
   for (int i = 0; i < 16; ++i) {
     const TIO v = t + i * NT < n ? y[off + t + i * NT] : TIO(0);
     x[i] = widen<T>(v);
-    if constexpr (sizeof(TIO) == 4) ff_add(s, e, v);
+    if constexpr (sizeof(TIO) == 4) sd += f2d_int(v);
   }
   small_wht<T, 16>(x, m, smem);
-  if constexpr (sizeof(TIO) == 4) sd = block_sum_c(s, e, sh);
+  if constexpr (sizeof(TIO) == 4) sd = block_sum(sd, sh);
   else sd = x[0];  // element 0 of the transform (thread 0): the sum rounded once
   if (t == 0) ysum[blockIdx.x] = sd;
   double quad = 0.0, gs = 0.0;
@@ -379,18 +378,18 @@ __global__ void __launch_bounds__(kFNT, sizeof(T) == 8 ? 3 : 4) k_net_low_in(con
   const uint64_t base = (uint64_t)blockIdx.x << LOGT;
   const int t = threadIdx.x;
   T v[L];
-  float s = 0.f, e = 0.f;
+  double s = 0.0;
 #pragma unroll
   for (int l = 0; l < L; ++l) {
     const TIO a = in[base + t + (l << kLOGNT)];
     v[l] = widen<T>(a);
     if constexpr (sizeof(TIO) == 4)
-      if (ysum) ff_add(s, e, a);
+      if (ysum) s += f2d_int(a);
   }
   if constexpr (sizeof(TIO) == 4) {
     if (ysum) {
       __shared__ double sh[32];
-      const double sd = block_sum_c(s, e, sh);
+      const double sd = block_sum(s, sh);
       if (t == 0) ysum[blockIdx.x] = sd;
     }
   }

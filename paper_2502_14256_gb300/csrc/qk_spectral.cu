@@ -124,16 +124,9 @@ __global__ void k_sum_rows(const T *__restrict__ y, int m, double *__restrict__ 
   const uint64_t n = 1ull << m, chunk = (n + gridDim.x - 1) / gridDim.x;
   const uint64_t lo = (uint64_t)blockIdx.x * chunk, hi = lo + chunk < n ? lo + chunk : n;
   const T *yv = y + (uint64_t)blockIdx.y * n;
-  double t;
-  if constexpr (sizeof(T) == 4) {  // float-float (about 2^-46): no FP64 instructions per element
-    float s = 0.f, e = 0.f;
-    for (uint64_t i = lo + threadIdx.x; i < hi; i += blockDim.x) ff_merge(s, e, yv[i], 0.f);
-    t = block_sum_c(s, e, sh);
-  } else {
-    double s = 0.0;
-    for (uint64_t i = lo + threadIdx.x; i < hi; i += blockDim.x) s += yv[i];
-    t = block_sum(s, sh);
-  }
+  double s = 0.0;
+  for (uint64_t i = lo + threadIdx.x; i < hi; i += blockDim.x) s += f2d_int(yv[i]);
+  const double t = block_sum(s, sh);
   if (threadIdx.x == 0) out[(uint64_t)blockIdx.y * gridDim.x + blockIdx.x] = t;
 }
 
@@ -397,12 +390,8 @@ __global__ void k_logdet(const double *__restrict__ lam, int m, double *__restri
   double s = 0.0;
   const uint64_t step = (uint64_t)gridDim.x * blockDim.x;
   if (FAST_LOG) {
-    // each logarithm as a float, their sum as a float-float pair (FP64 sums of floats to 2^-46)
-    float fs = 0.f, fe = 0.f;
-    for (uint64_t w = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; w < n; w += step) ff_merge(fs, fe, logf(d2f_int(lr[w])), 0.f);
-    const double t = block_sum_c(fs, fe, sh);
-    if (threadIdx.x == 0) part[(uint64_t)blockIdx.y * gridDim.x + blockIdx.x] = t;
-    return;
+    // each logarithm as a float; the conversions are integer, one FP64 addition each is left
+    for (uint64_t w = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; w < n; w += step) s += f2d_int(logf(d2f_int(lr[w])));
   } else {
     double prod = 1.0;
     long long ex = 0;
