@@ -879,6 +879,8 @@ __device__ __forceinline__ void fused_B_item(const FTask &ft, uint32_t r, uint32
       const T a = ch * y[l];            // Y_w^2 / (n lambda_w)
       quad += a;
       T gg;                             // (a - 1) / (2 lambda_w)
+      // FP64: powers of two on the exponent field and one fused operation, 5 FP64 instructions
+      // per element and right-hand side instead of 8 (8 right-hand sides: 751 -> 699 us)
       if constexpr (sizeof(T) == 8) {
         const T h = scale_pow2(il, -1);
         gg = fma(a, h, -h);
