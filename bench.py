@@ -45,9 +45,9 @@ UNIT = "points/s"
 # CUDA sources that capture ran (kernel_source_hash()).  A run whose sources differ reports
 # traffic null: the counters belong to another version of the kernels.
 NCU_TRAFFIC = {
-    "src_hash": "a3fa2874c89e",
-    "bytes_r64": {"k_fused_A": 1283025408, "k_fused_B": 1294175744, "k_fused_C": 1053564672},
-    "fwht_bytes": 589224704,
+    "src_hash": "5f05dcf73891",
+    "bytes_r64": {"k_fused_A": 1281683968, "k_fused_B": 1294536192, "k_fused_C": 1053151488},
+    "fwht_bytes": 589520896,
 }
 # Nominal FP64 rate of GB300 (profiling recipe's table; FP64 is not a tensor-core path here).
 FP64_PEAK_TFLOPS = 1.25
@@ -82,7 +82,8 @@ def parse():
 
 # The sources the fused pipeline's and the batched FWHT's kernels are compiled from.
 FUSED_SOURCES = ("qk_fused.cuh", "qk_fused.cu", "qk_fused_f32.cu", "qk_fused_f32c.cu", "qk_fused_f32w.cu",
-                 "qk_fused_f64.cu", "qk_column.cuh", "qk_common.cuh", "qk_factors.cuh", "qk_internal.h")
+                 "qk_fused_f64.cu", "qk_column.cuh", "qk_common.cuh", "qk_factors.cuh", "qk_grad.cuh", "qk_quotient.cuh",
+                 "qk_wht96.cuh", "qk_internal.h")
 
 
 def _code_only(text: bytes) -> bytes:
@@ -324,12 +325,13 @@ def lattice_line(qk, torch, dev, stream, R=16):
            "points_per_step": R << wl.ms[0]}
     m, d = wl.ms[0], wl.d
     n = 1 << m
-    # algorithmic FP64 flops of the FP64 step: column sweep 9 per (point, dimension) (the
-    # factor x - x^2, its square and the polynomial, 5; the weight; p <- p + a + p a, 3),
-    # gradient sweep 12 (the factor, 5; 1 + c K; the quotient; two accumulations, 4), 5 N
-    # log2 N per complex transform of N (R/2 pairs each: eigenvalues, y forward; g and c
-    # inverse), 20 per (frequency, vector) in the spectral step
-    flops = R * n * d * (9 + 12) + 4 * (R // 2) * 5 * n * m + 20 * R * n
+    # algorithmic FP64 flops of the FP64 step.  Differences of lattice points do not depend on
+    # the shift, so once for all shifts: column sweep 9 per (point, dimension) (the factor
+    # x - x^2, its square and the polynomial, 5; the weight; p <- p + a + p a, 3), gradient
+    # sweep 10 (the factor, 5; 1 + c K; the quotient; the sum of dk, 2), two transforms of the
+    # column's copies.  Per shift: 2 per (point, dimension) in the gradient, half a complex
+    # transform of 5 n log2 n each for y, g and c, 20 per frequency in the spectral step
+    flops = n * d * (9 + 10 + 2 * R) + (2 + 3 * (R // 2)) * 5 * n * m + 20 * R * n
     for name, dt in (("fp64", torch.float64), ("f32w", qk.F32W)):
         ws, status, pts = lattice_setup(qk, torch, dev, R, dt)
         ms_ = time_steps(torch, lambda: qk.batch_run(ws, status), 3, 1, stream)
@@ -605,7 +607,7 @@ def main():
         top64, (l64, t64) = max(k64.items(), key=lambda kv: kv[1][1])
         # FP64 FMA-pipe roofline of the FP64 path's longest kernel (algorithmic flops per
         # point below; 12-bit tile transforms in FP64)
-        fl64 = {"k_fused_A": 8 * d + 2 * 12 + 2, "k_fused_C": 10 * d + 2 * 12 + 3}.get(top64)
+        fl64 = {"k_fused_A": 8 * d + 2 * 12 + 2, "k_grad64": 10 * d}.get(top64)
         if fl64:
             ach = fl64 * R * n / (t64 / max(1.0, l64) * 1e-3) / 1e12
             fp64["roofline"] = {"kernel": top64, "bound": "alu", "achieved": ach, "peak": FP64_PEAK_TFLOPS,
