@@ -320,11 +320,19 @@ static int launch_integrand(const qk_pointset *ps, uint32_t r0, uint32_t nr, uin
 // 14 us for 10 rows of 2^15 doubles; rows are many times longer than a CTA.
 constexpr int kRowCta = 8, kRowNT = 512;
 
+// Every thread of every CTA of the cluster calls both (release on arrival, acquire on return).
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait;" ::: "memory"); }
+
 // FP64 sum over this cluster's row of f(i) for i < n; valid in thread 0 of the cluster's rank 0.
+// Another CTA's shared memory exists once that CTA has started: each arrives at the cluster's
+// barrier first thing and waits before its store, so the row's loads hide the wait (a CTA of
+// rank k has no element of a row shorter than 512 k and would store at once).
 template <typename F>
 __device__ __forceinline__ double cluster_row_sum(uint64_t n, F f) {
   __shared__ double sh[32];
   __shared__ double part[kRowCta];
+  cluster_arrive();
   uint32_t rank;
   asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
   double s0 = 0.0, s1 = 0.0;
@@ -333,13 +341,15 @@ __device__ __forceinline__ double cluster_row_sum(uint64_t n, F f) {
   for (; i + step < n; i += 2 * step) s0 += f(i), s1 += f(i + step);
   if (i < n) s0 += f(i);
   const double s = block_sum(s0 + s1, sh);
+  cluster_wait();
   if (threadIdx.x == 0) {
     uint32_t local = (uint32_t)__cvta_generic_to_shared(&part[rank]), remote;
     asm("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(remote) : "r"(local));
     asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(remote), "d"(s) : "memory");
   }
-  // every CTA of the cluster arrives and waits: the parts are in place, no CTA has left before
-  asm volatile("barrier.cluster.arrive.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
+  // the parts are in place, and no CTA has left before
+  cluster_arrive();
+  cluster_wait();
   double tot = 0.0;
   if (rank == 0 && threadIdx.x == 0)
     for (int k = 0; k < kRowCta; ++k) tot += part[k];
