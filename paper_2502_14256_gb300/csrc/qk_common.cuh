@@ -28,13 +28,15 @@ inline unsigned ceil_div_u(uint64_t a, uint64_t b) { return (unsigned)((a + b - 
 // Multiprocessors of the current device (queried once per device, cached).
 int sm_count();
 
-// Opt a kernel into more than 48 KB of dynamic shared memory, once per process
-// and kernel (the call is skipped entirely below 48 KB, so launches that need
-// no opt-in issue no extra runtime call, e.g. inside CUDA-graph capture).
+// Opt a kernel into more than 48 KB of shared memory, once per process and kernel.  The limit
+// holds for static and dynamic shared memory together, so the opt-in starts below it, at a
+// static part that no kernel here exceeds (launches that need less issue no extra runtime call,
+// e.g. inside CUDA-graph capture).
+constexpr size_t kSmemDefault = 48 * 1024, kSmemStaticMax = 4 * 1024;
 template <auto FN>
 inline void smem_optin(size_t bytes) {
   static size_t done = 0;  // one counter per kernel (FN is the kernel itself)
-  if (bytes <= 48 * 1024 || bytes <= done) return;
+  if (bytes <= kSmemDefault - kSmemStaticMax || bytes <= done) return;
   cudaFuncSetAttribute(FN, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   done = bytes;
 }
