@@ -21,7 +21,7 @@ from . import qk
 class BayesCubatureMLL(torch.autograd.Function):
     """Returns (mll, post_mean), each of shape (nr, nrhs), for randomizations r0 .. r0+nr-1.
 
-    forward(gamma (d,), log_ls (d,), log_eta (), y (nr, nrhs, n), spec) with spec a
+    forward(gamma (d,), log_ls (d,), log_eta () or one element, y (nr, nrhs, n), spec) with spec a
     tuple (ps, family, alpha, zeta, m, r0); gamma, log_ls, log_eta FP64 device tensors;
     y in the computation dtype (FP64 or FP32).  y is data: no gradient flows to it.
     """
@@ -50,7 +50,7 @@ class BayesCubatureMLL(torch.autograd.Function):
         qk.read_status(status)
         if want_grad:
             ctx.save_for_backward(grad, c, ls)
-        ctx.d, ctx.eta = d, eta
+        ctx.d, ctx.eta, ctx.eta_shape = d, eta, log_eta.shape
         return out[..., qk.QK_MLL_MLL].clone(), out[..., qk.QK_MLL_MEAN].clone()
 
     @staticmethod
@@ -67,7 +67,7 @@ class BayesCubatureMLL(torch.autograd.Function):
             total = torch.zeros_like(grad[..., :d + 1])
         total = total.sum(dim=(0, 1))
         dc = total[:d]
-        return dc * ls, dc * c, total[d] * ctx.eta, None, None
+        return dc * ls, dc * c, (total[d] * ctx.eta).reshape(ctx.eta_shape), None, None
 
 
 def mll_and_mean(gamma, log_ls, log_eta, y, ps, family: int, alpha: int, m: int, zeta: float = 1.0, r0: int = 0):
