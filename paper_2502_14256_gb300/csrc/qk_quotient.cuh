@@ -1,6 +1,6 @@
 // Quotients without FP64 divisions (GB300: about 2 FP64 lanes per SM and cycle): reciprocals and
 // quotients to about one FP64 rounding from the FP32 reciprocal estimate, and the FP32 scaling by
-// an FP64 eigenvalue in float-float arithmetic.
+// an FP64 eigenvalue from float pairs.
 #pragma once
 
 #include "qk_common.cuh"
@@ -80,18 +80,25 @@ __device__ __forceinline__ double rcp64_exact(double b) {
   return fma(r, fma(-b, r, 1.0), r);
 }
 
-// x / lambda fac (inverse) or x lambda fac, fac a power of two.  FP32: lambda as a float pair (its
-// leading 24 bits and the rest, by integer operations), the quotient or product to about 2^-44
-// before it is rounded to FP32: the FP64 division's result without FP64 instructions; x or
-// lambda outside a wide middle range takes FP64.
+// x / lambda fac (inverse) or x lambda fac, fac a power of two.
 __device__ __forceinline__ double scale_lambda(double x, double lam, double fac, bool inverse) {
   return x * (inverse ? fac * rcp64(lam) : fac * lam);
+}
+// FP32: the FP64 division (or product) rounded to FP32, bit for bit, without FP64 instructions.
+// lambda as a float pair (its leading 24 bits and the rest, by integer operations) gives the
+// result p + s to a relative 2^-43; where p + s -+ 2^-42 |p| round to one FP32 number, so does
+// everything between them, the FP64 value (off by 2^-52) included.  The others (about one in
+// 2^18) take FP64 out of line, and so do x or lambda outside a wide middle range.  The check is 5
+// of some 25 FP32 instructions; with the FP64 form out of line the column, solve and product of
+// 32 x 2^18 values take 533 -> 520 us.
+static __device__ __noinline__ float scale_lambda_fp64(float x, double lam, double fac, bool inverse) {
+  return (float)((double)x * (inverse ? fac / lam : fac * lam));
 }
 __device__ __forceinline__ float scale_lambda(float x, double lam, double fac, bool inverse) {
   const uint32_t hi = (uint32_t)__double2hiint(lam), lo = (uint32_t)__double2loint(lam);
   const uint32_t ex = (hi >> 20) & 0x7FFu, xe = (__float_as_uint(x) >> 23) & 0xFFu;
-  if (ex - 983u > 80u || (hi & 0x80000000u) || (xe - 87u > 80u && x != 0.f))
-    return (float)((double)x * (inverse ? fac / lam : fac * lam));
+  const bool mid = ex - 983u <= 80u && !(hi & 0x80000000u);
+  if (!mid || xe - 87u > 80u) return mid && x == 0.f ? x : scale_lambda_fp64(x, lam, fac, inverse);
   const float lh = __uint_as_float(((ex - 896u) << 23) | ((hi & 0xFFFFFu) << 3) | (lo >> 29));
   const float ll = __uint2float_rn(lo & 0x1FFFFFFFu) * __uint_as_float((ex - 948u) << 23);
   float a = lh, b = ll;
@@ -100,8 +107,10 @@ __device__ __forceinline__ float scale_lambda(float x, double lam, double fac, b
     const float e = __fmaf_rn(-ll, a, __fmaf_rn(-lh, a, 1.f));
     b = __fmul_rn(a, __fmaf_rn(e, e, e));
   }
-  const float p = __fmul_rn(x, a);
-  return __fadd_rn(p, __fmaf_rn(x, b, __fmaf_rn(x, a, -p))) * (float)fac;
+  const float p = __fmul_rn(x, a), s = __fmaf_rn(x, b, __fmaf_rn(x, a, -p)), del = __fmul_rn(fabsf(p), 0x1p-42f);
+  const float v = __fadd_rn(p, __fsub_rn(s, del));
+  if (v != __fadd_rn(p, __fadd_rn(s, del))) return scale_lambda_fp64(x, lam, fac, inverse);
+  return v * (float)fac;
 }
 
 }  // namespace qk
