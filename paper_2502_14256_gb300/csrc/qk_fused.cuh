@@ -609,14 +609,14 @@ __device__ __forceinline__ void xwht_col2(T (&vh)[FCfg<T>::L], T (&vl)[FCfg<T>::
 
 // log lambda for the log-determinant: FP32 tiles take the hardware log2 approximation
 // (absolute error ~2^-22 per term, about 1e-8 relative on a log det summed over 2^20
-// eigenvalues even if every term erred the same way; the sum itself is FP64).  1 / lambda: the
-// reciprocal estimate plus one Newton step (within 1 ulp); the solve's exact-residual
-// correction below absorbs it.
+// eigenvalues even if every term erred the same way; the sum itself is FP64).  1 / lambda: FP32
+// tiles take the reciprocal estimate plus one Newton step (within 1 ulp; the solve's
+// exact-residual correction below absorbs it), FP64 tiles the rounded reciprocal.
 __device__ __forceinline__ float fused_rcp(float v) {
   const float r = rcp_approx(v);
   return fmaf(fmaf(-v, r, 1.f), r, r);
 }
-__device__ __forceinline__ double fused_rcp(double v) { return rcp64(v); }
+__device__ __forceinline__ double fused_rcp(double v) { return rcp64_exact(v); }
 // Sum of logs of a thread's eigenvalues.  FP64: the log of the product of the mantissas (16
 // factors below 2) and the sum of the exponents: one multiplication per eigenvalue and one log
 // per thread, where a log is some 30 FP64 instructions; eigenvalues that are not positive normal

@@ -90,7 +90,8 @@ __device__ __forceinline__ TIO narrow(T v) {
 
 // MLL spectral step of one frequency: adds to the quadratic form and to sum g, returns g.
 __device__ __forceinline__ double mll_g(double Y, double lam, double inv_n, double &quad, double &gs) {
-  const double il = rcp64(lam), a = Y * Y * (inv_n * il), h = 0.5 * il, g = fma(a, h, -h);
+  double a;
+  const double g = mll_step(Y * Y, inv_n, lam, a);
   quad += a;
   gs += g;
   return g;

@@ -57,32 +57,66 @@ __device__ __forceinline__ bool ratio_lean(double a, double b, double &q) {
   return true;
 }
 
-// 1 / b as ratio_fast(1, b): one rounding, 3 FP64 instructions.
-__device__ __forceinline__ double rcp64(double b) {
-  const uint32_t hi = (uint32_t)__double2hiint(b), lo = (uint32_t)__double2loint(b);
-  const uint32_t ex = (hi >> 20) & 0x7FFu;
-  if (ex - 923u > 200u) return 1.0 / b;
+// The divide, out of line: predicated FP64 instructions take FP64 time.
+static __device__ __noinline__ double divide_rare(double a, double b) { return a / b; }
+
+// 1 / b for b in 2^-100 .. 2^100 as ratio_fast(1, b): one rounding, 3 FP64 instructions.
+__device__ __forceinline__ double rcp64_mid(uint32_t hi, uint32_t lo, uint32_t ex) {
   const uint32_t fb = (hi & 0x80000000u) | ((ex - 896u) << 23) | ((hi & 0xFFFFFu) << 3) | (lo >> 29);
-  const double r = f2d_exact(rcp_approx(__uint_as_float(fb)));
-  const double e = fma(-b, r, 1.0);
+  const double r = f2d_normal(rcp_approx(__uint_as_float(fb)));
+  const double e = fma(-__hiloint2double((int)hi, (int)lo), r, 1.0);
   return fma(r, fma(e, e, e), r);
+}
+__device__ __forceinline__ double rcp64(double b) {
+  const uint32_t hi = (uint32_t)__double2hiint(b), ex = (hi >> 20) & 0x7FFu;
+  if (ex - 923u > 200u) return divide_rare(1.0, b);
+  return rcp64_mid(hi, (uint32_t)__double2loint(b), ex);
 }
 
 // 1 / b correctly rounded: one more Newton step, whose residual is exact and whose last operation
-// is one rounding (Markstein 1990: correct unless b's mantissa is all ones, which takes the
-// divide).  For the lattices' spectral step, where sums over cancelling terms near a small
-// nugget show the last bit.
-__device__ __forceinline__ double rcp64_exact(double b) {
+// is one rounding (Markstein 1990: correct unless b's mantissa is all ones).  5 FP64
+// instructions.  False for that mantissa and for b outside 2^-100 .. 2^100: take the divide.
+__device__ __forceinline__ bool rcp64_rounded(double b, double &r) {
   const uint32_t hi = (uint32_t)__double2hiint(b), lo = (uint32_t)__double2loint(b);
   const uint32_t ex = (hi >> 20) & 0x7FFu;
-  if (ex - 923u > 200u || ((hi & 0xFFFFFu) == 0xFFFFFu && lo == 0xFFFFFFFFu)) return 1.0 / b;
-  const double r = rcp64(b);
-  return fma(r, fma(-b, r, 1.0), r);
+  if (ex - 923u > 200u || ((hi & 0xFFFFFu) == 0xFFFFFu && lo == 0xFFFFFFFFu)) return false;
+  const double r0 = rcp64_mid(hi, lo, ex);
+  r = fma(r0, fma(-b, r0, 1.0), r0);
+  return true;
+}
+__device__ __forceinline__ double rcp64_exact(double b) {
+  double r;
+  return rcp64_rounded(b, r) ? r : divide_rare(1.0, b);
+}
+// v fac, fac a power of two, by the exponent field: v and the product normal.
+__device__ __forceinline__ double times_pow2(double v, double fac) {
+  return __hiloint2double(__double2hiint(v) + (__double2hiint(fac) - 0x3FF00000), __double2loint(v));
+}
+// fac / b, fac a power of two in 2^-64 .. 1, correctly rounded.
+__device__ __forceinline__ double pow2_over(double fac, double b) {
+  double r;
+  return rcp64_rounded(b, r) ? times_pow2(r, fac) : divide_rare(fac, b);
+}
+
+// The MLL's step at one frequency, from |Y|^2, 1 / n and lambda: a = |Y|^2 / (n lambda) by the
+// rounded reciprocal and one correction (the rounded quotient, as the divide gives it; 2 FP64
+// instructions more than a product with the reciprocal, which is off by one more rounding),
+// returns g = (a - 1) / (2 lambda).  The divides where lambda has no rounded reciprocal or the
+// quotient's residual could underflow or overflow.
+__device__ __forceinline__ double mll_step(double y2, double inv_n, double lam, double &a) {
+  double r;
+  if (((uint32_t)__double2hiint(y2) >> 20) - 400u > 1300u || !rcp64_rounded(lam, r)) {
+    a = divide_rare(y2 * inv_n, lam);
+    return divide_rare(0.5 * (a - 1.0), lam);
+  }
+  const double z = times_pow2(y2, inv_n), q = z * r, h = times_pow2(r, 0.5);
+  a = fma(fma(-lam, q, z), r, q);
+  return fma(a, h, -h);
 }
 
 // x / lambda fac (inverse) or x lambda fac, fac a power of two.
 __device__ __forceinline__ double scale_lambda(double x, double lam, double fac, bool inverse) {
-  return x * (inverse ? fac * rcp64(lam) : fac * lam);
+  return x * (inverse ? pow2_over(fac, lam) : fac * lam);
 }
 // FP32: the FP64 division (or product) rounded to FP32, bit for bit, without FP64 instructions.
 // lambda as a float pair (its leading 24 bits and the rest, by integer operations) gives the

@@ -143,10 +143,9 @@ __global__ void k_mll_spectral(E *__restrict__ X, const double *__restrict__ lam
   const double inv_n = 1.0 / (double)n;
   for (uint64_t w = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; w < n; w += (uint64_t)gridDim.x * blockDim.x) {
     const E Y = xv[w];
-    const double l = lr[w];
-    const double il = rcp64(l), a = abs2(Y) * (inv_n * il);
+    double a;
+    const double g = mll_step(abs2(Y), inv_n, lr[w], a);
     q += a;
-    const double g = (0.5 * (a - 1.0)) * il;
     gs += g;
     xv[w] = from_real<E>(g);
   }
@@ -276,8 +275,8 @@ __global__ void k_scale_pairs(E *__restrict__ X, const double *__restrict__ lam,
     for (int h = 0; h < 2; ++h) {
       const uint64_t v = 2 * q + h < nvec ? 2 * q + h : 2 * q;  // an absent half scales a zero
       const double *lr = lam + ((v / nrhs) << m);
-      sk[h] = fac * (mode == 0 ? rcp64_exact(lr[k]) : lr[k]);
-      skk[h] = fac * (mode == 0 ? rcp64_exact(lr[kk]) : lr[kk]);
+      sk[h] = mode == 0 ? pow2_over(fac, lr[k]) : fac * lr[k];
+      skk[h] = mode == 0 ? pow2_over(fac, lr[kk]) : fac * lr[kk];
     }
     const double2 ck = make_double2(a.x * sk[0], a.y * sk[0]), dk = make_double2(b.x * sk[1], b.y * sk[1]);
     const double2 ckk = make_double2(a.x * skk[0], -a.y * skk[0]), dkk = make_double2(b.x * skk[1], -b.y * skk[1]);
