@@ -105,11 +105,11 @@ template <typename T> struct Lay {
   static constexpr int VEC = 16 / sizeof(T);   // elements per 128-bit access
 };
 // FP32: the padded tile.  FP64: three planes of 32-bit words (the 96-bit butterflies below,
-// kW96Plane words each) and 8 words of scratch; the FP64 tile of the fallback fits in them.
+// kW96Plane words each) and 16 words of scratch; the FP64 tile of the fallback fits in them.
 constexpr int kW96Plane = 4096 + 4 * (4096 / 32) + 16 * (4096 / 256);
 template <typename T>
 __host__ __device__ constexpr size_t xtile_bytes() {
-  return sizeof(T) == 8 ? (size_t)(3 * kW96Plane + 8) * sizeof(uint32_t)
+  return sizeof(T) == 8 ? (size_t)(3 * kW96Plane + 16) * sizeof(uint32_t)
                         : (size_t)((1 << FCfg<T>::LOGT) + Lay<T>::PADE * ((1 << FCfg<T>::LOGT) >> FCfg<T>::LOGL)) * sizeof(T);
 }
 template <typename T>
@@ -328,28 +328,12 @@ __device__ __forceinline__ void w96_stages(I96 (&x)[16], int bit0, int lo, int h
     }
 }
 
-// Tile values into integers over the tile's largest exponent E; false: take the FP64 path.
-// Every thread of the CTA calls it (one barrier).
-__device__ __forceinline__ bool w96_load(const double (&v)[16], I96 (&x)[16], uint32_t *sm, uint32_t &E) {
-  uint32_t hm = 0;
-#pragma unroll
-  for (int l = 0; l < 16; ++l) {
-    const uint32_t h = (uint32_t)__double2hiint(v[l]) & 0x7FFFFFFFu;
-    hm = h > hm ? h : hm;
-  }
-  E = block_max_exp(hm, sm + 3 * kW96Plane);
-  if (E < kW96MinExp || E > kW96MaxExp) return false;
-#pragma unroll
-  for (int l = 0; l < 16; ++l) x[l] = i96_from(v[l], E);
-  return true;
-}
-
-// The tile's sum, in integers and rounded once (FP64 compensated sums outside their exponent
-// range); valid in thread 0.  sm: the transform tile.
+// The tile's sum, in integers and rounded once (FP64 compensated sums where integers could lose
+// a bit); valid in thread 0.  sm: the transform tile.
 __device__ __forceinline__ double w96_sum(const double (&v)[16], uint32_t *sm) {
-  I96 x[16];
-  uint32_t E;
-  if (!w96_load(v, x, sm, E)) {
+  uint32_t far;
+  const uint32_t E = w96_exponent(v, [](int) { return true; }, sm + 3 * kW96Plane, far);
+  if (!E) {
     double s = 0.0, e = 0.0;
 #pragma unroll
     for (int l = 0; l < 16; ++l) ff_add(s, e, v[l]);
@@ -357,6 +341,9 @@ __device__ __forceinline__ double w96_sum(const double (&v)[16], uint32_t *sm) {
     __syncthreads();
     return r;
   }
+  I96 x[16];
+#pragma unroll
+  for (int l = 0; l < 16; ++l) x[l] = i96_from(v[l], E);
 #pragma unroll
   for (int l = 1; l < 16; ++l) x[0] = i96_add(x[0], x[l]);
 #pragma unroll
@@ -427,32 +414,9 @@ __device__ __forceinline__ void xwht_col_fp(T (&v)[FCfg<T>::L], T *sm, int c, in
   }
 }
 
-// The FP64 butterflies of a tile outside the integer path's exponent range (out of line: rare).
-static __device__ __noinline__ void xwht64_rare(double *v, double *sm, int c, int dir) {
-  double x[16];
-#pragma unroll
-  for (int l = 0; l < 16; ++l) x[l] = v[l];
-  if (c == 0) xwht_full_fp<double>(x, sm, dir);
-  else xwht_col_fp<double>(x, sm, c, dir);
-#pragma unroll
-  for (int l = 0; l < 16; ++l) v[l] = x[l];
-}
-
-// Full tile WHT (bits [0, LOGT)) from L0 to L2 (dir 0) or from L2 to L0 (dir 1), and
-// column-tile WHT (bits [c, LOGT)); FP64 tiles in 96-bit integers.
-__device__ __forceinline__ void xwht64(double (&v)[16], double *smd, int c, int dir) {
-  uint32_t *sm = reinterpret_cast<uint32_t *>(smd);
-  I96 x[16];
-  uint32_t E;
-  if (!w96_load(v, x, sm, E)) {
-    double tmp[16];
-#pragma unroll
-    for (int l = 0; l < 16; ++l) tmp[l] = v[l];
-    xwht64_rare(tmp, smd, c, dir);
-#pragma unroll
-    for (int l = 0; l < 16; ++l) v[l] = tmp[l];
-    return;
-  }
+// Full tile WHT (bits [0, LOGT), c = 0) from L0 to L2 (dir 0) or from L2 to L0 (dir 1), and
+// column-tile WHT (bits [c, LOGT)), in 96-bit integers.
+__device__ __forceinline__ void w96_wht(I96 (&x)[16], uint32_t *sm, int c, int dir) {
   if (c == 0) {
     if (dir == 0) {
       w96_stages(x, 8, 8, 12);
@@ -476,6 +440,60 @@ __device__ __forceinline__ void xwht64(double (&v)[16], double *smd, int c, int 
     w96_xpose<2, 0>(x, sm);
     w96_stages(x, 8, c, 12);
   }
+}
+
+// A tile whose values reach so far below 2^E that some may lose bits, or that has no integers
+// (E = 0): integers if none does, else FP64 butterflies, bits upwards as in the multi-pass
+// transform.  Out of line: rare (the look at every value inline: phase B of 8 right-hand sides 699
+// -> 737 us; here 721, of which 22 are the launches' tails behind an FP64 tile).
+static __device__ __noinline__ void xwht64_rare(double *vp, double *smd, int c, int dir, uint32_t E) {
+  double v[16];
+  bool cut = !E;
+#pragma unroll
+  for (int l = 0; l < 16; ++l) v[l] = vp[l], cut |= i96_cut(v[l], E);
+  if (!__syncthreads_or(cut)) {
+    I96 x[16];
+#pragma unroll
+    for (int l = 0; l < 16; ++l) x[l] = i96_from(v[l], E);
+    w96_wht(x, reinterpret_cast<uint32_t *>(smd), c, dir);
+#pragma unroll
+    for (int l = 0; l < 16; ++l) vp[l] = i96_to(x[l], E);
+    return;
+  }
+  if (c == 0) {
+    if (dir == 0) xpose<double>(v, smd, 0, 1);
+    else xpose<double>(v, smd, 2, 1);
+    reg_stages<double>(v, 0, 0, 4);
+    xpose<double>(v, smd, 1, 2);
+  } else if (dir == 0 && c < 8) {
+    xpose<double>(v, smd, 0, 2);
+  }
+  if (c < 8) reg_stages<double>(v, 4, c, 8);
+  if (c < 8 || dir) xpose<double>(v, smd, 2, 0);
+  reg_stages<double>(v, 8, c, 12);
+  if (dir == 0) xpose<double>(v, smd, 0, 2);
+#pragma unroll
+  for (int l = 0; l < 16; ++l) vp[l] = v[l];
+}
+
+// The same transform of FP64 values, in integers.
+__device__ __forceinline__ void xwht64(double (&v)[16], double *smd, int c, int dir) {
+  uint32_t *sm = reinterpret_cast<uint32_t *>(smd);
+  uint32_t far;
+  const uint32_t E = w96_exponent(v, [](int) { return true; }, sm + 3 * kW96Plane, far);
+  if (!E) {
+    double tmp[16];
+#pragma unroll
+    for (int l = 0; l < 16; ++l) tmp[l] = v[l];
+    xwht64_rare(tmp, smd, c, dir, far);
+#pragma unroll
+    for (int l = 0; l < 16; ++l) v[l] = tmp[l];
+    return;
+  }
+  I96 x[16];
+#pragma unroll
+  for (int l = 0; l < 16; ++l) x[l] = i96_from(v[l], E);
+  w96_wht(x, sm, c, dir);
 #pragma unroll
   for (int l = 0; l < 16; ++l) v[l] = i96_to(x[l], E);
 }

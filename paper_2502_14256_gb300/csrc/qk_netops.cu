@@ -185,16 +185,10 @@ __device__ __forceinline__ void small_wht(T (&x)[PER], int m, unsigned char *sme
     }
     __syncthreads();
   } else {
-    __shared__ uint32_t red[8];
-    uint32_t hm = 0;
-#pragma unroll
-    for (int i = 0; i < PER; ++i)
-      if (t + i * NT < n) {
-        const uint32_t h = (uint32_t)__double2hiint(x[i]) & 0x7FFFFFFFu;
-        hm = h > hm ? h : hm;
-      }
-    const uint32_t E = KEEP ? 0u : block_max_exp(hm, red);
-    if (E >= kW96MinExp && E <= kW96MaxExp) {
+    __shared__ uint32_t red[16];
+    uint32_t E = 0, far;
+    if constexpr (!KEEP) E = w96_exponent(x, [&](int i) { return t + i * NT < n; }, red, far);
+    if (E) {
       I96 *sm = reinterpret_cast<I96 *>(smem);
 #pragma unroll
       for (int i = 0; i < PER; ++i) {
