@@ -221,11 +221,25 @@ __device__ __forceinline__ void grad64_item(const ColJob &job, const typename Gr
     red[(NV * G + grp) * d + j] = s1;
   }
   __syncthreads();
+  // The G = 256 / d groups' sums in pairs, eight at a time into two chains: one chain over all of
+  // them was up to twice as far from the exact sum (d = 4, G = 64) and a dependent addition per
+  // group; pairs through shared memory, a barrier per level, cost 2 % at 8 vectors and d = 16.
+  auto eight = [&](const double *r, uint32_t g0) {
+    double x[8];
+#pragma unroll
+    for (uint32_t k = 0; k < 8; ++k) x[k] = g0 + k < G ? r[(g0 + k) * d] : 0.0;
+    return ((x[0] + x[1]) + (x[2] + x[3])) + ((x[4] + x[5]) + (x[6] + x[7]));
+  };
   for (uint32_t q = t; q < (NV + 1) * d; q += kGradNT) {
     const uint32_t v = q / d, jj = q - v * d;
     if (v < (uint32_t)NV && v >= nva) continue;
-    double s = 0.0;
-    for (uint32_t g = 0; g < G; ++g) s += red[(v * G + g) * d + jj];
+    const double *r = red + v * G * d + jj;
+    double s0 = eight(r, 0), s1 = G > 8 ? eight(r, 8) : 0.0;
+    for (uint32_t g = 16; g < G; g += 16) {
+      s0 += eight(r, g);
+      if (g + 8 < G) s1 += eight(r, g + 8);
+    }
+    const double s = s0 + s1;
     if (v < (uint32_t)NV) dst[v * dstride + jj] = s;
     else
       for (uint32_t x = 0; x < nva; ++x) dst[x * dstride + d + jj] = s;

@@ -479,10 +479,15 @@ __global__ void __launch_bounds__(kFinNT) k_mll_final(FinalArgs a) {
   gsh[t] = s0 + s1;
   __syncthreads();
   if (t < (uint32_t)kFinQ && q < nq2) {
-    double tot = 0.0;
-    for (uint32_t k = 0; k < NG; ++k) tot += gsh[k * kFinQ + t];
-    if (q < a.d) g[q] = tot;
-    else g[a.d + 1 + (q - a.d)] = mfac * tot;
+    double x[NG];
+#pragma unroll
+    for (uint32_t k = 0; k < NG; ++k) x[k] = gsh[k * kFinQ + t];
+#pragma unroll
+    for (uint32_t h = NG / 2; h; h >>= 1)  // in pairs, as in the sweep
+#pragma unroll
+      for (uint32_t k = 0; k < h; ++k) x[k] += x[k + h];
+    if (q < a.d) g[q] = x[0];
+    else g[a.d + 1 + (q - a.d)] = mfac * x[0];
   }
 }
 
