@@ -55,15 +55,8 @@ __device__ __forceinline__ double exp2neg(double, int e) {
   return __longlong_as_double((long long)(1023 - e) << 52);
 }
 
-// x = Z 2^-32 as T.  FP32: correctly rounded conversion.  FP64: exact, built as
-// (1 + Z 2^-32) from the mantissa bits minus 1 (one add; GB300 converts u32 to
-// f64 on its slow FP64 pipe at half the add rate).
-__device__ __forceinline__ float word_to_unit(float, uint32_t Z) {
-  return __uint2float_rn(Z) * 0x1p-32f;
-}
-__device__ __forceinline__ double word_to_unit(double, uint32_t Z) {
-  return __hiloint2double((int)(0x3FF00000u | (Z >> 12)), (int)(Z << 20)) - 1.0;
-}
+// x = Z 2^-32 as FP32, rounded to nearest.
+__device__ __forceinline__ float word_to_unit(uint32_t Z) { return __uint2float_rn(Z) * 0x1p-32f; }
 
 // Sum of v over the CTA (blockDim.x a multiple of 32, at most 1024); the result is
 // valid in thread 0.  sh: 32 doubles of shared scratch.  All threads must call it.
@@ -88,7 +81,7 @@ __device__ __forceinline__ void two_sum(T a, T b, T &s, T &e) {
   e = (a - (s - bb)) + (b - bb);
 }
 
-// Float-float ("compensated") sums.  On GB300 an FP64 add costs about 40 FP32 adds, so
+// Float-float ("compensated") sums.  On GB300 an FP64 add takes the time of some 57 FP32 adds, so
 // FP32 reductions keep their partial sums as unevaluated pairs s + e (about 48 bits)
 // and convert to FP64 once, at the end.
 __device__ __forceinline__ void ff_merge(float &s, float &e, float s2, float e2) {

@@ -1,5 +1,5 @@
-// One-dimensional kernel factors K_alpha evaluated from 32-bit words, in T =
-// float or double, and the product-minus-one recurrence for the first column.
+// One-dimensional kernel factors K_alpha of 32-bit words (SI here; DSI as coefficient rows in
+// qk_column.cuh) and the product-minus-one recurrence for the first column.
 //
 // DSI (arXiv 2502.14256, Sec. 5.3, Theorem; x = Z 2^-32, beta(x) = -floor(log2 x),
 // t_nu = 2^(-nu beta), beta(0) = t_nu(0) = 0):
@@ -21,16 +21,13 @@
 
 namespace qk {
 
-// Exact small integer -> T by the mantissa trick (one add, no conversion unit).
+// Exact small integer -> float by the mantissa trick (one add, no conversion unit).
 __device__ __forceinline__ float small_int_to(float, uint32_t v) {
   return __int_as_float(0x4B000000 | (int)v) - 8388608.0f;  // v < 2^23
 }
-__device__ __forceinline__ double small_int_to(double, uint32_t v) {
-  return __hiloint2double(0x43300000, (int)v) - 4503599627370496.0;  // v < 2^32
-}
 
-// v 2^-t as a double (RN) by integer operations: GB300 issues some 60 integer instructions in
-// the time of one FP64 add or conversion (t: binary places, |t| small).
+// v 2^-t as a double (RN) by integer operations: an FP64 add or conversion takes the issue time of
+// 32 integer adds (qk_wht96.cuh) (t: binary places, |t| small).
 __device__ __forceinline__ double u64_to_double(uint64_t v, int t) {
   const int c = __clzll((long long)v);
   const uint64_t x = v << (c & 63);                      // leading one at bit 63
@@ -47,44 +44,8 @@ __device__ __forceinline__ double u32_to_double(uint32_t v, int t) {  // exact
   return __hiloint2double(v ? (int)hi : 0, (int)(x << 21));
 }
 
-// S' = sum_{a >= 0, bit (31-a) of Z set} 8^-a, to the precision of T.
-__device__ __forceinline__ float octal_tail(float, uint32_t Z) {
-  return __uint2float_rn(spread3_10(Z >> 22)) * 0x1p-27f;  // a = 0..9
-}
-__device__ __forceinline__ double octal_tail(double, uint32_t Z) {
-  const uint32_t hi = spread3_10(Z >> 22);                     // a = 0..9
-  const uint32_t t11 = (Z >> 11) & 0x7FFu;                     // a = 10..20
-  const uint32_t lo = spread3_10(t11) | ((t11 >> 10) << 30);
-  return small_int_to(0.0, hi) * 0x1p-27 + small_int_to(0.0, lo) * 0x1p-60;
-}
-
-template <typename T, int ALPHA>
-__device__ __forceinline__ T dsi_factor(uint32_t Z) {
-  const bool nz = Z != 0u;
-  const int beta = nz ? (__clz(Z) + 1) : 0;
-  const T t1 = nz ? exp2neg(T(), beta) : T(0);
-  if constexpr (ALPHA == 1) {
-    return nz ? (T(1) - T(3) * t1) : T(1);
-  } else {
-    const T x = word_to_unit(T(), Z);
-    const T b = small_int_to(T(), (uint32_t)beta);
-    if constexpr (ALPHA == 2) {
-      return T(1.5) - b * x - T(2.5) * t1;
-    } else if constexpr (ALPHA == 3) {
-      const T t2 = t1 * t1;
-      return T(-1) + b * x * x - T(5) * (T(1) - t1) * x + T(43.0 / 18.0) * (T(1) - t2);
-    } else {
-      static_assert(ALPHA == 4, "DSI order 1..4");
-      const T t2 = t1 * t1;
-      const T t3 = t2 * t1;
-      const T x2 = x * x;
-      const T sp = octal_tail(T(), Z);
-      return T(-1) - T(2.0 / 3.0) * b * x2 * x + T(5) * (T(1) - t1) * x2 -
-             T(43.0 / 9.0) * (T(1) - t2) * x + T(701.0 / 294.0) * (T(1) - t3) -
-             b * sp * T(1.0 / 24.0);
-    }
-  }
-}
+// S' = sum_{a >= 0, bit (31-a) of Z set} 8^-a to FP32's precision: a = 0..9.
+__device__ __forceinline__ float octal_tail(uint32_t Z) { return __uint2float_rn(spread3_10(Z >> 22)) * 0x1p-27f; }
 
 template <typename T, int ALPHA>
 __device__ __forceinline__ T si_factor(uint32_t W) {
@@ -94,7 +55,7 @@ __device__ __forceinline__ T si_factor(uint32_t W) {
   if constexpr (sizeof(T) == 8) {
     q = u64_to_double((uint64_t)W * (uint32_t)(0u - W), 64);
   } else {
-    const T x = word_to_unit(T(), W);
+    const T x = word_to_unit(W);
     q = x * (T(1) - x);
   }
   if constexpr (ALPHA == 1) {
@@ -103,14 +64,6 @@ __device__ __forceinline__ T si_factor(uint32_t W) {
     static_assert(ALPHA == 2, "SI smoothness 1..2");
     return T(2.1646464674222763831) - T(64.939394022668291491) * (q * q);  // pi^4/45, 2pi^4/3
   }
-}
-
-// Family dispatch: FAM 0 = DSI (argument is the XOR difference word), 1 = SI
-// (argument is the mod-2^32 difference word).
-template <typename T, int FAM, int ALPHA>
-__device__ __forceinline__ T factor(uint32_t w) {
-  if constexpr (FAM == 0) return dsi_factor<T, ALPHA>(w);
-  else return si_factor<T, ALPHA>(w);
 }
 
 // Fused multiply-add in the precision of the arguments (never promoted).

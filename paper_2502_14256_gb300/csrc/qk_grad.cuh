@@ -5,8 +5,8 @@
 //   su[v][j] = sum_i u_v[i] dk1_i/dc_j,   s1[j] = sum_i dk1_i/dc_j,
 //   dk1_i/dc_j = k1_i q_ij,  q_ij = K_ij / (1 + c_j K_ij).
 //
-// Bound: FP64 issue (GB300: about 2 FP64 lanes per SM and cycle; some 60 other instructions
-// issue in the time of one FP64 instruction).  So the sweep spends FP64 instructions on the
+// Bound: FP64 issue (GB300: about 2 FP64 lanes per SM and cycle; 32 integer or 57 FP32
+// instructions issue in the time of one FP64 instruction).  So the sweep spends FP64 instructions on the
 // factors and the sums only: a thread owns one dimension j and walks over points, so its sums
 // stay in registers and no FP64 shuffles are needed; q_ij is formed once for up to 16
 // vectors (5 FP64 instructions at DSI order 2, then one fma per vector and one for s1: 14 at

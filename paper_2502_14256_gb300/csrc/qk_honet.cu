@@ -99,38 +99,36 @@ __global__ void __launch_bounds__(kHoNT) k_points_ho(uint32_t d, int order, cons
 }
 
 // ------------------------------------------------------------------ kernels
-// K_alpha(x) of the Theorem at x = Z 2^-64 (64-digit words): beta = clz64(Z) + 1,
-// t_nu = 2^(-nu beta) (products, so that FP32 underflows to 0 gracefully), and for order 4
-// S' = sum over set digits a of 8^-a read from the top 21 (FP64) or 10 (FP32) digits (the
-// rest lie below the precision of T: 8^-21 = 2^-63).
-template <typename T, int ALPHA>
-__device__ __forceinline__ T dsi_factor64(uint64_t Z) {
+// FP32 K_alpha(x) of the Theorem at x = Z 2^-64 (64-digit words; FP64: coefficient rows, qk_grad.cuh):
+// beta = clz64(Z) + 1, t_nu = 2^(-nu beta) (products, so that they underflow to 0 gracefully), and
+// for order 4 S' = sum over set digits a of 8^-a read from the top 10 digits (the rest lie below
+// FP32's precision).
+template <int ALPHA>
+__device__ __forceinline__ float dsi_factor64(uint64_t Z) {
   if (Z == 0ull) {
-    if constexpr (ALPHA == 1) return T(1);
-    else if constexpr (ALPHA == 2) return T(1.5);
-    else if constexpr (ALPHA == 3) return T(-1.0 + 43.0 / 18.0);
-    else return T(-1.0 + 701.0 / 294.0);
+    if constexpr (ALPHA == 1) return 1.f;
+    else if constexpr (ALPHA == 2) return 1.5f;
+    else if constexpr (ALPHA == 3) return float(-1.0 + 43.0 / 18.0);
+    else return float(-1.0 + 701.0 / 294.0);
   }
   const int beta = __clzll((long long)Z) + 1;
-  const T t1 = exp2neg(T(), beta);
+  const float t1 = exp2neg(0.f, beta);
   if constexpr (ALPHA == 1) {
-    return T(1) - T(3) * t1;
+    return 1.f - 3.f * t1;
   } else {
-    T x;
-    if constexpr (sizeof(T) == 8) x = __ull2double_rn(Z) * 0x1p-64;
-    else x = __ull2float_rn(Z) * 0x1p-64f;
-    const T b = (T)beta;
+    const float x = __ull2float_rn(Z) * 0x1p-64f;
+    const float b = (float)beta;
     if constexpr (ALPHA == 2) {
-      return T(1.5) - b * x - T(2.5) * t1;
+      return 1.5f - b * x - 2.5f * t1;
     } else if constexpr (ALPHA == 3) {
-      const T t2 = t1 * t1;
-      return T(-1) + b * x * x - T(5) * (T(1) - t1) * x + T(43.0 / 18.0) * (T(1) - t2);
+      const float t2 = t1 * t1;
+      return -1.f + b * x * x - 5.f * (1.f - t1) * x + float(43.0 / 18.0) * (1.f - t2);
     } else {
       static_assert(ALPHA == 4, "DSI order 1..4");
-      const T t2 = t1 * t1, t3 = t2 * t1, x2 = x * x;
-      const T sp = octal_tail(T(), (uint32_t)(Z >> 32));
-      return T(-1) - T(2.0 / 3.0) * b * x2 * x + T(5) * (T(1) - t1) * x2 - T(43.0 / 9.0) * (T(1) - t2) * x +
-             T(701.0 / 294.0) * (T(1) - t3) - b * sp * T(1.0 / 24.0);
+      const float t2 = t1 * t1, t3 = t2 * t1, x2 = x * x;
+      const float sp = octal_tail((uint32_t)(Z >> 32));
+      return -1.f - float(2.0 / 3.0) * b * x2 * x + 5.f * (1.f - t1) * x2 - float(43.0 / 9.0) * (1.f - t2) * x +
+             float(701.0 / 294.0) * (1.f - t3) - b * sp * float(1.0 / 24.0);
     }
   }
 }
@@ -183,7 +181,7 @@ __global__ void __launch_bounds__(kHoNT) k_kernel_col_ho(uint32_t d, int order, 
     for (int l = 0; l < kHoColL; ++l) {
       const uint64_t Z = b ^ zl[j * kHoColL + l];
       if constexpr (sizeof(T) == 8) p[l] = pm1_step(p[l], wj * dsi_tab_eval64<ALPHA>(tab, Z));
-      else p[l] = pm1_step(p[l], wj * dsi_factor64<T, ALPHA>(Z));
+      else p[l] = pm1_step(p[l], wj * dsi_factor64<ALPHA>(Z));
     }
   }
 #pragma unroll
@@ -273,7 +271,7 @@ __global__ void __launch_bounds__(kHoNT) k_grad_partials_ho(uint32_t d, int orde
     const float wj = (float)wd[j];
     const uint64_t b = zlane[j * 32 + lane] ^ zwarp[warp * d + j];
 #pragma unroll
-    for (int l = 0; l < kHoColL; ++l) p[l] = pm1_step(p[l], wj * dsi_factor64<float, ALPHA>(b ^ zl[j * kHoColL + l]));
+    for (int l = 0; l < kHoColL; ++l) p[l] = pm1_step(p[l], wj * dsi_factor64<ALPHA>(b ^ zl[j * kHoColL + l]));
   }
 #pragma unroll
   for (int l = 0; l < kHoColL; ++l) k1[l] = ok[l] ? (float)zeta * (1.f + p[l]) : 0.f;
@@ -285,7 +283,7 @@ __global__ void __launch_bounds__(kHoNT) k_grad_partials_ho(uint32_t d, int orde
     for (int l = 0; l < kHoColL; ++l) {
       if (!ok[l]) continue;
       const uint64_t bl = b ^ zl[j * kHoColL + l];
-      const float K = dsi_factor64<float, ALPHA>(bl);
+      const float K = dsi_factor64<ALPHA>(bl);
       const float f = fmadd(wj, K, 1.f);
       float dk;
       if (f != 0.f) {
@@ -295,7 +293,7 @@ __global__ void __launch_bounds__(kHoNT) k_grad_partials_ho(uint32_t d, int orde
         for (uint32_t jj = 0; jj < d; ++jj) {
           if (jj == j) continue;
           const uint64_t bj = zlane[jj * 32 + lane] ^ zwarp[warp * d + jj] ^ zl[jj * kHoColL + l];
-          dk *= 1.f + (float)wd[jj] * dsi_factor64<float, ALPHA>(bj);
+          dk *= 1.f + (float)wd[jj] * dsi_factor64<ALPHA>(bj);
         }
       }
       su += (double)uu[l] * (double)dk;

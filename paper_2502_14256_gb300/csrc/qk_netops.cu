@@ -99,9 +99,7 @@ __device__ __forceinline__ double mll_g(double Y, double lam, double inv_n, doub
 
 // What is stored for a result v where `prev` is the value there (NET_ADD) or y's (NET_RESIDUAL).
 __device__ __forceinline__ float op_value(float v, float prev, int op) {
-  if (op == NET_SET) return v;
-  if (op == NET_ADD) return prev + v;
-  return d2f_int(f2d_int(prev) - f2d_int(v));
+  return op == NET_SET ? v : prev + v;  // residuals are formed by FP64 transforms
 }
 __device__ __forceinline__ float op_value(double v, float prev, int op) {
   if (op == NET_RESIDUAL) return d2f_int(f2d_int(prev) - v);
@@ -616,14 +614,15 @@ int net_mll(uint32_t m, uint32_t nvec, uint32_t nrhs, const double *lam, const T
   MidArgs a{};
   a.nrhs = nrhs, a.lam = lam, a.part = part, a.back = sizeof(T) == 8;
   if ((rc = launch_mid<T, TIO, MID_MLL>(X, nullptr, m, nvec, a, st)) || !u) return rc;
-  if (sizeof(T) == 8) {
+  if constexpr (sizeof(T) == 8) {
     smem_optin<k_net_low_out<T, TIO>>(xtile_bytes<T>());
     k_net_low_out<T, TIO><<<tiles_of<T>(m) * nvec, kFNT, xtile_bytes<T>(), st>>>(X, nullptr, u, NET_SET);
     return check_launch("net MLL: low bits");
+  } else {
+    // FP32: the adjoint transform upwards from bit 0, as the multi-pass transform rounds it
+    if ((rc = launch_low_in<T, T>(X, X, m, nvec, nullptr, st))) return rc;
+    return launch_mid<T, TIO, MID_STORE>(X, u, m, nvec, MidArgs{}, st);
   }
-  // FP32: the adjoint transform upwards from bit 0, as the multi-pass transform rounds it
-  if ((rc = launch_low_in<T, T>(X, X, m, nvec, nullptr, st))) return rc;
-  return launch_mid<T, TIO, MID_STORE>(X, u, m, nvec, MidArgs{}, st);
 }
 
 template int net_eigs<float>(uint32_t, uint32_t, const float *, float *, double, double, double, const double *, double *, uint32_t *, cudaStream_t);

@@ -4,7 +4,8 @@
 //
 // Digital nets: the point at sequence position i is
 //   X_i = D (+) XOR_{bit k of h(i)} Ct[k],  h(i) = i (natural) or i ^ (i >> 1) (Gray),
-// and h is linear over GF(2).  A CTA covers 2048 consecutive positions
+// and h is linear over GF(2).  A CTA covers 2048 consecutive positions (columns of few tiles: 512
+// or 1024)
 // i = tile | (l << 8) | (warp << 5) | lane with disjoint bit fields, so
 //   X_i (+) X_0 = Z(h(lane)) (+) Z(h(warp << 5)) (+) Z(h(tile | l << 8)),
 // three small per-CTA tables in shared memory: each difference word costs one
