@@ -45,9 +45,9 @@ UNIT = "points/s"
 # CUDA sources that capture ran (kernel_source_hash()).  A run whose sources differ reports
 # traffic null: the counters belong to another version of the kernels.
 NCU_TRAFFIC = {
-    "src_hash": "5f05dcf73891",
-    "bytes_r64": {"k_fused_A": 1281683968, "k_fused_B": 1294536192, "k_fused_C": 1053151488},
-    "fwht_bytes": 589520896,
+    "src_hash": "67957ca7b5cb",
+    "bytes_r64": {"k_fused_A": 1282101504, "k_fused_B": 1294095104, "k_fused_C": 1053605632},
+    "fwht_bytes": 587863040,
 }
 # Nominal FP64 rate of GB300 (profiling recipe's table; FP64 is not a tensor-core path here).
 FP64_PEAK_TFLOPS = 1.25

@@ -206,8 +206,10 @@ QK_API int qk_eigs_extend(int32_t family, uint32_t m, uint32_t batch, int32_t dt
 
 /* Solve K c = y for `batch` Gram matrices and nrhs right-hand sides each:
  * c = V (y~ / lambda), y~ = conj(V) y (Sec. 5.4).  y, c: (batch, nrhs, n) in
- * dtype (may alias); lam: (batch, n) from qk_eigs.  The division is done in
- * FP64.  refine_steps >= 0 steps of iterative refinement c += K^-1 (y - K c),
+ * dtype (may alias); lam: (batch, n) from qk_eigs.  The scaling is y~ times the
+ * correctly rounded FP64 1 / lambda, rounded to dtype; FP32 nets form it from float pairs
+ * and take FP64 where the two could round differently, so the result is the same bit for
+ * bit.  refine_steps >= 0 steps of iterative refinement c += K^-1 (y - K c),
  * the residual evaluated with FP64 transforms (meaningful for QK_F32). */
 QK_API int qk_solve(int32_t family, uint32_t m, uint32_t batch, uint32_t nrhs, int32_t dtype,
              const double *lam, const void *y, void *c, int32_t refine_steps, void *ws,
@@ -239,7 +241,9 @@ QK_API int qk_mll(const qk_pointset *ps, const qk_kernel *k, uint32_t r0, uint32
  *              (bit-reversed) order, result in frequency order
  *   qk_ifftbr: the inverse of qk_fftbr (frequency order in, natural order out)
  * FFT data are interleaved complex (re, im) pairs of dtype.  Radix-2
- * butterflies (a +- W b)/sqrt(2) as in the paper's FFTBR/FWHT schemes. */
+ * butterflies (a +- W b)/sqrt(2) as in the paper's FFTBR/FWHT schemes.  FP64 qk_fwht above
+ * n = 2^12 sums each pass's tile exactly in integers and rounds once per pass (FP64
+ * butterflies where a tile's values do not fit 96 bits). */
 QK_API int qk_fwht(uint32_t m, uint64_t nvec, int32_t dtype, void *x, qk_stream stream);
 QK_API int qk_fftbr(uint32_t m, uint64_t nvec, int32_t dtype, void *x, qk_stream stream);
 QK_API int qk_ifftbr(uint32_t m, uint64_t nvec, int32_t dtype, void *x, qk_stream stream);
@@ -308,9 +312,10 @@ QK_API int qk_fwht_wait_selftest(uint32_t m, uint64_t nvec, int32_t dtype, void 
                                  uint32_t spin_limit, uint32_t *status, qk_stream stream);
 
 /* Test of the FP64 quotient of the gradient sweeps (no counterpart in the paper): q[i] =
- * a[i] / b[i] as those sweeps form it (two Newton steps on the FP32 reciprocal estimate,
- * then a product; the divide for b outside 2^-100 .. 2^100 in magnitude); a, b, q: n device
- * doubles.  Within 2 ulp of the correctly rounded quotient. */
+ * a[i] / b[i] as those sweeps form it (the FP32 reciprocal estimate and its residual as one
+ * double, a product and one correction; without the residual's double where b is within
+ * 2^-20 of a power of two; the divide for b outside 2^-100 .. 2^100 in magnitude); a, b, q:
+ * n device doubles.  Within 2 ulp of the correctly rounded quotient. */
 QK_API int qk_ratio_selftest(const double *a, const double *b, double *q, uint64_t n, qk_stream stream);
 
 /* --------------------------------------------------- higher-order nets --- */
@@ -381,7 +386,9 @@ enum qk_integrand_id { QK_F_SIMPLE1 = 0, QK_F_SIMPLE2 = 1, QK_F_OAKLEY = 2, QK_F
 /* y[r][i] = f(x_i) at the points of randomizations r0 .. r0+nr-1, positions i0 .. i0+n-1
  * (the points of qk_gen_points, not materialised), with baker != 0 at the baker-transformed
  * point 1 - 2|x - 1/2| instead (Sec. 4.2: periodises the integrand for lattices, mean
- * unchanged).  y: (nr, n) in dtype (QK_F64 or QK_F32; the arithmetic runs in dtype).
+ * unchanged).  y: (nr, n) in dtype (QK_F64 or QK_F32).  FP32 arithmetic for QK_F32; for
+ * QK_F64 sums over the dimensions are exact in fixed-point coefficients (units of 2^-53, for
+ * the corner peak 2^-57), products keep 63 bits, and the functions of them run in FP64.
  * The integrand's dimension must match ps->d where it is fixed (QK_EINVAL otherwise). */
 QK_API int qk_integrand(const qk_pointset *ps, uint32_t r0, uint32_t nr, uint64_t i0, uint64_t n, int32_t f,
                         int32_t baker, int32_t dtype, void *y, qk_stream stream);
